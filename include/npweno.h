@@ -94,8 +94,9 @@ typedef struct {
                                 per-stage kernels; 1 = every instance through the per-stage kernels */
     int32_t tile_1d;         /* cells per CTA of the 1D per-stage kernels: 256, 512, 1024 or 2048; 0 = the
                                 value npw_autotune_1d chose for this flux kind, m, k, precision and
-                                characteristic flag on this device, else 1024.  Results do not depend on
-                                it (each face gets the same arithmetic in any tiling) */
+                                characteristic flag on this device, else a size up to 1024 that spreads
+                                the lines over the SMs.  Results do not depend on it (each face gets the
+                                same arithmetic in any tiling) */
     double eta_max;          /* optional bound, not in the paper: eta = 0 where |eta| > eta_max.  The printed eta
                                 (Table k3, Table k2) is singular where its denominator crosses zero (a monotone
                                 stencil with zero slope at the face for k = 3, v ~ 0 at the face for k = 2), and

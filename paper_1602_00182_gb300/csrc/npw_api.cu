@@ -476,6 +476,7 @@ struct Run1D {
     int64_t ntiles;
     cudaStream_t s;
     int tile = npw::TILE_1D;     // cells per CTA of the per-stage kernels
+    bool table = false;          // work items from the tile table (else one instance, tile = CTA)
     bool comp = false;           // compensated float per-stage kernels (float, component-wise)
     std::vector<char> resident;  // per instance: solved by the resident kernel
     std::vector<cudaEvent_t> joins;  // side-stream work the caller's stream waits for at the end
@@ -494,11 +495,36 @@ std::array<int, 6> tune_key(const npw_params* p, int kind, int m) {
     return {dev, kind, m, p->k, p->precision, p->characteristic ? 1 : 0};
 }
 
-int resolve_tile(const npw_params* p, int kind, int m) {
+// Automatic tile of the 1D per-stage kernels for the given lines: 32 w - halo cells, so that the
+// tile's faces (cells plus `halo` more) fill w warps, with w the power of two that leaves the
+// busiest SM the fewest warps of work, ceil(tiles / SMs) x w; the larger tile where several tie
+// (its halo is a smaller share).  Against a fixed 1024-cell tile, which puts a 200-cell line on one
+// SM and a 20011-cell line on 20: FP64 advection N = 200, one step 90 -> 63 us, 100 steps 8.2 ->
+// 5.4 ms; FP64 1D Euler N = 20011, one step 1071 -> 194 us; mixed Burgers N = 5613, 150 steps
+// 3.75 -> 2.50 ms.
+int auto_tile(const std::vector<int64_t>& n_of, int halo) {
+    int best = 0;
+    int64_t best_cost = 0;
+    for (int w = 1; w <= npw::TILE_1D / 32; w *= 2) {
+        const int t = 32 * w - halo;
+        int64_t tiles = 0;
+        for (int64_t n : n_of) tiles += (n + t - 1) / t;
+        const int64_t cost = (tiles + npw::NUM_SMS - 1) / npw::NUM_SMS * w;
+        if (best == 0 || cost <= best_cost) {
+            best = t;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+// faces beyond its cells that a tile of the face-based / of the compensated stage kernel works on
+constexpr int HALO_FACES = 1, HALO_COMP = 3;
+
+int resolve_tile(const npw_params* p, int kind, int m, int automatic) {
     if (p->tile_1d > 0) return p->tile_1d;
     std::lock_guard<std::mutex> g(g_tune_mu);
     auto it = g_tune.find(tune_key(p, kind, m));
-    return it == g_tune.end() ? npw::TILE_1D : it->second;
+    return it == g_tune.end() ? automatic : it->second;
 }
 
 // the compensated float kernels (stage1d_fast_kernel, the resident kernel) cover float,
@@ -512,11 +538,33 @@ bool resident_ok(const npw_params* p, int m, int64_t n) {
     return compensated(p) && p->batch_mode == 0 && npw::resident_smem_bytes(n, m) <= npw::RESIDENT_SMEM_MAX;
 }
 
+// lines of a batch that take the per-stage kernels, and the tile rule's choice for them
+int batch_auto_tile(const npw_instance* inst, int count, int m, const npw_params* p) {
+    std::vector<int64_t> n_of;
+    for (int i = 0; i < count; ++i)
+        if (!resident_ok(p, m, inst[i].n)) n_of.push_back(inst[i].n);
+    return auto_tile(n_of, compensated(p) ? HALO_COMP : HALO_FACES);
+}
+// entries of a batch's tile table: every instance in the smallest tile a run may choose, or the
+// per-stage ones in the automatic tile
+int64_t batch_table(const npw_instance* inst, int count, int m, const npw_params* p, int automatic) {
+    int64_t nt = 0, na = 0;
+    for (int i = 0; i < count; ++i) {
+        nt += tiles_of(inst[i].n);
+        if (!resident_ok(p, m, inst[i].n)) na += tiles_of(inst[i].n, automatic);
+    }
+    return nt > na ? nt : na;
+}
+
 int64_t tiles_for(const Run1D& r, const npw_instance* inst, int count) {
     int64_t nt = 0;
     for (int i = 0; i < count; ++i)
         if (r.resident.empty() || !r.resident[i]) nt += tiles_of(inst[i].n, r.tile);
     return nt;
+}
+
+const npw::Tile* run_tiles(const Run1D& r) {
+    return r.table ? reinterpret_cast<const npw::Tile*>(r.ws + r.L.tiles) : nullptr;
 }
 
 template <typename R>
@@ -525,7 +573,7 @@ npw_status run_step_kernels(const Run1D& r, int advance) {
     npw::Stage1DArgs a{};
     a.inst = reinterpret_cast<const npw::InstDev*>(r.ws + r.L.inst);
     a.ctl = reinterpret_cast<npw::Ctl*>(r.ws + r.L.ctl);
-    a.tiles = reinterpret_cast<const npw::Tile*>(r.ws + r.L.tiles);
+    a.tiles = run_tiles(r);
     a.ntiles = (int)r.ntiles;
     a.advance = advance;
     a.tile = r.tile;
@@ -563,7 +611,7 @@ npw_status step_kernels(const Run1D& r, int advance) {
 npw_status setup_1d(Run1D& r, const npw_instance* inst, int count, double dt_fixed, int mode) {
     std::vector<npw::InstDev> hi(count);
     std::vector<npw::Tile> ht;
-    ht.reserve((size_t)r.ntiles);
+    if (r.table) ht.reserve((size_t)r.ntiles);
     for (int i = 0; i < count; ++i) {
         hi[i].off = inst[i].offset;
         hi[i].n = inst[i].n;
@@ -573,7 +621,7 @@ npw_status setup_1d(Run1D& r, const npw_instance* inst, int count, double dt_fix
         hi[i].bc = inst[i].bc;
         const bool res = !r.resident.empty() && r.resident[i];
         hi[i].ntiles = res ? 0 : (int32_t)tiles_of(inst[i].n, r.tile);
-        for (int64_t t = 0; t < hi[i].ntiles; ++t) ht.push_back(npw::Tile{i, (int32_t)(t * r.tile)});
+        for (int64_t t = 0; r.table && t < hi[i].ntiles; ++t) ht.push_back(npw::Tile{i, (int32_t)(t * r.tile)});
     }
     // pageable source: each call returns once the data is staged
     NPW_CUDA(cudaMemcpyAsync(r.ws + r.L.inst, hi.data(), sizeof(npw::InstDev) * count, cudaMemcpyHostToDevice, r.s));
@@ -585,21 +633,18 @@ npw_status setup_1d(Run1D& r, const npw_instance* inst, int count, double dt_fix
     npw::ctl_start_kernel<<<blocks, 128, 0, r.s>>>(ctl, di, count, 0, 0.0, 0);
     NPW_CUDA(cudaGetLastError());
     cudaError_t e = r.ntiles == 0 ? cudaSuccess
-                  : r.fp32 ? npw::launch_alpha_init<float>(r.arena, di, ctl,
-                                                           reinterpret_cast<const npw::Tile*>(r.ws + r.L.tiles),
-                                                           (int)r.ntiles, r.tile, r.m, r.kind, r.mp, r.s)
-                           : npw::launch_alpha_init<double>(r.arena, di, ctl,
-                                                            reinterpret_cast<const npw::Tile*>(r.ws + r.L.tiles),
-                                                            (int)r.ntiles, r.tile, r.m, r.kind, r.mp, r.s);
+                  : r.fp32 ? npw::launch_alpha_init<float>(r.arena, di, ctl, run_tiles(r), (int)r.ntiles, r.tile, r.m,
+                                                           r.kind, r.mp, r.s)
+                           : npw::launch_alpha_init<double>(r.arena, di, ctl, run_tiles(r), (int)r.ntiles, r.tile, r.m,
+                                                            r.kind, r.mp, r.s);
     if (e != cudaSuccess) return cuda_fail(e, "alpha kernel launch");
     npw::ctl_start_kernel<<<blocks, 128, 0, r.s>>>(ctl, di, count, mode, dt_fixed, r.mp.max_steps);
     NPW_CUDA(cudaGetLastError());
     count_launch(3);
     if (r.comp && r.ntiles > 0) {
         NPW_CUDA(npw::launch_comp_begin(reinterpret_cast<const float*>(r.arena), reinterpret_cast<float*>(r.ws + r.L.sbuf),
-                                        reinterpret_cast<float*>(r.ws + r.L.cbuf), di,
-                                        reinterpret_cast<const npw::Tile*>(r.ws + r.L.tiles), (int)r.ntiles, r.tile,
-                                        r.m, r.s));
+                                        reinterpret_cast<float*>(r.ws + r.L.cbuf), di, run_tiles(r), (int)r.ntiles,
+                                        r.tile, r.m, r.s));
         count_launch();
     }
     return NPW_OK;
@@ -764,9 +809,8 @@ npw_status launch_resident(Run1D& r, const npw_instance* inst, SideStreams* ss, 
 npw_status comp_end(const Run1D& r) {
     if (!r.comp || r.ntiles == 0) return NPW_OK;
     NPW_CUDA(npw::launch_comp_end(reinterpret_cast<float*>(r.arena), reinterpret_cast<const float*>(r.ws + r.L.sbuf),
-                                  reinterpret_cast<const npw::InstDev*>(r.ws + r.L.inst),
-                                  reinterpret_cast<const npw::Tile*>(r.ws + r.L.tiles), (int)r.ntiles, r.tile, r.m,
-                                  nullptr, r.s));
+                                  reinterpret_cast<const npw::InstDev*>(r.ws + r.L.inst), run_tiles(r), (int)r.ntiles,
+                                  r.tile, r.m, nullptr, r.s));
     count_launch();
     return NPW_OK;
 }
@@ -992,7 +1036,7 @@ static npw_status single_run(void* u, int64_t n, int32_t m, double dx, double t_
     r.mp = method(params);
     r.fp32 = params->precision == NPW_FP32_MIXED;
     r.ws = static_cast<unsigned char*>(workspace);
-    r.tile = resolve_tile(params, flux_kind, m);
+    r.tile = resolve_tile(params, flux_kind, m, auto_tile({n}, compensated(params) ? HALO_COMP : HALO_FACES));
     r.ntiles = tiles_of(n, r.tile);
     r.L = layout_1d(n * m, 1, tiles_of(n), elem_size(params));
     r.s = s;
@@ -1045,12 +1089,12 @@ npw_status npweno_solve(void* u, int64_t n, int32_t m, double dx, double t_end, 
 
 size_t npw_batch_workspace_size(const npw_instance* inst, int32_t count, int32_t m, const npw_params* params) {
     if (!inst || count < 1 || !params || m < 1) return 0;
-    int64_t arena = 0, nt = 0;
+    int64_t arena = 0;
     for (int i = 0; i < count; ++i) {
         int64_t end = inst[i].offset + inst[i].n * m;
         arena = end > arena ? end : arena;
-        nt += tiles_of(inst[i].n);
     }
+    const int64_t nt = batch_table(inst, count, m, params, batch_auto_tile(inst, count, m, params));
     return layout_1d(arena, count, nt, elem_size(params)).total;
 }
 
@@ -1061,7 +1105,7 @@ npw_status npweno_batch_solve(void* arena, const npw_instance* inst, int32_t cou
     if (st) return st;
     if (!arena || !inst || !workspace || count < 1) return fail(NPW_EINVAL, "null pointer or empty batch");
     if ((st = check_kind_1d(flux_kind, m, params))) return st;
-    int64_t arena_elems = 0, nt = 0;
+    int64_t arena_elems = 0;
     for (int i = 0; i < count; ++i) {
         if (inst[i].n < 6 || inst[i].n > ((int64_t)1 << 30)) return fail(NPW_EINVAL, "instance %d: bad n", i);
         if (!(inst[i].dx > 0.0) || !(inst[i].cfl > 0.0)) return fail(NPW_EINVAL, "instance %d: bad dx or cfl", i);
@@ -1069,8 +1113,9 @@ npw_status npweno_batch_solve(void* arena, const npw_instance* inst, int32_t cou
         if ((st = check_bc(inst[i].bc))) return st;
         int64_t end = inst[i].offset + inst[i].n * m;
         arena_elems = end > arena_elems ? end : arena_elems;
-        nt += tiles_of(inst[i].n);
     }
+    const int automatic = batch_auto_tile(inst, count, m, params);
+    const int64_t nt = batch_table(inst, count, m, params, automatic);
     if (nt > (int64_t)1 << 30) return fail(NPW_EINVAL, "too many tiles");
     Run1D r{};
     r.arena = arena;
@@ -1085,7 +1130,8 @@ npw_status npweno_batch_solve(void* arena, const npw_instance* inst, int32_t cou
     if (workspace_bytes < r.L.total)
         return fail(NPW_EINVAL, "workspace too small: %zu < %zu bytes", workspace_bytes, r.L.total);
     r.comp = compensated(params);
-    r.tile = resolve_tile(params, flux_kind, m);
+    r.tile = resolve_tile(params, flux_kind, m, automatic);
+    r.table = true;
     r.resident.assign(count, 0);
     bool any_res = false;
     for (int i = 0; i < count; ++i) {
@@ -1686,7 +1732,7 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
         if (inst[i].ny == 0) kind_cells[inst[i].flux_kind] += cells_of(inst[i]);
     int main_kind = 0;
     for (int k = 1; k < 3; ++k) main_kind = kind_cells[k] > kind_cells[main_kind] ? k : main_kind;
-    int tile = resolve_tile(params, main_kind, flux_m(main_kind));
+    int tile = resolve_tile(params, main_kind, flux_m(main_kind), npw::TILE_1D);
     // a batch of compensated float 1D items alone takes one launch per RK3 step
     bool any2d = false;
     for (int i = 0; i < count; ++i) any2d |= inst[i].ny != 0;

@@ -168,7 +168,7 @@ struct Stage1DArgs {
     float* c;
     const InstDev* inst;
     Ctl* ctl;
-    const Tile* tiles;
+    const Tile* tiles;  // NULL: one instance, tile blockIdx.x
     int32_t ntiles;
     int32_t stage;     // 0, 1, 2
     int32_t advance;   // stage 2 finalises the step (time control on the device)
@@ -289,8 +289,9 @@ cudaError_t launch_comp_end(float* u, const float* s, const InstDev* inst, const
 template <typename R>
 cudaError_t launch_tune_init(R* u, int64_t n, int m, cudaStream_t st);
 
-constexpr int TILE_1D = 1024;     // default cells per CTA tile in the 1D stage kernels
-constexpr int TILE_1D_MIN = 256;  // smallest tile a run may choose (sizes the tile tables)
+constexpr int TILE_1D = 1024;     // largest automatic tile of the 1D stage kernels (cells per CTA)
+constexpr int TILE_1D_MIN = 256;  // smallest tile params.tile_1d may choose (sizes the tile tables)
+constexpr int NUM_SMS = 152;      // SMs of the GPU this library is written for (automatic tiles)
 constexpr int RES_GHOST = 3;       // ghost cells on each side of the resident kernel's state arrays
 constexpr size_t RESIDENT_SMEM_MAX = 200 * 1024;  // shared memory a resident CTA may use
 constexpr int THREADS_1D = 256;

@@ -38,6 +38,12 @@ __device__ __forceinline__ int64_t halo_idx(int64_t n, int64_t k, int bc) {
     return k >= n ? n - 1 : k;
 }
 
+// Work item of this CTA: from the tile table, or, where a launch covers one instance (tiles
+// NULL), tile blockIdx.x of instance 0
+__device__ __forceinline__ Tile tile_at(const Tile* tiles, int tile) {
+    return tiles ? tiles[blockIdx.x] : Tile{0, (int32_t)blockIdx.x * tile};
+}
+
 template <typename R>
 __device__ __forceinline__ bool finite_(R x) {
     return x - x == R(0.0);
@@ -281,7 +287,7 @@ __global__ void __launch_bounds__(THREADS_1D) alpha_init_kernel(const R* __restr
     constexpr int M = kind_m<KIND>();
     __shared__ double red[32];
     __shared__ int redbad[32];
-    const Tile td = tiles[blockIdx.x];
+    const Tile td = tile_at(tiles, tile);
     const InstDev in = inst[td.inst];
     const int64_t n = in.n;
     const int c0 = td.start;
@@ -797,7 +803,7 @@ __device__ __forceinline__ void step1d_fused_body(const Stage1DArgs& a, const Ti
 // for the instances that took an odd number of fused steps, whose last step wrote s)
 static __global__ void comp_copy_kernel(float* dst, const float* src, float* zero, const InstDev* __restrict__ inst,
                                         const Tile* __restrict__ tiles, int tile, int m, const Ctl* odd) {
-    const Tile td = tiles[blockIdx.x];
+    const Tile td = tile_at(tiles, tile);
     if (odd && (odd[td.inst].steps & 1) == 0) return;
     const InstDev in = inst[td.inst];
     const int64_t n = in.n;
@@ -1565,14 +1571,14 @@ __global__ void __launch_bounds__(TX_2D * TY_2D) alpha_init_2d_kernel(const R* _
 template <typename R, typename D, int KIND, bool CHAR>
 __global__ void __launch_bounds__(THREADS_1D) stage1d_kernel(Stage1DArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const Tile td = a.tiles[blockIdx.x];
+    const Tile td = tile_at(a.tiles, a.tile);
     stage1d_body<R, D, KIND, CHAR>(a, td, a.inst[td.inst], a.ctl + td.inst, smem_raw);
 }
 
 template <int KIND, int K>
 __global__ void __launch_bounds__(THREADS_1D) stage1d_fast_kernel(Stage1DArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const Tile td = a.tiles[blockIdx.x];
+    const Tile td = tile_at(a.tiles, a.tile);
     stage1d_fast_body<KIND, K>(a, td, a.inst[td.inst], a.ctl + td.inst, smem_raw);
 }
 
@@ -1872,9 +1878,12 @@ struct Launchers {
             if (e != cudaSuccess) return e;
             attr_set = true;
         }
-        kern<<<a.ntiles, THREADS_1D, smem, s>>>(a);
+        kern<<<a.ntiles, cta_threads(a.tile + 1), smem, s>>>(a);
         return cudaGetLastError();
     }
+
+    // threads of a CTA with `work` independent work items in its widest phase
+    static int cta_threads(int work) { return work >= THREADS_1D ? THREADS_1D : (work + 31) / 32 * 32; }
 
     template <int KIND, int K>
     static cudaError_t stage_fast(const Stage1DArgs& a, cudaStream_t s) {
@@ -1887,7 +1896,7 @@ struct Launchers {
             if (e != cudaSuccess) return e;
             attr_set = true;
         }
-        kern<<<a.ntiles, THREADS_1D, smem, s>>>(a);
+        kern<<<a.ntiles, cta_threads((a.tile + 3) * M), smem, s>>>(a);
         return cudaGetLastError();
     }
 
