@@ -5,6 +5,7 @@
 #include <time.h>
 
 #include <chrono>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -119,6 +120,21 @@ npw::MethodParams method(const npw_params* p) {
     mp.adv_speed_f = (float)mp.adv_speed;
     mp.adv_speed_y_f = (float)mp.adv_speed_y;
     for (int k = 0; k < 4; ++k) mp.inflow_f[k] = (float)mp.inflow[k];
+    // common path of the mixed k = 3 arithmetic (see fast::face_eta and fast::cell_recon)
+    const bool ga = mp.rbf == NPW_RBF_GA;
+    const float ga_rows[6] = {float(2.0 / 3.0), float(-1.0 / 3.0), float(-1.0 / 3.0), 0.0f, 3.0f, -3.0f};
+    const float mq_rows[6] = {float(5.0 / 6.0), float(-2.0 / 3.0), float(-1.0 / 6.0), -1.5f, 6.0f, -4.5f};
+    for (int k = 0; k < 6; ++k) mp.pert_f[k] = ga ? ga_rows[k] : mq_rows[k];
+    const float margin = 1.0f + 0x1p-16f;
+    mp.guard_switch = !mp.monotone_switch || mp.switch_variant == 0;
+    mp.sw24_f = mp.monotone_switch ? 24.0f * margin : 0.0f;
+    mp.sw12_f = mp.monotone_switch ? 12.0f * margin : 0.0f;
+    mp.sws_f = mp.monotone_switch ? 0x1p-14f : 0.0f;
+    mp.guard_hi_f = mp.eta_guard_f * margin;
+    mp.eta_lo_f = mp.eta_eval == 0 && mp.guard_switch ? fmaxf(0x1p-98f, 4.0f * fabsf(mp.eps_M_f)) : INFINITY;
+    mp.eta_lim_f = mp.eta_max_f > 0.0f ? mp.eta_max_f : INFINITY;
+    mp.weno_eps4_f = 4.0f * mp.eps_weno_f;
+    mp.weno_max_f = mp.eps_weno_f >= 1e-18f ? 1e18f : -1.0f;
     return mp;
 }
 

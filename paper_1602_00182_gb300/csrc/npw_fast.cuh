@@ -27,15 +27,17 @@ namespace fast {
 
 // float copies of the method parameters (rounded on the host)
 struct FParams {
-    float eps_weno, eps_M_f, eps_M_lo, eta_guard, eta_max;
+    float eps_weno, eps_M_f, eta_guard, eta_max;
     double eps_M, eta_guard_d;
     int scheme, rbf, monotone_switch, switch_variant, eta_eval;
+    int guard_switch;
+    float pert[6];
+    float sw24, sw12, sws, guard_hi, eta_lo, eta_lim, weno_eps4, weno_max;
 };
 __device__ __forceinline__ FParams fparams(const MethodParams& mp) {
     FParams f;
     f.eps_weno = mp.eps_weno_f;
     f.eps_M_f = mp.eps_M_f;
-    f.eps_M_lo = mp.eps_M_lo_f;
     f.eta_guard = mp.eta_guard_f;
     f.eta_max = mp.eta_max_f;
     f.eps_M = mp.eps_M;
@@ -45,7 +47,65 @@ __device__ __forceinline__ FParams fparams(const MethodParams& mp) {
     f.monotone_switch = mp.monotone_switch;
     f.switch_variant = mp.switch_variant;
     f.eta_eval = mp.eta_eval;
+    f.guard_switch = mp.guard_switch;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) f.pert[k] = mp.pert_f[k];
+    f.sw24 = mp.sw24_f;
+    f.sw12 = mp.sw12_f;
+    f.sws = mp.sws_f;
+    f.guard_hi = mp.guard_hi_f;
+    f.eta_lo = mp.eta_lo_f;
+    f.eta_lim = mp.eta_lim_f;
+    f.weno_eps4 = mp.weno_eps4_f;
+    f.weno_max = mp.weno_max_f;
     return f;
+}
+
+// One float, or two of them in a register pair (the f32x2 instructions of sm_100 and later: one
+// issue slot for two operations, each rounded like the scalar one).  The common-path arithmetic
+// below is written once for both.
+struct F2 {
+    float2 v;
+};
+__device__ __forceinline__ unsigned long long f2_bits(F2 a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.v.x), "f"(a.v.y));
+    return r;
+}
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ F2 vadd(F2 a, F2 b) { return {__fadd2_rn(a.v, b.v)}; }
+__device__ __forceinline__ F2 vmul(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
+__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ F2 vsub(F2 a, F2 b) {
+    F2 r;
+    asm("{.reg .b64 t; sub.rn.f32x2 t, %2, %3; mov.b64 {%0, %1}, t;}"
+        : "=f"(r.v.x), "=f"(r.v.y)
+        : "l"(f2_bits(a)), "l"(f2_bits(b)));
+    return r;
+}
+template <typename V>
+__device__ __forceinline__ V vset(float x) {
+    if constexpr (sizeof(V) == sizeof(float))
+        return x;
+    else
+        return V{make_float2(x, x)};
+}
+template <typename V>
+constexpr int kLanes = sizeof(V) / sizeof(float);
+__device__ __forceinline__ float& lane_of(float& a, int) { return a; }
+__device__ __forceinline__ float lane_of(const float& a, int) { return a; }
+__device__ __forceinline__ float& lane_of(F2& a, int i) { return i ? a.v.y : a.v.x; }
+__device__ __forceinline__ float lane_of(const F2& a, int i) { return i ? a.v.y : a.v.x; }
+
+// reciprocal to about one ulp for a normal argument (subnormal results flushed): one instruction,
+// where a quotient only needs to be an estimate
+__device__ __forceinline__ float rcp_fast(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
 constexpr float kU = 5.9604645e-08f;  // 2^-24, unit roundoff of float
@@ -460,29 +520,143 @@ __device__ __forceinline__ float eta_eval(float w0, float w1, float w2, float w3
                             : eta_fp64(w0, w1, w2, w3, fp, guard, fl);
 }
 
-// eta of the face whose eta stencil is (w0..w3), 0 where the switch fires; flag bits: FL_SWITCH,
-// FL_ZERO_GUARD, FL_ZERO_BOUND
-__device__ __forceinline__ float face_eta(float w0, float w1, float w2, float w3, const FParams& fp,
-                                          uint32_t* flag) {
-    if (fp.scheme != NPW_RBF_ENO_ && fp.scheme != NPW_RBF_WENO_) return 0.0f;
-    if (fp.monotone_switch && switch_fires_f(w0, w1, w2, w3, fp.switch_variant)) {
-        *flag |= FL_SWITCH;
-        return 0.0f;
+// eta and its flags off the common path: the certified switch, then the shape parameter in the
+// form asked for.  Out of line, with its parameters by value: a warp calls it when a face of its
+// needs it (an extremum, a shock, a denominator near the guard).
+static __device__ __noinline__ uint2 face_eta_rare(float w0, float w1, float w2, float w3, float eta_guard,
+                                                   double eta_guard_d, float eps_M_f, double eps_M, float eta_max,
+                                                   int monotone_switch, int switch_variant, int eta_form) {
+    FParams fp;
+    fp.eta_guard = eta_guard;
+    fp.eta_guard_d = eta_guard_d;
+    fp.eps_M_f = eps_M_f;
+    fp.eps_M = eps_M;
+    fp.eta_eval = eta_form;
+    uint2 r = make_uint2(0u, 0u);
+    if (monotone_switch && switch_fires_f(w0, w1, w2, w3, switch_variant)) {
+        r.y = FL_SWITCH;
+        return r;
     }
-    const float e = eta_eval(w0, w1, w2, w3, fp, flag);
-    if (fp.eta_max > 0.0f && fabsf(e) > fp.eta_max) {
-        *flag |= FL_ZERO_BOUND;
-        return 0.0f;
+    const float e = eta_eval(w0, w1, w2, w3, fp, &r.y);
+    if (eta_max > 0.0f && fabsf(e) > eta_max) {
+        r.y |= FL_ZERO_BOUND;
+        return r;
     }
-    return e;
+    r.x = __float_as_uint(e);
+    return r;
+}
+
+template <typename V>
+__device__ __forceinline__ void two_sum_v(V a, V b, V& s, V& e) {
+    s = vadd(a, b);
+    const V bb = vsub(s, a);
+    e = vadd(vsub(a, vsub(s, bb)), vsub(b, bb));
+}
+template <typename V>
+__device__ __forceinline__ void two_diff_v(V a, V b, V& s, V& e) {  // two_sum(a, -b)
+    s = vsub(a, b);
+    const V bb = vsub(s, a);
+    e = vsub(vsub(a, vsub(s, bb)), vadd(b, bb));
+}
+
+// the certified switch of a stencil whose denominator is below the guard: FL_SWITCH, else FL_ZERO_GUARD
+static __device__ __noinline__ uint32_t guard_or_switch(float w0, float w1, float w2, float w3) {
+    return switch_fires_f(w0, w1, w2, w3, 0) ? FL_SWITCH : FL_ZERO_GUARD;
+}
+
+// eta of the face(s) whose eta stencil is (w0..w3), 0 where the switch fires; flag bits: FL_SWITCH,
+// FL_ZERO_GUARD, FL_ZERO_BOUND.  The common path decides nearly every face of smooth data from
+// four combinations of the float neighbour differences.  In the terms of switch_v0_cert the switch
+// cannot fire where
+//   |C| >= 24 |A| + 12 |B|,
+// and the denominator is C.  The float A, B and C are within 6u (s + 2 |d1|), 6u s and 6u (s + 14
+// |d1|) of the exact values, s = |d0| + |d2|, where 14 |d1| <= |C| + s: at most 166 u s + 21 u |C| on
+// the right-hand side and 12 u s + 6 u |C| on the left, which the margins 2^-16 relative and 2^-14 s
+// cover several times.  The guard's test carries the same margin.  There the arithmetic is that of
+// eta_doublefloat in its range of the fast reciprocal, so the value is the same bits.  The other
+// faces: a constant stencil, and one whose denominator is certainly below the guard, give 0 without
+// a quotient (gas at rest: a third to five sixths of the faces of the Euler cases); the rest (NaN
+// included: every comparison is then false) goes to face_eta_rare.
+template <typename V>
+__device__ __forceinline__ V face_eta(V w0, V w1, V w2, V w3, const FParams& fp, uint32_t* flag) {
+    constexpr int W = kLanes<V>;
+    V eta = vset<V>(0.0f);
+    if (fp.scheme != NPW_RBF_ENO_ && fp.scheme != NPW_RBF_WENO_) return eta;
+    const V d0 = vsub(w1, w0), d1 = vsub(w2, w1), d2 = vsub(w3, w2), t02 = vadd(d0, d2);
+    const V A = vfma(vset<V>(-2.0f), d1, t02), B = vsub(d2, d0), C = vfma(vset<V>(-14.0f), d1, t02);  // C: minus the denominator
+    bool ok[W], any = false;
+    float s[W], thr[W], aC[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        const float mag = fmaf(15.f, fabsf(lane_of(w1, i)) + fabsf(lane_of(w2, i)),
+                               fabsf(lane_of(w0, i)) + fabsf(lane_of(w3, i)));
+        s[i] = fabsf(lane_of(d0, i)) + fabsf(lane_of(d2, i));
+        aC[i] = fabsf(lane_of(C, i));
+        thr[i] = fp.guard_hi * mag;
+        const float rhs = fmaf(fp.sw24, fabsf(lane_of(A, i)), fmaf(fp.sw12, fabsf(lane_of(B, i)), fp.sws * s[i]));
+        ok[i] = aC[i] >= rhs && aC[i] > fmaf(0x1p-19f, s[i], thr[i]) + fp.eta_lo && aC[i] < 0x1p124f;
+        any |= ok[i];
+    }
+    if (any) {
+        V ah, al, bh, bl, nh, nl, dh, dl, t;
+        two_diff_v(w0, w3, ah, al);
+        two_diff_v(w2, w1, bh, bl);
+        const V three = vset<V>(3.0f), fifteen = vset<V>(15.0f);
+        const V p3 = vmul(three, bh), p15 = vmul(fifteen, bh);
+        const V p3m = vfma(vset<V>(-3.0f), bh, p3), p15m = vfma(vset<V>(-15.0f), bh, p15);  // minus the product errors
+        two_sum_v(ah, p3, nh, nl);
+        two_sum_v(ah, p15, dh, dl);
+        nl = vadd(nl, vadd(al, vsub(vmul(three, bl), p3m)));
+        dl = vadd(dl, vadd(al, vsub(vmul(fifteen, bl), p15m)));
+        // eps_M, then the renormalised pairs
+        two_sum_v(dh, vset<V>(fp.eps_M_f), dh, t);
+        dl = vadd(dl, t);
+        two_sum_v(nh, nl, nh, nl);
+        two_sum_v(dh, dl, dh, dl);
+        V rc, nq1;
+#pragma unroll
+        for (int i = 0; i < W; ++i) lane_of(rc, i) = rcp_fast(lane_of(dh, i));
+        const V q1 = vmul(nh, rc), p = vmul(q1, dh);
+#pragma unroll
+        for (int i = 0; i < W; ++i) lane_of(nq1, i) = -lane_of(q1, i);
+        const V pe = vfma(nq1, dh, p);  // minus the error of p
+        const V r = vadd(vadd(vsub(nh, p), pe), vfma(nq1, dl, nl));
+        eta = vadd(q1, vmul(r, rc));
+#pragma unroll
+        for (int i = 0; i < W; ++i)  // beyond the bound (or NaN): decided off the common path
+            ok[i] = ok[i] && fabsf(lane_of(eta, i)) <= fp.eta_lim;
+    }
+#pragma unroll
+    for (int i = 0; i < W; ++i)
+        if (__builtin_expect(!ok[i], 0)) {
+            const float w0i = lane_of(w0, i), w1i = lane_of(w1, i), w2i = lane_of(w2, i), w3i = lane_of(w3, i);
+            float e = 0.0f;
+            if (s[i] == 0.0f && aC[i] == 0.0f && fp.eta_guard > 0.0f) {
+                flag[i] |= FL_ZERO_GUARD;
+            } else if (fmaf(0x1p-19f, s[i], aC[i]) < thr[i] * (1.0f - 0x1p-14f) && thr[i] >= 0x1p-99f && fp.guard_switch) {
+                flag[i] |= fp.monotone_switch ? guard_or_switch(w0i, w1i, w2i, w3i) : FL_ZERO_GUARD;
+            } else {
+                const uint2 x = face_eta_rare(w0i, w1i, w2i, w3i, fp.eta_guard, fp.eta_guard_d, fp.eps_M_f, fp.eps_M,
+                                              fp.eta_max, fp.monotone_switch, fp.switch_variant, fp.eta_eval);
+                e = __uint_as_float(x.x);
+                flag[i] |= x.y;
+            }
+            lane_of(eta, i) = e;
+        }
+    return eta;
 }
 
 // ---------------------------------------------------------------------------------------
 // One cell: c[0..4] = cells i-2..i+2; eta_r = eta of face i+1/2, eta_l of face i-1/2.
 // Writes v^-_{i+1/2} and v^+_{i-1/2}.  Returns the ENO stencil (0 for WENO).
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ int cell_recon(const float* c, float eta_r, float eta_l, const FParams& mp,
-                                          float* vm, float* vp) {
+// WENO values of a cell whose smoothness indicators leave the range of the common path (differences
+// of the cell averages beyond ~5e8, or an eps_weno below 1e-18), out of line.  The weights use the
+// fast float division (within 2 ulp for divisors in [2^-126, 2^126]): beta + eps is clamped at
+// 1e18, so that every divisor below stays inside that range.
+static __device__ __noinline__ float2 weno_rare(float c0, float c1, float c2, float c3, float c4, float eta_r, float eta_l,
+                                               float eps, int rbf) {
+    const float c[5] = {c0, c1, c2, c3, c4};
     float cm[3], cp[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -490,25 +664,14 @@ __device__ __forceinline__ int cell_recon(const float* c, float eta_r, float eta
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             const float x = c[2 - r + j];
-            sm = fmaf(fmaf(pert_coef<float>(mp.rbf, r + 1, j), eta_r, poly_coef<float>(r + 1, j)), x, sm);
-            sp = fmaf(fmaf(pert_coef<float>(mp.rbf, r, j), eta_l, poly_coef<float>(r, j)), x, sp);
+            sm = fmaf(fmaf(pert_coef<float>(rbf, r + 1, j), eta_r, poly_coef<float>(r + 1, j)), x, sm);
+            sp = fmaf(fmaf(pert_coef<float>(rbf, r, j), eta_l, poly_coef<float>(r, j)), x, sp);
         }
         cm[r] = sm;
         cp[r] = sp;
     }
-    if (mp.scheme == NPW_ENO_ || mp.scheme == NPW_RBF_ENO_) {
-        const int r = eno_choice_f(c[0], c[1], c[2], c[3], c[4]);
-        *vm = r == 0 ? cm[0] : (r == 1 ? cm[1] : cm[2]);
-        *vp = r == 0 ? cp[0] : (r == 1 ? cp[1] : cp[2]);
-        return r;
-    }
-    // Jiang-Shu indicators (single precision), shared by both faces of the cell.  The weights
-    // use the fast float division (within 2 ulp for divisors in [2^-126, 2^126]): beta + eps is
-    // at least eps_weno and is clamped at 1e18 (differences of the cell averages near 1e9, far
-    // beyond any workload), so every divisor below stays inside that range.
     constexpr float kBeMax = 1e18f;
     float a, b, inv[3];
-    const float eps = mp.eps_weno;
     a = c[2] - 2.f * c[3] + c[4];
     b = fmaf(3.f, c[2], fmaf(-4.f, c[3], c[4]));
     float be = fminf(fmaf(13.f / 12.f * a, a, 0.25f * b * b) + eps, kBeMax);
@@ -524,8 +687,86 @@ __device__ __forceinline__ int cell_recon(const float* c, float eta_r, float eta
     // v^-: d = (3/10, 3/5, 1/10); v^+: d = (1/10, 3/5, 3/10)
     const float am0 = 0.3f * inv[0], am1 = 0.6f * inv[1], am2 = 0.1f * inv[2];
     const float ap0 = 0.1f * inv[0], ap1 = 0.6f * inv[1], ap2 = 0.3f * inv[2];
-    *vm = __fdividef(fmaf(am0, cm[0], fmaf(am1, cm[1], am2 * cm[2])), am0 + am1 + am2);
-    *vp = __fdividef(fmaf(ap0, cp[0], fmaf(ap1, cp[1], ap2 * cp[2])), ap0 + ap1 + ap2);
+    return make_float2(__fdividef(fmaf(am0, cm[0], fmaf(am1, cm[1], am2 * cm[2])), am0 + am1 + am2),
+                       __fdividef(fmaf(ap0, cp[0], fmaf(ap1, cp[1], ap2 * cp[2])), ap0 + ap1 + ap2));
+}
+
+// The six distinct coefficients c_rj + q_rj eta of a face: rows 1 (k[0..2]) and 3 (k[3..5]); rows 2
+// and 0 are their mirror images.
+template <typename V>
+__device__ __forceinline__ void face_coefs(V eta, const FParams& fp, V* k) {
+    const float poly[6] = {1.0f / 3.0f, 5.0f / 6.0f, -1.0f / 6.0f, 1.0f / 3.0f, -7.0f / 6.0f, 11.0f / 6.0f};
+#pragma unroll
+    for (int j = 0; j < 6; ++j) k[j] = vfma(vset<V>(fp.pert[j]), eta, vset<V>(poly[j]));
+}
+template <typename V>
+__device__ __forceinline__ V dot3(V k0, V x0, V k1, V x1, V k2, V x2) {
+    return vfma(k2, x2, vfma(k1, x1, vmul(k0, x0)));
+}
+
+// Jiang-Shu indicators in single precision, shared by both faces of the cell, formed four times
+// too large (a power of two, which saves the product with 1/4 and cancels exactly in the weights);
+// one reciprocal instruction per weight, whose argument lies in its normal range because 4 (beta +
+// eps) is in [4e-18, 1e18] (else weno_rare).
+template <typename V>
+__device__ __forceinline__ int cell_recon(const V* c, V eta_r, V eta_l, const FParams& fp, V* vm, V* vp) {
+    constexpr int W = kLanes<V>;
+    V kr[6], kl[6], cm[3], cp[3];
+    face_coefs(eta_r, fp, kr);
+    face_coefs(eta_l, fp, kl);
+    cm[0] = dot3(kr[0], c[2], kr[1], c[3], kr[2], c[4]);
+    cm[1] = dot3(kr[2], c[1], kr[1], c[2], kr[0], c[3]);
+    cm[2] = dot3(kr[3], c[0], kr[4], c[1], kr[5], c[2]);
+    cp[0] = dot3(kl[5], c[2], kl[4], c[3], kl[3], c[4]);
+    cp[1] = dot3(kl[0], c[1], kl[1], c[2], kl[2], c[3]);
+    cp[2] = dot3(kl[2], c[0], kl[1], c[1], kl[0], c[2]);
+    if (fp.scheme == NPW_ENO_ || fp.scheme == NPW_RBF_ENO_) {
+        int r = 0;
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            r = eno_choice_f(lane_of(c[0], i), lane_of(c[1], i), lane_of(c[2], i), lane_of(c[3], i), lane_of(c[4], i));
+            lane_of(*vm, i) = r == 0 ? lane_of(cm[0], i) : (r == 1 ? lane_of(cm[1], i) : lane_of(cm[2], i));
+            lane_of(*vp, i) = r == 0 ? lane_of(cp[0], i) : (r == 1 ? lane_of(cp[1], i) : lane_of(cp[2], i));
+        }
+        return r;
+    }
+    const V m2 = vset<V>(-2.0f), m4 = vset<V>(-4.0f), p3 = vset<V>(3.0f);
+    const V a0 = vadd(vfma(m2, c[3], c[2]), c[4]), b0 = vfma(p3, c[2], vfma(m4, c[3], c[4]));
+    const V a1 = vadd(vfma(m2, c[2], c[1]), c[3]), b1 = vsub(c[1], c[3]);
+    const V a2 = vadd(vfma(m2, c[1], c[0]), c[2]), b2 = vfma(m4, c[1], vfma(p3, c[2], c[0]));
+    const V c13 = vset<V>(4.0f * (13.f / 12.f)), eps = vset<V>(fp.weno_eps4);
+    V be[3];
+    be[0] = vadd(vfma(vmul(c13, a0), a0, vmul(b0, b0)), eps);
+    be[1] = vadd(vfma(vmul(c13, a1), a1, vmul(b1, b1)), eps);
+    be[2] = vadd(vfma(vmul(c13, a2), a2, vmul(b2, b2)), eps);
+    V inv[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const V sq = vmul(be[r], be[r]);
+#pragma unroll
+        for (int i = 0; i < W; ++i) lane_of(inv[r], i) = rcp_fast(lane_of(sq, i));
+    }
+    // v^-: d = (3/10, 3/5, 1/10); v^+: d = (1/10, 3/5, 3/10)
+    const V d1 = vset<V>(0.1f), d3 = vset<V>(0.3f);
+    const V w1 = vmul(vset<V>(0.6f), inv[1]);
+    const V am0 = vmul(d3, inv[0]), am2 = vmul(d1, inv[2]), ap0 = vmul(d1, inv[0]), ap2 = vmul(d3, inv[2]);
+    const V sm = vadd(vadd(am0, w1), am2), sp = vadd(vadd(ap0, w1), ap2);
+    V rm, rp;
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        lane_of(rm, i) = rcp_fast(lane_of(sm, i));
+        lane_of(rp, i) = rcp_fast(lane_of(sp, i));
+    }
+    *vm = vmul(vfma(am0, cm[0], vfma(w1, cm[1], vmul(am2, cm[2]))), rm);
+    *vp = vmul(vfma(ap0, cp[0], vfma(w1, cp[1], vmul(ap2, cp[2]))), rp);
+#pragma unroll
+    for (int i = 0; i < W; ++i)
+        if (__builtin_expect(!(fmaxf(fmaxf(lane_of(be[0], i), lane_of(be[1], i)), lane_of(be[2], i)) <= fp.weno_max), 0)) {
+            const float2 v = weno_rare(lane_of(c[0], i), lane_of(c[1], i), lane_of(c[2], i), lane_of(c[3], i),
+                                       lane_of(c[4], i), lane_of(eta_r, i), lane_of(eta_l, i), fp.eps_weno, fp.rbf);
+            lane_of(*vm, i) = v.x;
+            lane_of(*vp, i) = v.y;
+        }
     return 0;
 }
 
@@ -730,7 +971,7 @@ __device__ __forceinline__ uint32_t face_field(const float* w, const MethodParam
     if (mp0.k == 2) return face_field_k2(w, mp0, vm, vp, tl, tr, eta_out);
     uint32_t fl = 0;
     const FParams mp = fparams(mp0);
-    const float eta = face_eta(w[1], w[2], w[3], w[4], mp, &fl);
+    const float eta = face_eta<float>(w[1], w[2], w[3], w[4], mp, &fl);
     float dummy;
     const int rl = cell_recon(w, eta, eta, mp, vm, &dummy);
     const int rr = cell_recon(w + 1, eta, eta, mp, &dummy, vp);

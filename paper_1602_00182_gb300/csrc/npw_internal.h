@@ -37,12 +37,15 @@ __host__ __device__ __forceinline__ uint8_t flag_byte(uint32_t fl) {
 // k = 2): the switch fired, eta evaluated, and of those zeroed by the guard / the bound.
 struct EtaCount {
     uint32_t sw = 0, ev = 0, guard = 0, bound = 0;
-    // one face of k = 3 from its flag word
+    // one face of k = 3 from its flag word (0 on the common path)
     __device__ __forceinline__ void face_k3(uint32_t fl) {
-        sw += fl & FL_SWITCH;
-        ev += (fl & FL_SWITCH) ^ 1u;
-        guard += (fl >> 6) & 1u;
-        bound += (fl >> 7) & 1u;
+        ev += 1u;
+        if (__builtin_expect(fl != 0u, 0)) {
+            sw += fl & FL_SWITCH;
+            ev -= fl & FL_SWITCH;
+            guard += (fl >> 6) & 1u;
+            bound += (fl >> 7) & 1u;
+        }
     }
     // both face values (v^- of the left cell, v^+ of the right cell) of a k = 2 face
     __device__ __forceinline__ void face_k2(uint32_t fl) {
@@ -86,6 +89,15 @@ struct MethodParams {
     float eps_weno_f, eps_M_f, eps_M_lo_f, eta_guard_f, eta_max_f;  // eps_M ~ eps_M_f + eps_M_lo_f
     float gamma_f, adv_speed_f, adv_speed_y_f;
     float inflow_f[4];
+    // mixed precision, k = 3: constants of the common path of the shape parameter and of the
+    // reconstruction (fast::face_eta, fast::cell_recon)
+    float pert_f[6];   // perturbation rows 1 (entries 0..2) and 3 (entries 3..5) of the table; 2 and 0 mirror them
+    int guard_switch;  // 1: switch variant 0, or no switch (a stencil below the guard needs that switch only)
+    float sw24_f, sw12_f, sws_f;       // 24, 12 (with a margin) and the weight of the roundings; 0: switch off
+    float guard_hi_f;                  // guard threshold with a margin
+    float eta_lo_f;                    // smallest denominator of the common path; infinity: the common path is off
+    float eta_lim_f;                   // eta_max, or infinity
+    float weno_eps4_f, weno_max_f;     // 4 eps_weno; largest 4 (beta + eps) of the common path
 };
 
 // a method parameter in the arithmetic type R: the double value, or its float copy
