@@ -1241,6 +1241,12 @@ npw_status npw_autotune_1d(int32_t flux_kind, int32_t m, const npw_params* param
 // ---------------------------------------------------------------------------------------
 // 2D
 // ---------------------------------------------------------------------------------------
+}  // extern "C"
+namespace {
+void plan_2d(npw::Inst2D& d, bool warp_tiles);
+}  // namespace
+extern "C" {
+
 size_t npw_workspace_size_2d(int64_t nx, int64_t ny, int32_t m, const npw_params* params) {
     if (!params || nx < 1 || ny < 1 || m < 1) return 0;
     size_t esz = elem_size(params);
@@ -1294,9 +1300,9 @@ static npw_status run_2d(void* u, int64_t nx, int64_t ny, int32_t m, double dx, 
     hi.cfl = cfl;
     hi.bc = bc;
     hi.bc_y = params->bc_y < 0 ? bc : params->bc_y;
-    hi.tiles_x = (int32_t)((nx + npw::TX_2D - 1) / npw::TX_2D);
-    hi.tiles_y = (int32_t)((ny + npw::TY_2D - 1) / npw::TY_2D);
-    const int tiles = hi.tiles_x * hi.tiles_y;
+    plan_2d(hi, npw::warp_tiles_2d(fp32, params->k));
+    const int items = hi.tiles_x * hi.tiles_y;
+    const int tiles = (int)(((nx + npw::TX_2D - 1) / npw::TX_2D) * ((ny + npw::TY_2D - 1) / npw::TY_2D));  // alpha^0
     NPW_CUDA(cudaMemcpyAsync(dinst, &hi, sizeof hi, cudaMemcpyHostToDevice, s));
     npw::MethodParams mp = method(params);
     npw::ctl_start_2d_kernel<<<1, 32, 0, s>>>(ctl, dinst, 0, 0.0, 0);
@@ -1322,8 +1328,8 @@ static npw_status run_2d(void* u, int64_t nx, int64_t ny, int32_t m, double dx, 
             a.uout = out_[stg];
             a.stage = stg;
             auto ev = stage_begin(s);
-            cudaError_t ee = fp32 ? npw::launch_stage2d<float>(a, tiles, flux_kind, s)
-                                  : npw::launch_stage2d<double>(a, tiles, flux_kind, s);
+            cudaError_t ee = fp32 ? npw::launch_stage2d<float>(a, items, flux_kind, s)
+                                  : npw::launch_stage2d<double>(a, items, flux_kind, s);
             stage_end(ev, s);
             if (ee != cudaSuccess) return cuda_fail(ee, "stage 2d launch");
         }
@@ -1519,6 +1525,13 @@ QLayout queue_layout(int64_t arena_elems, int count, int64_t nitems, size_t esz,
     o = align256(o + sizeof(int32_t) * (size_t)count);
     L.total = o;
     return L;
+}
+
+// tiles of a 2D instance: those of the warp-task body or of the others
+void plan_2d(npw::Inst2D& d, bool warp_tiles) {
+    const int tx = warp_tiles ? npw::TX_WARP : npw::TX_2D, ty = warp_tiles ? npw::TY_WARP : npw::TY_2D;
+    d.tiles_x = (int32_t)((d.nx + tx - 1) / tx);
+    d.tiles_y = (int32_t)((d.ny + ty - 1) / ty);
 }
 
 bool is_2d_kind(const npw_queue_instance& q) { return q.ny != 0; }
@@ -1792,8 +1805,7 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
             d.cfl = q.cfl;
             d.bc = q.bc;
             d.bc_y = q.bc_y < 0 ? q.bc : q.bc_y;
-            d.tiles_x = (int32_t)((q.nx + npw::TX_2D - 1) / npw::TX_2D);
-            d.tiles_y = (int32_t)((q.ny + npw::TY_2D - 1) / npw::TY_2D);
+            plan_2d(d, npw::warp_tiles_2d(r.fp32, params->k));
             has2d = true;
             m2d = flux_m(q.flux_kind) > m2d ? flux_m(q.flux_kind) : m2d;
         }
@@ -1845,8 +1857,8 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
     q.tile = tile;
     q.head = reinterpret_cast<unsigned int*>(ws + r.L.head);
     q.mp = method(params);
-    r.smem = r.fp32 ? npw::queue_smem_bytes<float>(tile, has1d, m1d, has2d, m2d, r.characteristic)
-                    : npw::queue_smem_bytes<double>(tile, has1d, m1d, has2d, m2d, r.characteristic);
+    r.smem = r.fp32 ? npw::queue_smem_bytes<float>(tile, has1d, m1d, has2d, m2d, r.characteristic, params->k)
+                    : npw::queue_smem_bytes<double>(tile, has1d, m1d, has2d, m2d, r.characteristic, params->k);
     if (r.fused) r.smem = npw::fused1d_smem_floats(tile, m1d) * sizeof(float);
     // start: reset, alpha^0 over the items, first dt
     NPW_CUDA(npw::launch_queue_ctl(q.ctl, q.inst1, q.inst2, q.is2d, nullptr, count, 0, 0, r.s));
@@ -1910,7 +1922,9 @@ struct LaneLayout {
 // one lane's part of the arena, starting at byte `begin`
 LaneLayout lane_layout(size_t begin, int64_t heap_cells, int max_slots, size_t esz, bool comp) {
     LaneLayout L{};
-    L.max_items = heap_cells / (npw::TX_2D * npw::TY_2D) + 2 * (int64_t)max_slots;
+    // a 2D request of at least 6 x 6 cells has at most cells / 42 + 1 tiles of 30 x 11, a 1D one cells /
+    // 63 + 1 tiles of 63 cells
+    L.max_items = heap_cells / 32 + 2 * (int64_t)max_slots;
     size_t o = align256(begin);
     L.begin = o;
     L.inst1 = o;
@@ -2135,8 +2149,7 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
             d.cfl = sl.req.cfl;
             d.bc = sl.req.bc;
             d.bc_y = sl.req.bc_y < 0 ? sl.req.bc : sl.req.bc_y;
-            d.tiles_x = (int32_t)((sl.req.n + npw::TX_2D - 1) / npw::TX_2D);
-            d.tiles_y = (int32_t)((sl.req.ny + npw::TY_2D - 1) / npw::TY_2D);
+            plan_2d(d, npw::warp_tiles_2d(lane.fp32, lane.mp.k));
         }
         if (sl.fresh) fresh.push_back(k);
     }
@@ -2222,9 +2235,9 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
         if (g.fused)
             smem = npw::fused1d_smem_floats(g.tile, g.m) * sizeof(float);
         else if (lane.fp32)
-            smem = npw::queue_smem_bytes<float>(g.tile, !g.is2d, g.m, g.is2d, g.m, false);
+            smem = npw::queue_smem_bytes<float>(g.tile, !g.is2d, g.m, g.is2d, g.m, false, q0.mp.k);
         else
-            smem = npw::queue_smem_bytes<double>(g.tile, !g.is2d, g.m, g.is2d, g.m, false);
+            smem = npw::queue_smem_bytes<double>(g.tile, !g.is2d, g.m, g.is2d, g.m, false, q0.mp.k);
         for (int step = 0; step < steps; ++step) {
             if (g.fused) {
                 q.stage = npw::QUEUE_FUSED_STEP;

@@ -259,7 +259,7 @@ __device__ __forceinline__ int sdiff_abs_less(float a, float b, float c, float p
 // the ENO choice where the float test of its first (s1 = kUncertain) or second step is not
 // certain, out of line: the second step from the second differences to a few units of u^2,
 // else the FP64 evaluation
-__device__ __forceinline__ int eno_choice_rest(float c0, float c1, float c2, float c3, float c4, int s1) {
+static __device__ __noinline__ int eno_choice_rest(float c0, float c1, float c2, float c3, float c4, int s1) {
     if (s1 != kUncertain) {
         const int x = s1 > 0 ? sdiff_abs_less(c0, c1, c2, c1, c2, c3) : sdiff_abs_less(c1, c2, c3, c2, c3, c4);
         if (x >= 0) {
@@ -559,91 +559,167 @@ __device__ __forceinline__ void two_diff_v(V a, V b, V& s, V& e) {  // two_sum(a
     e = vsub(vsub(a, vsub(s, bb)), vadd(b, bb));
 }
 
-// the certified switch of a stencil whose denominator is below the guard: FL_SWITCH, else FL_ZERO_GUARD
-static __device__ __noinline__ uint32_t guard_or_switch(float w0, float w1, float w2, float w3) {
-    return switch_fires_f(w0, w1, w2, w3, 0) ? FL_SWITCH : FL_ZERO_GUARD;
+// The switch (variant 0) where the common test does not decide, from A, B and the denominator C (float,
+// with the errors stated at face_eta) and s: 1 fires, 0 does not, -1 not certain.  12 p' at the two
+// ends of the stencil is E +- 12 B with E = 24 A + C: opposite signs fire; with equal signs only a
+// vertex inside (|B| < 4 |A|) whose value has the other sign fires, and 12 p'(vertex) has the sign of
+// A G with G = 2 A C - 3 B^2.  e bounds the error of A, B, and a sixteenth of those of C and E.
+__device__ __forceinline__ int switch_level2(float A, float B, float C, float s) {
+    const float aA = fabsf(A), aB = fabsf(B), aC = fabsf(C);
+    const float e = 0x1p-19f * (s + aC);
+    const float E = fmaf(24.f, A, C), aE = fabsf(E), eE = 32.f * e;
+    const float b12 = 12.f * aB;
+    if (b12 > aE + eE * 2.f) return 1;
+    if (!(aE > b12 + eE * 2.f)) return -1;
+    if (aB > fmaf(4.f, aA, 8.f * e)) return 0;
+    if (!(aB < fmaf(4.f, aA, -8.f * e)) || !(aA > e)) return -1;
+    const float G = fmaf(2.f * A, C, -3.f * B * B);
+    const float eG = 40.f * e * (aA + aB + aC + e);
+    if (!(fabsf(G) > eG)) return -1;
+    return (G > 0.f) == ((A > 0.f) == (E > 0.f)) ? 0 : 1;
 }
 
-// eta of the face(s) whose eta stencil is (w0..w3), 0 where the switch fires; flag bits: FL_SWITCH,
-// FL_ZERO_GUARD, FL_ZERO_BOUND.  The common path decides nearly every face of smooth data from
-// four combinations of the float neighbour differences.  In the terms of switch_v0_cert the switch
-// cannot fire where
-//   |C| >= 24 |A| + 12 |B|,
-// and the denominator is C.  The float A, B and C are within 6u (s + 2 |d1|), 6u s and 6u (s + 14
-// |d1|) of the exact values, s = |d0| + |d2|, where 14 |d1| <= |C| + s: at most 166 u s + 21 u |C| on
-// the right-hand side and 12 u s + 6 u |C| on the left, which the margins 2^-16 relative and 2^-14 s
-// cover several times.  The guard's test carries the same margin.  There the arithmetic is that of
-// eta_doublefloat in its range of the fast reciprocal, so the value is the same bits.  The other
-// faces: a constant stencil, and one whose denominator is certainly below the guard, give 0 without
-// a quotient (gas at rest: a third to five sixths of the faces of the Euler cases); the rest (NaN
-// included: every comparison is then false) goes to face_eta_rare.
-template <typename V>
-__device__ __forceinline__ V face_eta(V w0, V w1, V w2, V w3, const FParams& fp, uint32_t* flag) {
+// eta of N faces (of one or two lanes' worth of fields each) whose eta stencils are w[n][0..3], 0 where
+// the switch fires; flag bits: FL_SWITCH, FL_ZERO_GUARD, FL_ZERO_BOUND.  The common test decides
+// nearly every face of smooth data from four combinations of the float neighbour differences.  In the
+// terms of switch_v0_cert the switch cannot fire where
+//   |C| >= 24 |A| + 12 |B|.
+// The float A, B and C are within 6u (s + 2 |d1|), 6u s and 6u (s + 14 |d1|) of the exact values, s =
+// |d0| + |d2|, where 14 |d1| <= |C| + s: at most 166 u s + 21 u |C| on the right-hand side and 12 u s +
+// 6 u |C| on the left, which the margins 2^-16 relative and 2^-14 s cover several times.  The guard's
+// test carries the same margin.  A face that fails the test takes switch_level2 and, where both
+// switch and guard are then certain, still needs no call: at shocks and in the round-off of gas at
+// rest most faces do, and a call costs a warp the latency of its whole chain.  Where the switch
+// does not fire and the guard is clear the arithmetic is that of eta_doublefloat in its range of the
+// fast reciprocal, so the value is the same bits.  What is left (NaN included: every comparison is
+// then false) goes to face_eta_rare.
+template <typename V, int N>
+__device__ __forceinline__ void face_eta_n(const V (&w)[N][4], const FParams& fp, V (&eta)[N], uint32_t (&flag)[N][kLanes<V>]) {
     constexpr int W = kLanes<V>;
-    V eta = vset<V>(0.0f);
-    if (fp.scheme != NPW_RBF_ENO_ && fp.scheme != NPW_RBF_WENO_) return eta;
-    const V d0 = vsub(w1, w0), d1 = vsub(w2, w1), d2 = vsub(w3, w2), t02 = vadd(d0, d2);
-    const V A = vfma(vset<V>(-2.0f), d1, t02), B = vsub(d2, d0), C = vfma(vset<V>(-14.0f), d1, t02);  // C: minus the denominator
-    bool ok[W], any = false;
-    float s[W], thr[W], aC[W];
 #pragma unroll
-    for (int i = 0; i < W; ++i) {
-        const float mag = fmaf(15.f, fabsf(lane_of(w1, i)) + fabsf(lane_of(w2, i)),
-                               fabsf(lane_of(w0, i)) + fabsf(lane_of(w3, i)));
-        s[i] = fabsf(lane_of(d0, i)) + fabsf(lane_of(d2, i));
-        aC[i] = fabsf(lane_of(C, i));
-        thr[i] = fp.guard_hi * mag;
-        const float rhs = fmaf(fp.sw24, fabsf(lane_of(A, i)), fmaf(fp.sw12, fabsf(lane_of(B, i)), fp.sws * s[i]));
-        ok[i] = aC[i] >= rhs && aC[i] > fmaf(0x1p-19f, s[i], thr[i]) + fp.eta_lo && aC[i] < 0x1p124f;
-        any |= ok[i];
+    for (int n = 0; n < N; ++n) {
+        eta[n] = vset<V>(0.0f);
+#pragma unroll
+        for (int i = 0; i < W; ++i) flag[n][i] = 0u;
     }
-    if (any) {
-        V ah, al, bh, bl, nh, nl, dh, dl, t;
-        two_diff_v(w0, w3, ah, al);
-        two_diff_v(w2, w1, bh, bl);
-        const V three = vset<V>(3.0f), fifteen = vset<V>(15.0f);
-        const V p3 = vmul(three, bh), p15 = vmul(fifteen, bh);
-        const V p3m = vfma(vset<V>(-3.0f), bh, p3), p15m = vfma(vset<V>(-15.0f), bh, p15);  // minus the product errors
-        two_sum_v(ah, p3, nh, nl);
-        two_sum_v(ah, p15, dh, dl);
-        nl = vadd(nl, vadd(al, vsub(vmul(three, bl), p3m)));
-        dl = vadd(dl, vadd(al, vsub(vmul(fifteen, bl), p15m)));
-        // eps_M, then the renormalised pairs
-        two_sum_v(dh, vset<V>(fp.eps_M_f), dh, t);
-        dl = vadd(dl, t);
-        two_sum_v(nh, nl, nh, nl);
-        two_sum_v(dh, dl, dh, dl);
-        V rc, nq1;
+    if (fp.scheme != NPW_RBF_ENO_ && fp.scheme != NPW_RBF_WENO_) return;
+    // per face: 1 common arithmetic, 0 done (eta = 0), -1 rare
+    int todo[N][W];
+    bool all = true, some = false;
+    V A[N], B[N], C[N];
+    float s[N][W], thr[N][W];
 #pragma unroll
-        for (int i = 0; i < W; ++i) lane_of(rc, i) = rcp_fast(lane_of(dh, i));
-        const V q1 = vmul(nh, rc), p = vmul(q1, dh);
+    for (int n = 0; n < N; ++n) {
+        const V d0 = vsub(w[n][1], w[n][0]), d1 = vsub(w[n][2], w[n][1]), d2 = vsub(w[n][3], w[n][2]), t02 = vadd(d0, d2);
+        A[n] = vfma(vset<V>(-2.0f), d1, t02);
+        B[n] = vsub(d2, d0);
+        C[n] = vfma(vset<V>(-14.0f), d1, t02);  // minus the denominator
 #pragma unroll
-        for (int i = 0; i < W; ++i) lane_of(nq1, i) = -lane_of(q1, i);
-        const V pe = vfma(nq1, dh, p);  // minus the error of p
-        const V r = vadd(vadd(vsub(nh, p), pe), vfma(nq1, dl, nl));
-        eta = vadd(q1, vmul(r, rc));
-#pragma unroll
-        for (int i = 0; i < W; ++i)  // beyond the bound (or NaN): decided off the common path
-            ok[i] = ok[i] && fabsf(lane_of(eta, i)) <= fp.eta_lim;
-    }
-#pragma unroll
-    for (int i = 0; i < W; ++i)
-        if (__builtin_expect(!ok[i], 0)) {
-            const float w0i = lane_of(w0, i), w1i = lane_of(w1, i), w2i = lane_of(w2, i), w3i = lane_of(w3, i);
-            float e = 0.0f;
-            if (s[i] == 0.0f && aC[i] == 0.0f && fp.eta_guard > 0.0f) {
-                flag[i] |= FL_ZERO_GUARD;
-            } else if (fmaf(0x1p-19f, s[i], aC[i]) < thr[i] * (1.0f - 0x1p-14f) && thr[i] >= 0x1p-99f && fp.guard_switch) {
-                flag[i] |= fp.monotone_switch ? guard_or_switch(w0i, w1i, w2i, w3i) : FL_ZERO_GUARD;
-            } else {
-                const uint2 x = face_eta_rare(w0i, w1i, w2i, w3i, fp.eta_guard, fp.eta_guard_d, fp.eps_M_f, fp.eps_M,
-                                              fp.eta_max, fp.monotone_switch, fp.switch_variant, fp.eta_eval);
-                e = __uint_as_float(x.x);
-                flag[i] |= x.y;
-            }
-            lane_of(eta, i) = e;
+        for (int i = 0; i < W; ++i) {
+            const float mag = fmaf(15.f, fabsf(lane_of(w[n][1], i)) + fabsf(lane_of(w[n][2], i)),
+                                   fabsf(lane_of(w[n][0], i)) + fabsf(lane_of(w[n][3], i)));
+            const float aC = fabsf(lane_of(C[n], i));
+            s[n][i] = fabsf(lane_of(d0, i)) + fabsf(lane_of(d2, i));
+            thr[n][i] = fp.guard_hi * mag;
+            const float rhs =
+                fmaf(fp.sw24, fabsf(lane_of(A[n], i)), fmaf(fp.sw12, fabsf(lane_of(B[n], i)), fp.sws * s[n][i]));
+            const bool ok = aC >= rhs && aC > fmaf(0x1p-19f, s[n][i], thr[n][i]) + fp.eta_lo && aC < 0x1p124f;
+            todo[n][i] = ok ? 1 : -1;
+            all = all && ok;
+            some = some || ok;
         }
-    return eta;
+    }
+    if (!all) {
+#pragma unroll
+        for (int n = 0; n < N; ++n)
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                const float aC = fabsf(lane_of(C[n], i)), si = s[n][i];
+                if (todo[n][i] < 0) {
+                    if (si == 0.0f && aC == 0.0f && fp.eta_guard > 0.0f) {  // constant
+                        flag[n][i] = FL_ZERO_GUARD;
+                        todo[n][i] = 0;
+                    } else if (fp.guard_switch) {
+                        const int sw = fp.monotone_switch && aC < 0x1p60f && si < 0x1p60f && aC + si > 0x1p-40f
+                                           ? switch_level2(lane_of(A[n], i), lane_of(B[n], i), -lane_of(C[n], i), si)
+                                           : (fp.monotone_switch ? -1 : 0);
+                        if (sw == 1) {
+                            flag[n][i] = FL_SWITCH;
+                            todo[n][i] = 0;
+                        } else if (sw == 0) {
+                            if (fmaf(0x1p-19f, si, aC) < thr[n][i] * (1.0f - 0x1p-14f) && thr[n][i] >= 0x1p-99f) {
+                                flag[n][i] = FL_ZERO_GUARD;
+                                todo[n][i] = 0;
+                            } else if (aC > fmaf(0x1p-19f, si, thr[n][i]) + fp.eta_lo && aC < 0x1p124f) {
+                                todo[n][i] = 1;
+                                some = true;
+                            }
+                        }
+                    }
+                }
+            }
+    }
+    if (some) {
+        const V three = vset<V>(3.0f), fifteen = vset<V>(15.0f);
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            V ah, al, bh, bl, nh, nl, dh, dl, t;
+            two_diff_v(w[n][0], w[n][3], ah, al);
+            two_diff_v(w[n][2], w[n][1], bh, bl);
+            const V p3 = vmul(three, bh), p15 = vmul(fifteen, bh);
+            const V p3m = vfma(vset<V>(-3.0f), bh, p3), p15m = vfma(vset<V>(-15.0f), bh, p15);  // minus the product errors
+            two_sum_v(ah, p3, nh, nl);
+            two_sum_v(ah, p15, dh, dl);
+            nl = vadd(nl, vadd(al, vsub(vmul(three, bl), p3m)));
+            dl = vadd(dl, vadd(al, vsub(vmul(fifteen, bl), p15m)));
+            // eps_M, then the renormalised pairs
+            two_sum_v(dh, vset<V>(fp.eps_M_f), dh, t);
+            dl = vadd(dl, t);
+            two_sum_v(nh, nl, nh, nl);
+            two_sum_v(dh, dl, dh, dl);
+            V rc, nq1;
+#pragma unroll
+            for (int i = 0; i < W; ++i) lane_of(rc, i) = rcp_fast(lane_of(dh, i));
+            const V q1 = vmul(nh, rc), p = vmul(q1, dh);
+#pragma unroll
+            for (int i = 0; i < W; ++i) lane_of(nq1, i) = -lane_of(q1, i);
+            const V pe = vfma(nq1, dh, p);  // minus the error of p
+            const V r = vadd(vadd(vsub(nh, p), pe), vfma(nq1, dl, nl));
+            const V e = vadd(q1, vmul(r, rc));
+#pragma unroll
+            for (int i = 0; i < W; ++i) {
+                if (todo[n][i] == 1) lane_of(eta[n], i) = lane_of(e, i);
+                // beyond the bound (or NaN): off the common path
+                if (todo[n][i] == 1 && !(fabsf(lane_of(e, i)) <= fp.eta_lim)) {
+                    todo[n][i] = -1;
+                    all = false;
+                }
+            }
+        }
+    }
+    if (!all) {
+#pragma unroll
+        for (int n = 0; n < N; ++n)
+#pragma unroll
+            for (int i = 0; i < W; ++i)
+                if (__builtin_expect(todo[n][i] < 0, 0)) {
+                    const uint2 x = face_eta_rare(lane_of(w[n][0], i), lane_of(w[n][1], i), lane_of(w[n][2], i),
+                                                  lane_of(w[n][3], i), fp.eta_guard, fp.eta_guard_d, fp.eps_M_f, fp.eps_M,
+                                                  fp.eta_max, fp.monotone_switch, fp.switch_variant, fp.eta_eval);
+                    lane_of(eta[n], i) = __uint_as_float(x.x);
+                    flag[n][i] = x.y;
+                }
+    }
+}
+
+// one face of one field
+__device__ __forceinline__ float face_eta(float w0, float w1, float w2, float w3, const FParams& fp, uint32_t* flag) {
+    const float w[1][4] = {{w0, w1, w2, w3}};
+    float eta[1];
+    uint32_t fl[1][1];
+    face_eta_n<float, 1>(w, fp, eta, fl);
+    *flag |= fl[0][0];
+    return eta[0];
 }
 
 // ---------------------------------------------------------------------------------------
@@ -971,7 +1047,7 @@ __device__ __forceinline__ uint32_t face_field(const float* w, const MethodParam
     if (mp0.k == 2) return face_field_k2(w, mp0, vm, vp, tl, tr, eta_out);
     uint32_t fl = 0;
     const FParams mp = fparams(mp0);
-    const float eta = face_eta<float>(w[1], w[2], w[3], w[4], mp, &fl);
+    const float eta = face_eta(w[1], w[2], w[3], w[4], mp, &fl);
     float dummy;
     const int rl = cell_recon(w, eta, eta, mp, vm, &dummy);
     const int rr = cell_recon(w + 1, eta, eta, mp, &dummy, vp);

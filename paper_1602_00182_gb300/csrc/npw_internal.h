@@ -165,6 +165,7 @@ struct Inst2D {
     int32_t bc;      // boundary of the x direction (columns)
     int32_t tiles_x, tiles_y;
     int32_t bc_y;    // boundary of the y direction (rows)
+    // tiles_x, tiles_y: TX_2D x TY_2D tiles, or TX_WARP x TY_WARP in the mixed k = 3 runs (warp_tiles_2d)
 };
 
 struct Stage1DArgs {
@@ -278,7 +279,7 @@ cudaError_t launch_queue_stage(const QueueArgs& q, bool characteristic, int shap
 template <typename R>
 cudaError_t launch_queue_alpha(const QueueArgs& q, cudaStream_t s);
 template <typename R>
-size_t queue_smem_bytes(int tile, bool has1d, int m1d, bool has2d, int m2d, bool characteristic);
+size_t queue_smem_bytes(int tile, bool has1d, int m1d, bool has2d, int m2d, bool characteristic, int k);
 // resident whole-solve launch (float state only); max_n = largest n in the list
 cudaError_t launch_resident_f32(const ResidentArgs& a, int m, int kind, int64_t max_n, int threads, cudaStream_t s);
 size_t resident_smem_bytes(int64_t n, int m);
@@ -309,5 +310,9 @@ constexpr size_t RESIDENT_SMEM_MAX = 200 * 1024;  // shared memory a resident CT
 constexpr int THREADS_1D = 256;
 constexpr int TX_2D = 32;      // 2D tile
 constexpr int TY_2D = 8;
+constexpr int TX_WARP = 30;    // tile of the warp-task body (stage2d_warp_body)
+constexpr int TY_WARP = 11;
+// the 2D runs of the warp-task body: mixed precision, k = 3
+__host__ __device__ constexpr bool warp_tiles_2d(bool fp32, int k) { return fp32 && k == 3; }
 
 }  // namespace npw

@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "npw_device.cuh"
 #include "npw_fast.cuh"
@@ -1084,9 +1085,8 @@ __device__ __forceinline__ float halo_get(const float* u, const Inst2D& in, int 
 }
 
 // ---------------------------------------------------------------------------------------
-// 2D stage kernel of the mixed path (float state, component-wise) in phases, each a balanced
+// 2D stage kernel of the mixed path, k = 2 (float state, component-wise) in phases, each a balanced
 // loop over independent work items:
-//   E  (k = 3) eta of every (face, field) of both directions (FP64 quotient, switch)
 //   C  reconstruction of every (cell, field) of both directions: v^- at its right / upper face
 //      and v^+ at its left / lower face, one set of smoothness indicators for both (k = 2: the
 //      cell's own switch and shape parameters, with the transverse term of the 5-cell cross)
@@ -1299,6 +1299,218 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
         const double bx = block_max_nan_f(vmx, bad, red, redbad);
         const double by = block_max_nan_f(vmy, bad, red2, redbad2);
         if (tid == 0) {
+            atomicMax(&ctl->alpha_next_bits, (unsigned long long)__double_as_longlong(bx));
+            atomicMax(&ctl->alpha_y_next_bits, (unsigned long long)__double_as_longlong(by));
+            __threadfence();
+            const unsigned prev = atomicAdd(&ctl->tiles_done, 1u);
+            if (prev == (unsigned)(in.tiles_x * in.tiles_y) - 1u) {
+                __threadfence();
+                finalize_2d(ctl, in);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// 2D stage of the mixed path, k = 3 (float state, component-wise), in warp tasks.  The phases are
+// those of stage2d_fast_body (eta of every face; reconstruction of every cell, both directions; flux;
+// update), but a task is one row of the tile and one pair of fields, a lane one face, cell or column
+// of it: TX_WARP + 2 = 32 cells of a row fill the lanes, and with TY_WARP = 11 the 46, 48, 23 and 11
+// tasks of the phases (2D Euler) leave the eight warps nearly even.  A task's addresses are then a
+// lane offset from a row, where the flat loop over (face, field) spent as much on indices as on the
+// method, and the two fields of a pair share every f32x2 instruction.  Each face value has the
+// arithmetic of the flat body, so the results are the same bits.  Bound by instruction issue (64% of
+// the slots) and the barriers between the phases; FMA pipe 44%.  One stage of 2048^2 2D Euler cells: 645
+// -> 320 M warp instructions, 643 -> 407 us.  (A form that kept a row window in registers and marched
+// without shared memory issued 256 M, but its 17 KB loop body missed the instruction cache: 657 us.)
+// Shared memory (V: a pair of fields, or the one field): the (TX_WARP + 6) x (TY_WARP + 6) block and
+// three face arrays of 32 lanes x (TY_WARP x-face rows, TY_WARP + 1 y-face rows).
+// ---------------------------------------------------------------------------------------
+template <int M>
+struct FieldV {  // fields two at a time
+    using V = fast::F2;
+    static constexpr int P = M / 2;
+};
+template <>
+struct FieldV<1> {
+    using V = float;
+    static constexpr int P = 1;
+};
+template <int M>
+__host__ __device__ constexpr int stage2d_warp_smem_floats() {
+    return M * ((TX_WARP + 6) * (TY_WARP + 6) + 3 * 32 * (2 * TY_WARP + 1));
+}
+
+template <int KIND>
+__device__ __forceinline__ void stage2d_warp_body(const Stage2DArgs& a, const Inst2D& in, Ctl* ctl, int tile, float* smem) {
+    constexpr int M = kind_m<KIND>();
+    using V = typename FieldV<M>::V;
+    constexpr int P = FieldV<M>::P, W = fast::kLanes<V>;
+    constexpr int BX = TX_WARP + 6, BY = TY_WARP + 6, NR = 2 * TY_WARP + 1;  // face rows: x rows, then y rows
+    V* su = reinterpret_cast<V*>(smem);  // [P][BY][BX]
+    V* ef = su + P * BY * BX;            // [P][NR][32] eta per face; then the fluxes
+    V* vmf = ef + P * NR * 32;           // v^- per face
+    V* vpf = vmf + P * NR * 32;          // v^+ per face
+    __shared__ float red[32], red2[32];
+    __shared__ int redbad[32], redbad2[32];
+    __shared__ float s_par[5];  // alpha_x, alpha_y, dt, 1 / dx, 1 / dy in float
+    if (*(volatile int32_t*)&ctl->done) return;  // uniform over the CTA
+    const int nx = (int)in.nx, ny = (int)in.ny;
+    const int tx0 = (tile % in.tiles_x) * TX_WARP, ty0 = (tile / in.tiles_x) * TY_WARP;
+    const int cols = min(TX_WARP, nx - tx0), rows = min(TY_WARP, ny - ty0);
+    const int64_t cells = in.nx * in.ny;
+    const float* uin = reinterpret_cast<const float*>(a.uin) + in.off;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int NW = THREADS_1D / 32;
+    const fast::FParams fp = fast::fparams(a.mp);
+    // the block, a row per warp: lanes take columns lane and lane + 32 (the boundary maps once per
+    // lane and once per row; -1: the inflow state, whatever the other index)
+    {
+        auto map = [](int i, int n, int bc) {
+            if (bc == NPW_BC_PERIODIC) return i < 0 ? i + n : (i >= n ? i - n : i);
+            return i < 0 ? (bc == NPW_BC_INFLOW ? -1 : 0) : (i >= n ? n - 1 : i);
+        };
+        const int x0 = map(tx0 - 3 + min(lane, cols + 5), nx, in.bc), x1 = map(tx0 - 3 + min(lane + 32, cols + 5), nx, in.bc);
+        const bool in0 = lane < cols + 6, in1 = lane + 32 < cols + 6;
+#pragma unroll 1
+        for (int by = warp; by < rows + 6; by += NW) {
+            const int y = map(ty0 - 3 + by, ny, in.bc_y);
+            const float* row = uin + (int64_t)max(y, 0) * nx;
+            V* to = su + by * BX + lane;
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+                const float* at = row + k * cells;
+                float v0 = at[max(x0, 0)], v1 = 0.0f;
+                if (in1) v1 = at[max(x1, 0)];
+                if ((x0 | y) < 0) v0 = a.mp.inflow_f[k];
+                if ((x1 | y) < 0) v1 = a.mp.inflow_f[k];
+                if (in0) fast::lane_of(to[k / W * BY * BX], k % W) = v0;
+                if (in1) fast::lane_of(to[k / W * BY * BX + 32], k % W) = v1;
+            }
+        }
+    }
+    if (threadIdx.x == 0) {
+        s_par[0] = (float)(*(volatile double*)&ctl->alpha);
+        s_par[1] = (float)(*(volatile double*)&ctl->alpha_y);
+        s_par[2] = (float)(*(volatile double*)&ctl->dt);
+        s_par[3] = 1.0f / (float)in.dx;
+        s_par[4] = 1.0f / (float)in.dy;
+    }
+    __syncthreads();
+    EtaCount ec;
+    const bool last_x = tx0 + cols == nx, last_y = ty0 + rows == ny;
+    // E: task t = (face row, pair); x rows first (lane = face qx between cells qx - 1 and qx), then y rows
+    // (lane = column), the warps taking them in turn
+    auto e_task = [&](int p, int q, auto dir) {
+        constexpr bool X = decltype(dir)::value;
+        constexpr int step = X ? 1 : BX;
+        if (lane >= (X ? cols + 1 : cols)) return;
+        const V* at = su + p * BY * BX + (X ? (q + 3) * BX + lane + 1 : (q + 1) * BX + lane + 3);
+        const V w[1][4] = {{at[0], at[step], at[2 * step], at[3 * step]}};
+        V eta[1];
+        uint32_t fl[1][W];
+        fast::face_eta_n<V, 1>(w, fp, eta, fl);
+        ef[(p * NR + (X ? q : TY_WARP + q)) * 32 + lane] = eta[0];
+        if (X ? (lane < cols || last_x) : (q < rows || last_y))
+#pragma unroll
+            for (int i = 0; i < W; ++i) ec.face_k3(fl[0][i]);
+    };
+    int t = warp;
+#pragma unroll 1
+    for (; t < P * rows; t += NW) e_task(t % P, t / P, std::true_type{});
+#pragma unroll 1
+    for (t -= P * rows; t < P * (rows + 1); t += NW) e_task(t % P, t / P, std::false_type{});
+    flush_counts(ec, ctl, a.mp);
+    __syncthreads();
+    // C: task = (cell row, pair); x: lane = cell lane - 1, rows 0..TY-1; y: lane = column, q = cell row + 1
+    auto c_task = [&](int p, int q, auto dir) {
+        constexpr bool X = decltype(dir)::value;
+        constexpr int step = X ? 1 : BX;
+        if (lane >= (X ? cols + 2 : cols)) return;
+        const V* at = su + p * BY * BX + (X ? (q + 3) * BX + lane : q * BX + lane + 3);
+        // faces on the right (above) and on the left (below) of the cell
+        const int fr = (p * NR + (X ? q : TY_WARP + q)) * 32 + lane, fl = fr - (X ? 1 : 32);
+        const bool has_r = X ? lane <= cols : q <= rows, has_l = X ? lane >= 1 : q >= 1;
+        V c[5], vm, vp;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) c[j] = at[j * step];
+        V er = fast::vset<V>(0.0f), el = er;
+        if (has_r) er = ef[fr];
+        if (has_l) el = ef[fl];
+        fast::cell_recon<V>(c, er, el, fp, &vm, &vp);
+        if (has_r) vmf[fr] = vm;
+        if (has_l) vpf[fl] = vp;
+    };
+    t = warp;
+#pragma unroll 1
+    for (; t < P * rows; t += NW) c_task(t % P, t / P, std::true_type{});
+#pragma unroll 1
+    for (t -= P * rows; t < P * (rows + 2); t += NW) c_task(t % P, t / P, std::false_type{});
+    __syncthreads();
+    // F: task = face row, all fields; the fluxes overwrite the eta array
+    const float ax = s_par[0], ay = s_par[1];
+#pragma unroll 1
+    for (t = warp; t < 2 * rows + 1; t += NW) {
+        const bool is_x = t < rows;
+        const int f = (is_x ? t : TY_WARP + t - rows) * 32 + lane;
+        if (lane < (is_x ? cols + 1 : cols)) {
+            float vm[M], vp[M], h[M];
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+                vm[k] = fast::lane_of(vmf[k / W * NR * 32 + f], k % W);
+                vp[k] = fast::lane_of(vpf[k / W * NR * 32 + f], k % W);
+            }
+            if (is_x)
+                lf_flux<float, KIND, M>(vm, vp, ax, a.mp, 0, h);
+            else
+                lf_flux<float, KIND, M>(vm, vp, ay, a.mp, 1, h);
+#pragma unroll
+            for (int k = 0; k < M; ++k) fast::lane_of(ef[k / W * NR * 32 + f], k % W) = h[k];
+        }
+    }
+    __syncthreads();
+    // U: task = row, lane = column
+    float* uout = reinterpret_cast<float*>(a.uout) + in.off;
+    const float* un = reinterpret_cast<const float*>(a.un) + in.off;
+    const float dtR = s_par[2], idxR = s_par[3], idyR = s_par[4];
+    float vmx = 0.0f, vmy = 0.0f;
+    bool bad = false;
+#pragma unroll 1
+    for (int q = warp; q < rows; q += NW) {
+        if (lane >= cols) continue;
+        float U[M];
+        const int64_t at = (int64_t)(ty0 + q) * nx + tx0 + lane;
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const V* hx = ef + (k / W * NR + q) * 32 + lane;
+            const V* hy = hx + TY_WARP * 32;
+            float L = -((fast::lane_of(hx[1], k % W) - fast::lane_of(hx[0], k % W)) * idxR);
+            L = L - (fast::lane_of(hy[32], k % W) - fast::lane_of(hy[0], k % W)) * idyR;
+            const float uk = fast::lane_of(su[(k / W * BY + q + 3) * BX + lane + 3], k % W);
+            const int64_t gidx = k * cells + at;
+            float o;
+            if (a.stage == 0)
+                o = uk + dtR * L;
+            else if (a.stage == 1)
+                o = 0.75f * un[gidx] + 0.25f * (uk + dtR * L);
+            else
+                o = stage3_w1<float>() * un[gidx] + stage3_w2<float>() * (uk + dtR * L);
+            uout[gidx] = o;
+            U[k] = o;
+            bad |= !finite_(o);
+        }
+        if (a.stage == 2) {
+            const float sx = wave_speed<float, KIND>(U, a.mp, 0);
+            const float sy = wave_speed<float, KIND>(U, a.mp, 1);
+            bad |= !finite_(sx) || !finite_(sy);
+            vmx = sx > vmx ? sx : vmx;
+            vmy = sy > vmy ? sy : vmy;
+        }
+    }
+    if (a.stage == 2 && a.advance) {
+        const double bx = block_max_nan_f(vmx, bad, red, redbad);
+        const double by = block_max_nan_f(vmy, bad, red2, redbad2);
+        if (threadIdx.x == 0) {
             atomicMax(&ctl->alpha_next_bits, (unsigned long long)__double_as_longlong(bx));
             atomicMax(&ctl->alpha_y_next_bits, (unsigned long long)__double_as_longlong(by));
             __threadfence();
@@ -1538,8 +1750,9 @@ __global__ void __launch_bounds__(TX_2D * TY_2D) alpha_init_2d_kernel(const R* _
     __shared__ double red2[32];
     __shared__ int redbad2[32];
     const Inst2D in = *inst;
-    const int tx0 = (blockIdx.x % in.tiles_x) * TX_2D;
-    const int ty0 = (blockIdx.x / in.tiles_x) * TY_2D;
+    const int tiles_x = (int)((in.nx + TX_2D - 1) / TX_2D);
+    const int tx0 = (blockIdx.x % tiles_x) * TX_2D;
+    const int ty0 = (blockIdx.x / tiles_x) * TY_2D;
     const int64_t cells = in.nx * in.ny;
     const int qy = threadIdx.x / TX_2D, qx = threadIdx.x - qy * TX_2D;
     const int64_t gi = tx0 + qx, gj = ty0 + qy;
@@ -1588,6 +1801,12 @@ __global__ void __launch_bounds__(TX_2D * TY_2D) stage2d_fast_kernel(Stage2DArgs
     stage2d_fast_body<KIND, K>(a, *a.inst, a.ctl, blockIdx.x, smem_f);
 }
 
+template <int KIND>
+__global__ void __launch_bounds__(THREADS_1D, 4) stage2d_warp_kernel(Stage2DArgs a) {
+    extern __shared__ __align__(16) float smem_f[];
+    stage2d_warp_body<KIND>(a, *a.inst, a.ctl, blockIdx.x, smem_f);
+}
+
 template <typename R, typename D, int KIND>
 __global__ void __launch_bounds__(TX_2D * TY_2D) stage2d_kernel(Stage2DArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1617,17 +1836,21 @@ __device__ __forceinline__ void queue_item_1d(const Stage1DArgs& a1, const Tile 
 template <typename R, int K, int KIND>
 __device__ __forceinline__ void queue_item_2d(const Stage2DArgs& a2, const Inst2D& in, Ctl* ctl, int tile,
                                               unsigned char* smem) {
-    if constexpr (sizeof(R) == sizeof(float))
+    if constexpr (warp_tiles_2d(sizeof(R) == sizeof(float), K))
+        stage2d_warp_body<KIND>(a2, in, ctl, tile, reinterpret_cast<float*>(smem));
+    else if constexpr (sizeof(R) == sizeof(float))
         stage2d_fast_body<KIND, K>(a2, in, ctl, tile, reinterpret_cast<float*>(smem));
     else
         stage2d_body<R, double, KIND>(a2, in, ctl, tile, smem);
 }
 
-// CTAs per SM the register allocation aims for: 5 for the specialised mixed-precision k = 3
-// kernels (48 registers a thread; their shared memory allows at least as many), else no bound
+// CTAs per SM the register allocation aims for: 5 for the specialised mixed-precision k = 3 1D
+// kernels (48 registers a thread; their shared memory allows at least as many), 4 for the 2D ones
+// (64 registers for the pairs of fields), else no bound
 template <typename R, int K, bool CHAR, int SHAPE>
 constexpr int queue_min_blocks() {
-    return (sizeof(R) == sizeof(float) && K == 3 && !CHAR && SHAPE != QS_ANY && SHAPE != QS_2D_ADV) ? 5 : 1;
+    if (!(sizeof(R) == sizeof(float) && K == 3 && !CHAR && SHAPE != QS_ANY)) return 1;
+    return SHAPE == QS_2D_ADV || SHAPE == QS_2D_BURG || SHAPE == QS_2D_EULER ? 4 : 5;
 }
 
 template <typename R, int K, bool CHAR, int SHAPE>
@@ -1710,13 +1933,18 @@ __device__ __forceinline__ void queue_stage_body(const QueueArgs& q) {
 }
 
 
-// the kernels: one without a register bound, one bounded at 5 CTAs per SM (see queue_min_blocks)
+// the kernels: one without a register bound, one bounded at 5 and one at 4 CTAs per SM (see
+// queue_min_blocks)
 template <typename R, int K, bool CHAR, int SHAPE>
 __global__ void __launch_bounds__(THREADS_1D) queue_stage_kernel(QueueArgs q) {
     queue_stage_body<R, K, CHAR, SHAPE>(q);
 }
 template <typename R, int K, bool CHAR, int SHAPE>
 __global__ void __launch_bounds__(THREADS_1D, 5) queue_stage_kernel_b5(QueueArgs q) {
+    queue_stage_body<R, K, CHAR, SHAPE>(q);
+}
+template <typename R, int K, bool CHAR, int SHAPE>
+__global__ void __launch_bounds__(THREADS_1D, 4) queue_stage_kernel_b4(QueueArgs q) {
     queue_stage_body<R, K, CHAR, SHAPE>(q);
 }
 
@@ -1754,12 +1982,11 @@ __global__ void __launch_bounds__(THREADS_1D) queue_alpha_kernel(QueueArgs q) {
     if (two_d) {
         const Inst2D in = q.inst2[w.inst];
         const int64_t cells = in.nx * in.ny;
-        const int tx0 = (w.start % in.tiles_x) * TX_2D, ty0 = (w.start / in.tiles_x) * TY_2D;
-        const int qy = threadIdx.x / TX_2D, qx = threadIdx.x - qy * TX_2D;
-        const int64_t gi = tx0 + qx, gj = ty0 + qy;
-        if (gi < in.nx && gj < in.ny) {
-            const R* base = u + in.off;
-            const int64_t i = gj * in.nx + gi;
+        // item w.start of the instance's tiles: an even share of the cells
+        const int64_t nitems = (int64_t)in.tiles_x * in.tiles_y, share = (cells + nitems - 1) / nitems;
+        const int64_t end = min(cells, (w.start + 1) * share);
+        const R* base = u + in.off;
+        for (int64_t i = w.start * share + threadIdx.x; i < end; i += blockDim.x) {
             if (kind == NPW_FLUX_EULER2D_)
                 queue_speed_cell<R, NPW_FLUX_EULER2D_>(base, cells, i, q.mp, true, &sx, &sy, &bad);
             else if (kind == NPW_FLUX_BURGERS_)
@@ -1965,17 +2192,26 @@ struct Launchers {
                 }
                 return cudaGetLastError();
             }
-            // the mixed path: the phased kernel, k = 3 or k = 2
+            // the mixed path: the warp-task kernel for k = 3, the flat phased kernel for k = 2
             switch (kind * 4 + a.mp.k) {
                 case NPW_FLUX_ADVECTION * 4 + 3:
-                    stage2d_fast_kernel<NPW_FLUX_ADVECTION_, 3><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<1>() * sizeof(float), s>>>(a);
+                    stage2d_warp_kernel<NPW_FLUX_ADVECTION_><<<tiles, THREADS_1D, stage2d_warp_smem_floats<1>() * sizeof(float), s>>>(a);
                     break;
                 case NPW_FLUX_BURGERS * 4 + 3:
-                    stage2d_fast_kernel<NPW_FLUX_BURGERS_, 3><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<1>() * sizeof(float), s>>>(a);
+                    stage2d_warp_kernel<NPW_FLUX_BURGERS_><<<tiles, THREADS_1D, stage2d_warp_smem_floats<1>() * sizeof(float), s>>>(a);
                     break;
-                case NPW_FLUX_EULER2D * 4 + 3:
-                    stage2d_fast_kernel<NPW_FLUX_EULER2D_, 3><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<4>() * sizeof(float), s>>>(a);
+                case NPW_FLUX_EULER2D * 4 + 3: {
+                    static bool carveout = false;  // four CTAs of 45 KB an SM
+                    if (!carveout) {
+                        const cudaError_t e = cudaFuncSetAttribute(stage2d_warp_kernel<NPW_FLUX_EULER2D_>,
+                                                                   cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                                   (int)cudaSharedmemCarveoutMaxShared);
+                        if (e != cudaSuccess) return e;
+                        carveout = true;
+                    }
+                    stage2d_warp_kernel<NPW_FLUX_EULER2D_><<<tiles, THREADS_1D, stage2d_warp_smem_floats<4>() * sizeof(float), s>>>(a);
                     break;
+                }
                 case NPW_FLUX_ADVECTION * 4 + 2:
                     stage2d_fast_kernel<NPW_FLUX_ADVECTION_, 2><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<1>() * sizeof(float), s>>>(a);
                     break;
