@@ -518,10 +518,10 @@ std::array<int, 6> tune_key(const npw_params* p, int kind, int m) {
 // SM and a 20011-cell line on 20: FP64 advection N = 200, one step 90 -> 63 us, 100 steps 8.2 ->
 // 5.4 ms; FP64 1D Euler N = 20011, one step 1071 -> 194 us; mixed Burgers N = 5613, 150 steps
 // 3.75 -> 2.50 ms.
-int auto_tile(const std::vector<int64_t>& n_of, int halo) {
+int auto_tile(const std::vector<int64_t>& n_of, int halo, int min_warps = 1) {
     int best = 0;
     int64_t best_cost = 0;
-    for (int w = 1; w <= npw::TILE_1D / 32; w *= 2) {
+    for (int w = min_warps; w <= npw::TILE_1D / 32; w *= 2) {
         const int t = 32 * w - halo;
         int64_t tiles = 0;
         for (int64_t n : n_of) tiles += (n + t - 1) / t;
@@ -535,6 +535,28 @@ int auto_tile(const std::vector<int64_t>& n_of, int halo) {
 }
 // faces beyond its cells that a tile of the face-based / of the compensated stage kernel works on
 constexpr int HALO_FACES = 1, HALO_COMP = 3;
+
+// The work queue's tile of these 1D lines.  Fused steps: 484, 228 or 100 cells (whole warp tasks, see
+// step1d_fused_warp_body), the one whose busiest SM of four resident CTAs has the least to do, tile +
+// 28 cells' worth per tile.  Else auto_tile, in tiles of at least 255 cells for the characteristic
+// float body, whose CTAs hold few warps per SM.  Against fixed 1024-cell (fused: 512-cell) tiles: 64
+// characteristic Euler lines of 256 to 16384 cells, 60 steps, 6.9 -> 4.9 ms; the FP64 lane of a server
+// with 24 requests up to 4096 cells went from 24 to 7 ms.
+int queue_tile(const std::vector<int64_t>& n_of, bool fused, bool characteristic_f32) {
+    if (!fused) return auto_tile(n_of, HALO_FACES, characteristic_f32 ? 8 : 2);
+    int best = 0;
+    int64_t best_cost = 0;
+    for (int t : {100, 228, 484}) {
+        int64_t tiles = 0;
+        for (int64_t n : n_of) tiles += (n + t - 1) / t;
+        const int64_t cost = (tiles + 4 * npw::NUM_SMS - 1) / (4 * npw::NUM_SMS) * (t + 28);
+        if (best == 0 || cost <= best_cost) {
+            best = t;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
 
 int resolve_tile(const npw_params* p, int kind, int m, int automatic) {
     if (p->tile_1d > 0) return p->tile_1d;
@@ -1567,7 +1589,7 @@ npw_status check_queue(const npw_queue_instance* inst, int count, const npw_para
         if (q.offset < 0) return fail(NPW_EINVAL, "instance %d: negative offset", i);
         const int64_t end = q.offset + cells_of(q);
         arena = end > arena ? end : arena;
-        items += items_of(q, npw::TILE_1D_MIN);
+        items += items_of(q, npw::TILE_QUEUE_MIN);
     }
     if (items > ((int64_t)1 << 30)) return fail(NPW_EINVAL, "too many work items");
     *arena_elems = arena;
@@ -1761,18 +1783,18 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
         if (inst[i].ny == 0) kind_cells[inst[i].flux_kind] += cells_of(inst[i]);
     int main_kind = 0;
     for (int k = 1; k < 3; ++k) main_kind = kind_cells[k] > kind_cells[main_kind] ? k : main_kind;
-    int tile = resolve_tile(params, main_kind, flux_m(main_kind), npw::TILE_1D);
     // a batch of compensated float 1D items alone takes one launch per RK3 step
     bool any2d = false;
-    for (int i = 0; i < count; ++i) any2d |= inst[i].ny != 0;
+    std::vector<int64_t> lines;
+    for (int i = 0; i < count; ++i) {
+        any2d |= inst[i].ny != 0;
+        if (inst[i].ny == 0 && !resident_ok(params, flux_m(inst[i].flux_kind), inst[i].nx)) lines.push_back(inst[i].nx);
+    }
     r.fused = r.comp && !any2d;
-    // automatic tile of fused steps: at most the size whose shared memory (six arrays of
-    // tile + 18 cells per field) still lets the register-bound 5 CTAs share an SM (on the 1D
-    // Euler batch: 512 cells 5.3e9 cell-updates/s, 1024 4.6e9, 2048 2.3e9)
-    if (params->tile_1d <= 0 && r.fused)
-        while (tile > npw::TILE_1D_MIN && npw::fused1d_smem_floats(tile, flux_m(main_kind)) * sizeof(float) >
-                                              (size_t)44 * 1024)
-            tile /= 2;
+    // (npw_autotune_1d times the per-stage kernels: its choice is not for fused steps)
+    const int automatic = queue_tile(lines, r.fused, r.fp32 && r.characteristic);
+    const int tile = r.fused ? (params->tile_1d > 0 ? params->tile_1d : automatic)
+                             : resolve_tile(params, main_kind, flux_m(main_kind), automatic);
     // descriptors; mixed-precision 1D instances that fit in shared memory run resident
     std::vector<npw::InstDev> h1(count);
     std::vector<npw::Inst2D> h2(count);
@@ -1972,15 +1994,6 @@ double now_s(std::chrono::steady_clock::time_point t0) {
     return std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
 }
 
-// 1D tile of the float lane's fused steps: the largest whose six shared arrays (tile + 18 cells
-// per field) stay within 44 KB, so that five CTAs share an SM (1024 cells for m = 1, 512 for
-// 1D Euler)
-int fused_tile(int m) {
-    int t = npw::TILE_1D;
-    while (t > npw::TILE_1D_MIN && npw::fused1d_smem_floats(t, m) * sizeof(float) > (size_t)44 * 1024) t /= 2;
-    return t;
-}
-
 }  // namespace
 
 struct npw_server {
@@ -2132,12 +2145,10 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
         g.is2d = sl.is2d;
         g.m = sl.m;
         g.fused = sl.fused;
-        g.tile = sl.fused ? fused_tile(sl.m) : npw::TILE_1D;
         hk[k] = sl.req.flux_kind;
         h2d[k] = sl.is2d;
         if (!sl.is2d) {
-            h1[k] = npw::InstDev{sl.off, sl.req.n, sl.req.dx, sl.req.t_end, sl.req.cfl, sl.req.bc,
-                                 (int32_t)tiles_of(sl.req.n, g.tile)};
+            h1[k] = npw::InstDev{sl.off, sl.req.n, sl.req.dx, sl.req.t_end, sl.req.cfl, sl.req.bc, 0};
         } else {
             npw::Inst2D& d = h2[k];
             d.off = sl.off;
@@ -2152,6 +2163,13 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
             plan_2d(d, npw::warp_tiles_2d(lane.fp32, lane.mp.k));
         }
         if (sl.fresh) fresh.push_back(k);
+    }
+    for (Group& g : grp) {
+        if (g.is2d || g.members.empty()) continue;
+        std::vector<int64_t> lines;
+        for (int k : g.members) lines.push_back(h1[k].n);
+        g.tile = queue_tile(lines, g.fused, false);
+        for (int k : g.members) h1[k].ntiles = (int32_t)tiles_of(h1[k].n, g.tile);
     }
     // work items, contiguous per group; the admitted requests' items likewise
     for (int gi = 0; gi < kGroups; ++gi) {

@@ -304,6 +304,7 @@ cudaError_t launch_tune_init(R* u, int64_t n, int m, cudaStream_t st);
 
 constexpr int TILE_1D = 1024;     // largest automatic tile of the 1D stage kernels (cells per CTA)
 constexpr int TILE_1D_MIN = 256;  // smallest tile params.tile_1d may choose (sizes the tile tables)
+constexpr int TILE_QUEUE_MIN = 63;  // smallest tile of the work queue and the server (sizes their item tables)
 constexpr int NUM_SMS = 152;      // SMs of the GPU this library is written for (automatic tiles)
 constexpr int RES_GHOST = 3;       // ghost cells on each side of the resident kernel's state arrays
 constexpr size_t RESIDENT_SMEM_MAX = 200 * 1024;  // shared memory a resident CTA may use

@@ -637,8 +637,8 @@ __device__ __forceinline__ void stage1d_fast_body(const Stage1DArgs& a, const Ti
 // boundary rule from the tile's own stage values (a periodic ghost is the same computation as
 // the cell it wraps to).  u^n is read from `uin` and u^{n+1} written to `uout`: the two state
 // buffers alternate between steps (neighbouring tiles read the halo of u^n in the same launch).
-// Shared memory (floats, span = tile + 18 cells per field): u^n, the stage input, d, eta, v^-,
-// v^+.
+// Shared memory (floats, span = tile + 18 cells per field): u^n, the stage input, d, v^-, v^+ (k = 3:
+// and eta).  This body is k = 2, whose shape parameters belong to the cell; k = 3 follows below.
 // ---------------------------------------------------------------------------------------
 // the stage values of the ghost cells of [lo, hi) (extended indices; cell e is global cell
 // c0 - FUSE_HALO + e) from the boundary rule: transmissive and the right end of an inflow
@@ -656,7 +656,7 @@ __device__ __forceinline__ void fused_fill_ghosts(float* x, int lo, int hi, int 
     }
 }
 
-template <int KIND, int K>
+template <int KIND>
 __device__ __forceinline__ void step1d_fused_body(const Stage1DArgs& a, const Tile td, const InstDev& in, Ctl* ctl,
                                                   unsigned char* smem_raw) {
     constexpr int M = kind_m<KIND>();
@@ -668,8 +668,7 @@ __device__ __forceinline__ void step1d_fused_body(const Stage1DArgs& a, const Ti
     float* su0 = reinterpret_cast<float*>(smem_raw);  // u^n
     float* sx = su0 + span_max * M;                    // input of the current stage
     float* sd = sx + span_max * M;                     // d1, then d2
-    float* se = sd + span_max * M;                     // eta of face e (between e-1 and e)
-    float* svm = se + span_max * M;                    // v^- at the right face of cell e
+    float* svm = sd + span_max * M;                    // v^- at the right face of cell e
     float* svp = svm + span_max * M;                   // v^+ at the left face of cell e
     if (*(volatile int32_t*)&ctl->done) return;       // uniform over the CTA
     const int64_t n = in.n;
@@ -714,17 +713,6 @@ __device__ __forceinline__ void step1d_fused_body(const Stage1DArgs& a, const Ti
 #pragma unroll 1
     for (int st = 0; st < 3; ++st) {
         const int L = 3 * (st + 1), R = span - 3 * (st + 1);  // cells updated by this stage: [L, R)
-        // F: eta of the faces q in [L - 1, R + 2) (face q between cells q - 1 and q)
-        if constexpr (K == 3) {
-            for (int idx = threadIdx.x; idx < (R - L + 3) * M; idx += blockDim.x) {
-                const int q = L - 1 + idx / M, k = idx - (q - L + 1) * M;
-                uint32_t fl = 0;
-                se[q * M + k] = fast::face_eta(sx[(q - 2) * M + k], sx[(q - 1) * M + k], sx[q * M + k],
-                                               sx[(q + 1) * M + k], fp, &fl);
-                if (face_owned(q - H, cnt, last_tile)) ec.face_k3(fl);
-            }
-            __syncthreads();
-        }
         // C: cells e in [L - 1, R + 1): v^- at face e + 1, v^+ at face e
         for (int idx = threadIdx.x; idx < (R - L + 2) * M; idx += blockDim.x) {
             const int e = L - 1 + idx / M, k = idx - (e - L + 1) * M;
@@ -732,13 +720,9 @@ __device__ __forceinline__ void step1d_fused_body(const Stage1DArgs& a, const Ti
 #pragma unroll
             for (int j = 0; j < 5; ++j) c[j] = sx[(e - 2 + j) * M + k];
             float vm, vp;
-            if constexpr (K == 3) {
-                fast::cell_recon(c, se[(e + 1) * M + k], se[e * M + k], fp, &vm, &vp);
-            } else {
-                const uint32_t d = fast::cell_recon_k2(c + 1, 0.0, a.mp, fp, &vm, &vp);
-                if (face_owned(e + 1 - H, cnt, last_tile)) fast::count_k2(ec, d, 0);
-                if (face_owned(e - H, cnt, last_tile)) fast::count_k2(ec, d, 1);
-            }
+            const uint32_t d = fast::cell_recon_k2(c + 1, 0.0, a.mp, fp, &vm, &vp);
+            if (face_owned(e + 1 - H, cnt, last_tile)) fast::count_k2(ec, d, 0);
+            if (face_owned(e - H, cnt, last_tile)) fast::count_k2(ec, d, 1);
             svm[e * M + k] = vm;
             svp[e * M + k] = vp;
         }
@@ -781,6 +765,196 @@ __device__ __forceinline__ void step1d_fused_body(const Stage1DArgs& a, const Ti
             __syncthreads();
             if (!periodic && (e0 > L || e0 + n < (int64_t)R)) {
                 fused_fill_ghosts<M>(sx, L, R, c0, n, in.bc, a.mp);
+                __syncthreads();
+            }
+        }
+    }
+    flush_counts(ec, ctl, a.mp);
+    if (a.advance) {
+        const double b = block_max_nan_f(vmaxf, bad, red, redbad);
+        if (threadIdx.x == 0) {
+            atomicMax(&ctl->alpha_next_bits, (unsigned long long)__double_as_longlong(b));
+            __threadfence();
+            const unsigned prev = atomicAdd(&ctl->tiles_done, 1u);
+            if (prev == (unsigned)in.ntiles - 1u) {
+                __threadfence();
+                finalize_1d(ctl, in);
+            }
+        }
+    }
+}
+
+// the same ghost cells in the field-major arrays of the warp-task body ([M][S])
+template <int M>
+__device__ __forceinline__ void fused_fill_ghosts_fm(float* x, int S, int lo, int hi, int c0, int64_t n, int bc,
+                                                     const MethodParams& mp) {
+    const int e0 = FUSE_HALO - c0;                   // extended index of cell 0
+    const int64_t e1 = (int64_t)e0 + n - 1;          // of cell n - 1
+    for (int e = lo + (int)threadIdx.x; e < hi; e += blockDim.x) {
+        if (e >= e0 && e <= e1) continue;
+#pragma unroll
+        for (int k = 0; k < M; ++k)
+            x[k * S + e] = e < e0 ? (bc == NPW_BC_INFLOW ? mp.inflow_f[k] : x[k * S + e0]) : x[k * S + (int)e1];
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// The fused step of k = 3 in warp tasks: the phases of step1d_fused_body with field-major arrays; a task
+// of the eta and reconstruction phases is 64 faces or cells of one field, lane l taking l and l + 32
+// of them as one f32x2 pair; a task of the update phase is 31 cells, each lane forming the flux on
+// its left and taking the one on its right from its neighbour (the flat body formed both).  A task's
+// addresses are a lane offset, where the flat loop divided every index by the field count.  Same
+// arithmetic per face, same bits.  The automatic tiles (484, 228, 100 cells) make the largest stage
+// fill whole tasks: tile + 15 faces in blocks of 64, tile + 12 cells in tasks of 31.  Bound by
+// instruction issue (70% of the slots).  1D Euler, 96 lines of 256 to 65536 cells, 60 steps: one step
+// 135 -> 93 M warp instructions at equal work, the run 6.78 -> 5.02 ms.
+// ---------------------------------------------------------------------------------------
+template <int KIND>
+__device__ __forceinline__ void step1d_fused_warp_body(const Stage1DArgs& a, const Tile td, const InstDev& in, Ctl* ctl,
+                                                       unsigned char* smem_raw) {
+    constexpr int M = kind_m<KIND>(), H = FUSE_HALO, NW = THREADS_1D / 32;
+    using fast::F2;
+    __shared__ float red[32];
+    __shared__ int redbad[32];
+    __shared__ float s_lam;
+    const int S = a.tile + 2 * H;                     // stride of a field
+    float* su0 = reinterpret_cast<float*>(smem_raw);  // u^n
+    float* sx = su0 + S * M;                          // input of the current stage
+    float* sd = sx + S * M;                           // d1, then d2
+    float* se = sd + S * M;                           // eta of face e (between e-1 and e)
+    float* svm = se + S * M;                          // v^- at the right face of cell e
+    float* svp = svm + S * M;                         // v^+ at the left face of cell e
+    if (*(volatile int32_t*)&ctl->done) return;       // uniform over the CTA
+    const int n = (int)in.n;
+    const int c0 = td.start;
+    const int cnt = min(n - c0, a.tile);
+    const int span = cnt + 2 * H;
+    const float* uin = reinterpret_cast<const float*>(a.uin) + in.off;
+    float* uout = reinterpret_cast<float*>(a.uout) + in.off;
+    float* cr = a.c + in.off;
+    const bool periodic = in.bc == NPW_BC_PERIODIC;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int j = threadIdx.x; j < span; j += blockDim.x) {
+        int g = c0 - H + j;
+        bool inflow = false;
+        if (periodic) {  // n >= 6: at most two wraps on either side
+            if (g < 0) g += n;
+            if (g < 0) g += n;
+            if (g >= n) g -= n;
+            if (g >= n) g -= n;
+        } else {
+            inflow = g < 0 && in.bc == NPW_BC_INFLOW;
+            g = g < 0 ? 0 : (g >= n ? n - 1 : g);
+        }
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const float x = inflow ? a.mp.inflow_f[k] : uin[(int64_t)k * n + g];
+            su0[k * S + j] = x;
+            sx[k * S + j] = x;
+        }
+    }
+    if (threadIdx.x == 0) s_lam = (float)(*(volatile double*)&ctl->dt / in.dx);
+    const float alpha = (float)*(volatile double*)&ctl->alpha;
+    const fast::FParams fp = fast::fparams(a.mp);
+    const bool last_tile = c0 + cnt == n;
+    const int e0 = H - c0;  // extended index of global cell 0
+    EtaCount ec;
+    float vmaxf = 0.0f;
+    bool bad = false;
+    __syncthreads();
+    const float lam = s_lam;
+#pragma unroll 1
+    for (int st = 0; st < 3; ++st) {
+        const int L = 3 * (st + 1), R = span - 3 * (st + 1);  // cells updated by this stage: [L, R)
+        // E: eta of the faces q in [L - 1, R + 2) (face q between cells q - 1 and q)
+        const int nbe = (R - L + 3 + 63) / 64;
+#pragma unroll 1
+        for (int t = warp; t < nbe * M; t += NW) {
+            const int k = t / nbe, q = L - 1 + (t - k * nbe) * 64 + lane;
+            if (q >= R + 2) continue;
+            const bool two = q + 32 < R + 2;
+            const float *x = sx + k * S + q, *y = two ? x + 32 : x;
+            F2 w[1][4], eta[1];
+            uint32_t fl[1][2];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) w[0][j] = F2{make_float2(x[j - 2], y[j - 2])};
+            fast::face_eta_n<F2, 1>(w, fp, eta, fl);
+            se[k * S + q] = eta[0].v.x;
+            if (two) se[k * S + q + 32] = eta[0].v.y;
+            if (face_owned(q - H, cnt, last_tile)) ec.face_k3(fl[0][0]);
+            if (two && face_owned(q + 32 - H, cnt, last_tile)) ec.face_k3(fl[0][1]);
+        }
+        __syncthreads();
+        // C: cells e in [L - 1, R + 1): v^- at face e + 1, v^+ at face e
+        const int nbc = (R - L + 2 + 63) / 64;
+#pragma unroll 1
+        for (int t = warp; t < nbc * M; t += NW) {
+            const int k = t / nbc, e = L - 1 + (t - k * nbc) * 64 + lane;
+            if (e >= R + 1) continue;
+            const bool two = e + 32 < R + 1;
+            const int i = k * S + e, o = two ? 32 : 0;
+            F2 c[5], vm, vp;
+#pragma unroll
+            for (int j = 0; j < 5; ++j) c[j] = F2{make_float2(sx[i + j - 2], sx[i + o + j - 2])};
+            fast::cell_recon<F2>(c, F2{make_float2(se[i + 1], se[i + o + 1])}, F2{make_float2(se[i], se[i + o])}, fp, &vm, &vp);
+            svm[i] = vm.v.x;
+            svp[i] = vp.v.x;
+            if (two) {
+                svm[i + 32] = vm.v.y;
+                svp[i + 32] = vp.v.y;
+            }
+        }
+        __syncthreads();
+        // U: flux of the face on the left of cell e, eq. PDE1 and the stage in increment form
+#pragma unroll 1
+        for (int b = L + warp * 31; b < R; b += NW * 31) {
+            const int e = b + lane;
+            float vl[M], vr[M], hl[M], hr[M];
+#pragma unroll
+            for (int k = 0; k < M; ++k) hl[k] = 0.0f;
+            if (e <= R) {
+#pragma unroll
+                for (int k = 0; k < M; ++k) {
+                    vl[k] = svm[k * S + e - 1];
+                    vr[k] = svp[k * S + e];
+                }
+                lf_flux<float, KIND, M>(vl, vr, alpha, a.mp, 0, hl);
+            }
+#pragma unroll
+            for (int k = 0; k < M; ++k) hr[k] = __shfl_down_sync(0xffffffffu, hl[k], 1);
+            const int g = c0 - H + e;
+            if (lane == 31 || e >= R || (!periodic && (g < 0 || g >= n))) continue;  // (a ghost: filled below)
+            if (st < 2) {
+#pragma unroll
+                for (int k = 0; k < M; ++k) {
+                    const float du = lam * (hl[k] - hr[k]);
+                    const float d = st == 0 ? du : 0.25f * (sd[k * S + e] + du);
+                    sd[k * S + e] = d;
+                    sx[k * S + e] = su0[k * S + e] + d;
+                }
+            } else {
+                float U[M];
+#pragma unroll
+                for (int k = 0; k < M; ++k) {
+                    const float du = lam * (hl[k] - hr[k]);
+                    const int64_t ix = (int64_t)k * n + g;
+                    const float base = su0[k * S + e];
+                    const float y = kTwoThirdsF * (sd[k * S + e] + du) + cr[ix];
+                    const float t = base + y;
+                    cr[ix] = y - (t - base);
+                    uout[ix] = t;
+                    U[k] = t;
+                    bad |= !finite_(t);
+                }
+                const float sp = wave_speed<float, KIND>(U, a.mp, 0);
+                bad |= !finite_(sp);
+                vmaxf = sp > vmaxf ? sp : vmaxf;
+            }
+        }
+        if (st < 2) {
+            __syncthreads();
+            if (!periodic && (e0 > L || e0 + n < R)) {
+                fused_fill_ghosts_fm<M>(sx, S, L, R, c0, n, in.bc, a.mp);
                 __syncthreads();
             }
         }
@@ -1826,9 +2000,12 @@ template <typename R, int K, bool CHAR, int KIND>
 __device__ __forceinline__ void queue_item_1d(const Stage1DArgs& a1, const Tile w, const InstDev& in, Ctl* ctl,
                                               unsigned char* smem) {
     if constexpr (sizeof(R) == sizeof(float) && !CHAR) {
-        if (a1.stage == QUEUE_FUSED_STEP)
-            step1d_fused_body<KIND, K>(a1, w, in, ctl, smem);
-        else
+        if (a1.stage == QUEUE_FUSED_STEP) {
+            if constexpr (K == 3)
+                step1d_fused_warp_body<KIND>(a1, w, in, ctl, smem);
+            else
+                step1d_fused_body<KIND>(a1, w, in, ctl, smem);
+        } else
             stage1d_fast_body<KIND, K>(a1, w, in, ctl, smem);
     } else
         stage1d_body<R, double, KIND, CHAR && KIND == NPW_FLUX_EULER1D_>(a1, w, in, ctl, smem);
@@ -1844,13 +2021,11 @@ __device__ __forceinline__ void queue_item_2d(const Stage2DArgs& a2, const Inst2
         stage2d_body<R, double, KIND>(a2, in, ctl, tile, smem);
 }
 
-// CTAs per SM the register allocation aims for: 5 for the specialised mixed-precision k = 3 1D
-// kernels (48 registers a thread; their shared memory allows at least as many), 4 for the 2D ones
-// (64 registers for the pairs of fields), else no bound
+// CTAs per SM the register allocation aims for: 4 for the specialised mixed-precision k = 3 kernels
+// (64 registers a thread for the f32x2 pairs; their shared memory allows as many), else no bound
 template <typename R, int K, bool CHAR, int SHAPE>
 constexpr int queue_min_blocks() {
-    if (!(sizeof(R) == sizeof(float) && K == 3 && !CHAR && SHAPE != QS_ANY)) return 1;
-    return SHAPE == QS_2D_ADV || SHAPE == QS_2D_BURG || SHAPE == QS_2D_EULER ? 4 : 5;
+    return sizeof(R) == sizeof(float) && K == 3 && !CHAR && SHAPE != QS_ANY ? 4 : 1;
 }
 
 template <typename R, int K, bool CHAR, int SHAPE>
@@ -1933,14 +2108,9 @@ __device__ __forceinline__ void queue_stage_body(const QueueArgs& q) {
 }
 
 
-// the kernels: one without a register bound, one bounded at 5 and one at 4 CTAs per SM (see
-// queue_min_blocks)
+// the kernels: one without a register bound, one bounded at 4 CTAs per SM (see queue_min_blocks)
 template <typename R, int K, bool CHAR, int SHAPE>
 __global__ void __launch_bounds__(THREADS_1D) queue_stage_kernel(QueueArgs q) {
-    queue_stage_body<R, K, CHAR, SHAPE>(q);
-}
-template <typename R, int K, bool CHAR, int SHAPE>
-__global__ void __launch_bounds__(THREADS_1D, 5) queue_stage_kernel_b5(QueueArgs q) {
     queue_stage_body<R, K, CHAR, SHAPE>(q);
 }
 template <typename R, int K, bool CHAR, int SHAPE>
