@@ -782,9 +782,16 @@ npw_status launch_resident_set(const ResidentLaunch& rl, const std::vector<int32
         const int64_t n = n_of[i];
         cls[n > 4096 ? 0 : (n > 2048 ? 1 : (n > 1024 ? 2 : 3))].push_back(i);
     }
-    // two 512-thread CTAs per SM for the largest class (64 registers per thread fill the register
-    // file either way) measured 10% faster than one 1024-thread CTA
-    static const int threads[4] = {512, 512, 256, 128};
+    // Threads of a CTA.  k = 3 (116 registers a thread, 512 threads an SM): a class with a CTA for no
+    // more than every SM takes the larger CTA, since its longest instance is then the critical path; a
+    // larger class takes two or more CTAs per SM, one computing while another waits at its barrier.
+    // Burgers, N in [64, 8192], 300 steps: 1024 instances (146 in the largest class) 9.1 ms with 512
+    // threads, 12.5 ms with 256; 4096 instances (585) 30.1 and 28.1 ms.  k = 2 (64 registers): 512-thread
+    // CTAs for the two largest classes.
+    static const int few[4] = {512, 512, 512, 256}, many[4] = {256, 256, 256, 128}, k2[4] = {512, 512, 256, 128};
+    int threads[4];
+    for (int c = 0; c < 4; ++c)
+        threads[c] = rl.mp.k == 2 ? k2[c] : ((int)cls[c].size() <= npw::NUM_SMS ? few[c] : many[c]);
     std::vector<int32_t> all;
     size_t offs[5] = {0, 0, 0, 0, 0};
     for (int c = 0; c < 4; ++c) {

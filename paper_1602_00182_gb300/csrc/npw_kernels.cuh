@@ -408,54 +408,35 @@ __device__ __forceinline__ void stage1d_body(const Stage1DArgs& a, const Tile td
 }
 
 // ---------------------------------------------------------------------------------------
-// One warp's pass over the cells [lo, hi) of a line, for one RK stage of the resident kernel
-// (the per-stage kernel runs the same arithmetic in phases over its tile): lane l of the chunk
-// at base takes
-//   face f = base + l: its eta (k = 3, cells f-2..f+1);
-//   cell f - 1: its reconstruction (cells f-3..f+1), v^+ at face f - 1 with the eta of face
-//     f - 1 (lane l - 1) and v^- at face f with the eta of face f;
+// One warp's pass over the cells [lo, hi) of a line, for one RK stage of the resident kernel, k = 2 (the
+// shape parameters belong to the cell): lane l of the chunk at base takes
+//   cell f - 1, f = base + l: its reconstruction (cells f-2..f), v^- at face f and v^+ at face f - 1;
 //   face f - 1: the Lax-Friedrichs flux from v^- of cell f - 2 (lane l - 1) and v^+ of cell f - 1;
 //   cell f - 2: the update, upd(j, flux of face j, flux of face j + 1).
-// Lane 0 takes the lane l - 1 values from lane 31 of the previous chunk.  Faces lo..hi, cells
-// lo-1..hi and the updates of cells lo..hi-1 are covered by f = lo..hi+1; faces lo and hi are
-// also computed by the warps on either side, from the same data, so the copies agree bit for
-// bit.  X(k, i) is the stage input of field k at cell i, for i in lo-3..hi+2.
+// Lane 0 takes the lane l - 1 values from lane 31 of the previous chunk.  Faces lo and hi are also
+// computed by the warps on either side, from the same data, so the copies agree bit for bit.
+// X(k, i) is the stage input of field k at cell i.
 // ---------------------------------------------------------------------------------------
-template <int KIND, int K, int M, typename LoadX, typename Upd>
+template <int KIND, int M, typename LoadX, typename Upd>
 __device__ __forceinline__ void warp_line_pass(int lo, int hi, int n, int lane, const fast::FParams& fp,
                                                const MethodParams& mp, float alpha, LoadX X, Upd upd, EtaCount& ec) {
-    float c_eta[M], c_vm[M], c_h[M];
+    float c_vm[M], c_h[M];
 #pragma unroll
-    for (int k = 0; k < M; ++k) c_eta[k] = c_vm[k] = c_h[k] = 0.0f;
+    for (int k = 0; k < M; ++k) c_vm[k] = c_h[k] = 0.0f;
     for (int base = lo; base <= hi + 1; base += 32) {
         const int f = base + lane, i = f - 1, j = f - 2;
-        const bool face_ok = f <= hi, cell_ok = i <= hi;
         float vm[M], vp[M];
 #pragma unroll
         for (int k = 0; k < M; ++k) {
-            float c[5], eta = 0.0f;
             vm[k] = vp[k] = 0.0f;
-            if (cell_ok) {
+            if (i <= hi) {
+                float c[3];
 #pragma unroll
-                for (int q = 0; q < 5; ++q) c[q] = X(k, i - 2 + q);
-                if (K == 3 && face_ok) {
-                    uint32_t fl = 0;
-                    eta = fast::face_eta(c[1], c[2], c[3], c[4], fp, &fl);
-                    if (f < hi || f == n) ec.face_k3(fl);
-                }
-            }
-            if constexpr (K == 3) {
-                float eprev = __shfl_up_sync(0xffffffffu, eta, 1);
-                if (lane == 0) eprev = c_eta[k];
-                c_eta[k] = __shfl_sync(0xffffffffu, eta, 31);
-                if (cell_ok) fast::cell_recon(c, eta, i >= lo ? eprev : 0.0f, fp, &vm[k], &vp[k]);
-            } else {
-                if (cell_ok) {
-                    // v^- of cell i at face f, v^+ at face f - 1
-                    const uint32_t d = fast::cell_recon_k2(c + 1, 0.0, mp, fp, &vm[k], &vp[k]);
-                    if (f < hi || f == n) fast::count_k2(ec, d, 0);
-                    if (f - 1 >= lo && (f - 1 < hi || f - 1 == n)) fast::count_k2(ec, d, 1);
-                }
+                for (int q = 0; q < 3; ++q) c[q] = X(k, i - 1 + q);
+                // v^- of cell i at face f, v^+ at face f - 1
+                const uint32_t d = fast::cell_recon_k2(c, 0.0, mp, fp, &vm[k], &vp[k]);
+                if (f < hi || f == n) fast::count_k2(ec, d, 0);
+                if (f - 1 >= lo && (f - 1 < hi || f - 1 == n)) fast::count_k2(ec, d, 1);
             }
         }
         // flux of face f - 1
@@ -477,6 +458,61 @@ __device__ __forceinline__ void warp_line_pass(int lo, int hi, int n, int lane, 
         // update of cell j = f - 2 (cells lo..hi-1)
         if (j >= lo && j < hi) upd(j, hl, h);
     }
+}
+
+// ---------------------------------------------------------------------------------------
+// One block of the resident kernel's stage for k = 3: position p = 0..63 is cell b0 - 1 + p, lane l holding
+// p = l and p = l + 32 as one f32x2 pair.  Each position takes the eta of the face on its right, the
+// reconstruction of its cell (with the eta of the position before), the flux on its left (with v^- of the
+// position before) and, for p = 1..62, the update of its cell from its own and the next position's
+// flux, all exchanged by lane shuffles: BLOCK_CELLS cells b0..b0 + 61 without a carry between blocks,
+// so that any warp takes any block.  X(k, i): the stage input, i in -3..n + 2; upd(j, flux of face j,
+// flux of face j + 1).
+// ---------------------------------------------------------------------------------------
+constexpr int BLOCK_CELLS = 62;
+template <int KIND, int M, typename LoadX, typename Upd>
+__device__ __forceinline__ void warp_block_pass(int b0, int n, int lane, const fast::FParams& fp, const MethodParams& mp,
+                                                float alpha, LoadX X, Upd upd, EtaCount& ec) {
+    using fast::F2;
+    auto before = [lane](F2 v) {  // the position before (p = 0 gets its own value)
+        const float xe = __shfl_sync(0xffffffffu, v.v.x, 31);
+        F2 r{make_float2(__shfl_up_sync(0xffffffffu, v.v.x, 1), __shfl_up_sync(0xffffffffu, v.v.y, 1))};
+        if (lane == 0) r.v.y = xe;
+        return r;
+    };
+    const int ix = min(b0 - 1 + lane, n), iy = min(b0 + 31 + lane, n);
+    float ax[M], ay[M], bx[M], by[M], hx[M], hy[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        F2 c[5], eta[1], vm, vp;
+        uint32_t fl[1][2];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) c[q] = F2{make_float2(X(k, ix - 2 + q), X(k, iy - 2 + q))};
+        const F2 w[1][4] = {{c[1], c[2], c[3], c[4]}};
+        fast::face_eta_n<F2, 1>(w, fp, eta, fl);
+        // face b0 + p, counted by this block for p < 62, and face n wherever it falls
+        if (b0 + lane <= n) ec.face_k3(fl[0][0]);
+        const int f = b0 + 32 + lane;
+        if (f <= n && (lane < 30 || (lane == 30 && f == n))) ec.face_k3(fl[0][1]);
+        fast::cell_recon<F2>(c, eta[0], before(eta[0]), fp, &vm, &vp);
+        const F2 vl = before(vm);
+        ax[k] = vl.v.x;
+        ay[k] = vl.v.y;
+        bx[k] = vp.v.x;
+        by[k] = vp.v.y;
+    }
+    lf_flux<float, KIND, M>(ax, bx, alpha, mp, 0, hx);
+    lf_flux<float, KIND, M>(ay, by, alpha, mp, 0, hy);
+    float rx[M], ry[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        const float y0 = __shfl_sync(0xffffffffu, hy[k], 0);
+        rx[k] = __shfl_down_sync(0xffffffffu, hx[k], 1);
+        ry[k] = __shfl_down_sync(0xffffffffu, hy[k], 1);
+        if (lane == 31) rx[k] = y0;
+    }
+    if (lane >= 1 && b0 - 1 + lane < n) upd(b0 - 1 + lane, hx, rx);
+    if (lane <= 30 && b0 + 31 + lane < n) upd(b0 + 31 + lane, hy, ry);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -995,12 +1031,10 @@ static __global__ void comp_copy_kernel(float* dst, const float* src, float* zer
 // ---------------------------------------------------------------------------------------
 // Resident whole-solve kernel (float state, component-wise).  One CTA owns one instance for
 // its whole run: u^n and the two stage values live in shared memory, and thread 0 advances
-// t, alpha and dt between steps.  Each warp owns a contiguous range of cells [lo, hi) and
-// runs a stage on it in one pass without waiting for the other warps: per chunk of 32 faces,
-// each lane forms the eta of its face, reconstructs the cell to its left, computes the flux of
-// the face before and updates the cell before that, taking its left neighbour's values by lane
-// shuffles.  The faces lo and hi are also computed by the neighbouring warps, from the same
-// data, so the copies agree bit for bit.  Warps therefore drift apart within a stage; the only
+// t, alpha and dt between steps.  The warps run a stage without waiting for each other: k = 3 in
+// blocks of 62 cells (warp_block_pass), k = 2 over a contiguous range each (warp_line_pass); the
+// faces between two warps are computed by both, from the same data, so the copies agree bit for
+// bit.  Warps therefore drift apart within a stage; the only
 // CTA-wide barrier is between stages (the next stage reads the neighbours' halo).  Stage values
 // are double-buffered (u^n -> uA -> uB -> u^{n+1}) so no warp overwrites a value another still
 // reads.  Shared memory per field: u^n, uA, uB, each n cells with RES_GHOST ghost cells per side.
@@ -1034,7 +1068,7 @@ __device__ __forceinline__ void res_store(float* p, int i, int n, int bc, float 
 }
 
 template <int KIND, int K>
-__global__ void __launch_bounds__(1024) solve1d_resident_kernel(ResidentArgs a) {
+__global__ void __launch_bounds__(K == 3 ? 512 : 1024) solve1d_resident_kernel(ResidentArgs a) {
     constexpr int M = kind_m<KIND>();
     extern __shared__ __align__(16) float smf[];
     __shared__ float red[32];
@@ -1129,7 +1163,7 @@ __global__ void __launch_bounds__(1024) solve1d_resident_kernel(ResidentArgs a) 
             // stage1d_fast_kernel); stage 3 writes the new state into uA
             const float* D = stage == 1 ? uA : uB;
 #define NPW_X(idx) (stage == 0 ? un[(idx)] : un[(idx)] + D[(idx)])
-            if (lo < hi) {
+            if (K == 3 || lo < hi) {
                 auto X = [&](int k, int i) { return NPW_X(k * NS + RES_GHOST + i); };
                 auto upd = [&](int j, const float* hl, const float* hr) {
                     float U[M];
@@ -1161,7 +1195,13 @@ __global__ void __launch_bounds__(1024) solve1d_resident_kernel(ResidentArgs a) 
                         vmaxf = sp > vmaxf ? sp : vmaxf;
                     }
                 };
-                warp_line_pass<KIND, K, M>(lo, hi, n, lane, fp, a.mp, alphaf, X, upd, ec);
+                if constexpr (K == 3) {
+#pragma unroll 1
+                    for (int b0 = warp * BLOCK_CELLS; b0 < n; b0 += nwarps * BLOCK_CELLS)
+                        warp_block_pass<KIND, M>(b0, n, lane, fp, a.mp, alphaf, X, upd, ec);
+                } else {
+                    warp_line_pass<KIND, M>(lo, hi, n, lane, fp, a.mp, alphaf, X, upd, ec);
+                }
             }
             __syncthreads();
 #undef NPW_X
