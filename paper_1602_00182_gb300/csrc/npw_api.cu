@@ -125,6 +125,8 @@ npw::MethodParams method(const npw_params* p) {
     const float ga_rows[6] = {float(2.0 / 3.0), float(-1.0 / 3.0), float(-1.0 / 3.0), 0.0f, 3.0f, -3.0f};
     const float mq_rows[6] = {float(5.0 / 6.0), float(-2.0 / 3.0), float(-1.0 / 6.0), -1.5f, 6.0f, -4.5f};
     for (int k = 0; k < 6; ++k) mp.pert_f[k] = ga ? ga_rows[k] : mq_rows[k];
+    mp.has_guard = mp.eta_guard > 0.0;
+    mp.has_bound = mp.eta_max > 0.0;
     const float margin = 1.0f + 0x1p-16f;
     mp.guard_switch = !mp.monotone_switch || mp.switch_variant == 0;
     mp.sw24_f = mp.monotone_switch ? 24.0f * margin : 0.0f;
@@ -511,18 +513,29 @@ std::array<int, 6> tune_key(const npw_params* p, int kind, int m) {
     return {dev, kind, m, p->k, p->precision, p->characteristic ? 1 : 0};
 }
 
-// Automatic tile of the 1D per-stage kernels for the given lines: 32 w - halo cells, so that the
-// tile's faces (cells plus `halo` more) fill w warps, with w the power of two that leaves the
+// the compensated float kernels (stage1d_fast_kernel, the resident kernel) cover float,
+// component-wise (k = 3 and k = 2); FP64 and characteristic runs take the face-based stage kernel
+bool compensated(const npw_params* p) {
+    return p->precision == NPW_FP32_MIXED && !p->characteristic;
+}
+
+// Automatic tile of the 1D per-stage kernels for the given lines: w warps' worth of cells (32 w less the
+// faces beyond the cells, or w chunks of the double body), with w the power of two that leaves the
 // busiest SM the fewest warps of work, ceil(tiles / SMs) x w; the larger tile where several tie
 // (its halo is a smaller share).  Against a fixed 1024-cell tile, which puts a 200-cell line on one
 // SM and a 20011-cell line on 20: FP64 advection N = 200, one step 90 -> 63 us, 100 steps 8.2 ->
 // 5.4 ms; FP64 1D Euler N = 20011, one step 1071 -> 194 us; mixed Burgers N = 5613, 150 steps
 // 3.75 -> 2.50 ms.
-int auto_tile(const std::vector<int64_t>& n_of, int halo, int min_warps = 1) {
+enum StageKind { STAGE_FACES, STAGE_COMP, STAGE_DOUBLE };
+StageKind stage_kind(const npw_params* p) {
+    if (compensated(p)) return STAGE_COMP;
+    return p->precision == NPW_FP64 && p->k == 3 && !p->characteristic ? STAGE_DOUBLE : STAGE_FACES;
+}
+int auto_tile(const std::vector<int64_t>& n_of, StageKind kind, int min_warps = 1) {
     int best = 0;
     int64_t best_cost = 0;
     for (int w = min_warps; w <= npw::TILE_1D / 32; w *= 2) {
-        const int t = 32 * w - halo;
+        const int t = kind == STAGE_DOUBLE ? npw::CHUNK_D * w : 32 * w - (kind == STAGE_COMP ? 3 : 1);
         int64_t tiles = 0;
         for (int64_t n : n_of) tiles += (n + t - 1) / t;
         const int64_t cost = (tiles + npw::NUM_SMS - 1) / npw::NUM_SMS * w;
@@ -533,8 +546,6 @@ int auto_tile(const std::vector<int64_t>& n_of, int halo, int min_warps = 1) {
     }
     return best;
 }
-// faces beyond its cells that a tile of the face-based / of the compensated stage kernel works on
-constexpr int HALO_FACES = 1, HALO_COMP = 3;
 
 // The work queue's tile of these 1D lines.  Fused steps: 484, 228 or 100 cells (whole warp tasks, see
 // step1d_fused_warp_body), the one whose busiest SM of four resident CTAs has the least to do, tile +
@@ -542,8 +553,8 @@ constexpr int HALO_FACES = 1, HALO_COMP = 3;
 // float body, whose CTAs hold few warps per SM.  Against fixed 1024-cell (fused: 512-cell) tiles: 64
 // characteristic Euler lines of 256 to 16384 cells, 60 steps, 6.9 -> 4.9 ms; the FP64 lane of a server
 // with 24 requests up to 4096 cells went from 24 to 7 ms.
-int queue_tile(const std::vector<int64_t>& n_of, bool fused, bool characteristic_f32) {
-    if (!fused) return auto_tile(n_of, HALO_FACES, characteristic_f32 ? 8 : 2);
+int queue_tile(const std::vector<int64_t>& n_of, bool fused, StageKind kind, bool characteristic_f32) {
+    if (!fused) return auto_tile(n_of, kind, characteristic_f32 ? 8 : 2);
     int best = 0;
     int64_t best_cost = 0;
     for (int t : {100, 228, 484}) {
@@ -565,12 +576,6 @@ int resolve_tile(const npw_params* p, int kind, int m, int automatic) {
     return it == g_tune.end() ? automatic : it->second;
 }
 
-// the compensated float kernels (stage1d_fast_kernel, the resident kernel) cover float,
-// component-wise (k = 3 and k = 2); FP64 and characteristic runs take the face-based stage kernel
-bool compensated(const npw_params* p) {
-    return p->precision == NPW_FP32_MIXED && !p->characteristic;
-}
-
 // instances the resident kernel can take: compensated float path, fits in shared memory
 bool resident_ok(const npw_params* p, int m, int64_t n) {
     return compensated(p) && p->batch_mode == 0 && npw::resident_smem_bytes(n, m) <= npw::RESIDENT_SMEM_MAX;
@@ -581,7 +586,7 @@ int batch_auto_tile(const npw_instance* inst, int count, int m, const npw_params
     std::vector<int64_t> n_of;
     for (int i = 0; i < count; ++i)
         if (!resident_ok(p, m, inst[i].n)) n_of.push_back(inst[i].n);
-    return auto_tile(n_of, compensated(p) ? HALO_COMP : HALO_FACES);
+    return auto_tile(n_of, stage_kind(p));
 }
 // entries of a batch's tile table: every instance in the smallest tile a run may choose, or the
 // per-stage ones in the automatic tile
@@ -1081,7 +1086,7 @@ static npw_status single_run(void* u, int64_t n, int32_t m, double dx, double t_
     r.mp = method(params);
     r.fp32 = params->precision == NPW_FP32_MIXED;
     r.ws = static_cast<unsigned char*>(workspace);
-    r.tile = resolve_tile(params, flux_kind, m, auto_tile({n}, compensated(params) ? HALO_COMP : HALO_FACES));
+    r.tile = resolve_tile(params, flux_kind, m, auto_tile({n}, stage_kind(params)));
     r.ntiles = tiles_of(n, r.tile);
     r.L = layout_1d(n * m, 1, tiles_of(n), elem_size(params));
     r.s = s;
@@ -1799,7 +1804,7 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
     }
     r.fused = r.comp && !any2d;
     // (npw_autotune_1d times the per-stage kernels: its choice is not for fused steps)
-    const int automatic = queue_tile(lines, r.fused, r.fp32 && r.characteristic);
+    const int automatic = queue_tile(lines, r.fused, stage_kind(params), r.fp32 && r.characteristic);
     const int tile = r.fused ? (params->tile_1d > 0 ? params->tile_1d : automatic)
                              : resolve_tile(params, main_kind, flux_m(main_kind), automatic);
     // descriptors; mixed-precision 1D instances that fit in shared memory run resident
@@ -2175,7 +2180,7 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
         if (g.is2d || g.members.empty()) continue;
         std::vector<int64_t> lines;
         for (int k : g.members) lines.push_back(h1[k].n);
-        g.tile = queue_tile(lines, g.fused, false);
+        g.tile = queue_tile(lines, g.fused, lane.mp.k == 3 ? STAGE_DOUBLE : STAGE_FACES, false);
         for (int k : g.members) h1[k].ntiles = (int32_t)tiles_of(h1[k].n, g.tile);
     }
     // work items, contiguous per group; the admitted requests' items likewise

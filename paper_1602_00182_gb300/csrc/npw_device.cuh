@@ -17,9 +17,15 @@
 #pragma once
 #include <cstdint>
 
+#include "npw_double.cuh"
 #include "npw_internal.h"
 
 namespace npw {
+
+// n / x: the operator, or in double its correctly rounded form with fewer FP64 instructions
+__device__ __forceinline__ float quotient(float n, float x) { return n / x; }
+__device__ __forceinline__ double quotient(double n, double x) { return f64::div(n, x); }
+
 
 // ---------------------------------------------------------------------------------------
 // Table k3.  row = r + 1 for r = -1..2; row r gives the value at face x_{i+1/2} from the
@@ -328,6 +334,66 @@ __device__ __forceinline__ R cell_face_value_k2(const R* c, int side, R eta_c, R
     return v;
 }
 
+// value of a k = 2 cell as cell_face_value_k2<double> gives it (no shift): the ENO candidate alone, or
+// the WENO3 mean with one reciprocal per denominator
+__device__ __forceinline__ double cell_value_k2_d(const double* c, int side, double eta_c, double eta_x, int r,
+                                                  const MethodParams& mp) {
+    const bool ga = mp.rbf == NPW_RBF_GA_;
+    auto cand = [&](int q) {
+        const int row = side == 0 ? q : q - 1;
+        const double eta = row == 0 ? eta_c : eta_x;
+        // rows -1 (3/2, -1/2), 0 (1/2, 1/2), 1 (-1/2, 3/2) with their perturbations
+        const double p0 = row == 0 ? 0.5 : (row < 0 ? 1.5 : -0.5), p1 = row == 0 ? 0.5 : (row < 0 ? -0.5 : 1.5);
+        const double far_ = ga ? -2.0 : -1.5, near_ = ga ? 0.0 : 0.5, mid = ga ? 0.5 : 0.25;
+        const double q0 = row == 0 ? mid : (row < 0 ? far_ : near_), q1 = row == 0 ? mid : (row < 0 ? near_ : far_);
+        return (p0 + q0 * eta) * c[1 - q] + (p1 + q1 * eta) * c[2 - q];
+    };
+    if (mp.scheme == NPW_ENO_ || mp.scheme == NPW_RBF_ENO_) return r == 0 ? cand(0) : cand(1);
+    const double g0 = c[2] - c[1], g1 = c[1] - c[0];
+    double x0 = mp.eps_weno + g0 * g0, x1 = mp.eps_weno + g1 * g1;
+    x0 = x0 * x0;
+    x1 = x1 * x1;
+    const double a0 = f64::div(side == 0 ? 2.0 / 3.0 : 1.0 / 3.0, x0), a1 = f64::div(side == 0 ? 1.0 / 3.0 : 2.0 / 3.0, x1);
+    const double sum = a0 + a1;
+    return f64::div(a0, sum) * cand(0) + f64::div(a1, sum) * cand(1);
+}
+
+// face_field_k2<double> with fewer FP64-pipe instructions and the same bits (see npw_double.cuh)
+__device__ __forceinline__ uint32_t face_field_k2_d(const double* w, const MethodParams& mp, double* vm, double* vp,
+                                                    double tl, double tr, double* eta_out) {
+    uint32_t fl = 0;
+    const bool eno = mp.scheme == NPW_ENO_ || mp.scheme == NPW_RBF_ENO_;
+    int rl = 0, rr = 0;
+    if (eno) {
+        const double d0 = w[2] - w[1], d1 = w[3] - w[2], d2 = w[4] - w[3];
+        rl = f64::abs_less(d0, d1) ? 1 : 0;
+        rr = f64::abs_less(d1, d2) ? 1 : 0;
+    }
+    double el = 0.0, er = 0.0, elx = 0.0, erx = 0.0;
+    if (mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_) {
+        // -a + 2b - c of either cell, the switch's denominator and the numerator of v^- of the left cell
+        const double sl = fma(2.0, w[2], -w[1]) - w[3], sr = fma(2.0, w[3], -w[2]) - w[4];
+        // v^-: r = 0 the central row, 1 the extrapolating one; v^+: the other way round (eta_out: central)
+        const int need_l = eno && !eta_out ? (rl == 0 ? 1 : 2) : 3, need_r = eno ? (rr == 1 ? 1 : 2) : 3;
+        if (mp.monotone_switch && f64::k2_switch(w[1], w[2], w[3], sl))
+            fl |= FL_SWITCH;
+        else
+            f64::eta_k2_pair(w[1], w[2], w[3], sl, tl, need_l, mp, &el, &elx, &fl);
+        if (mp.monotone_switch && f64::k2_switch(w[2], w[3], w[4], sr)) {
+            fl |= FL_SWITCH_R_K2;
+        } else {
+            uint32_t zr = 0;
+            f64::eta_k2_pair(w[4], w[3], w[2], fma(2.0, w[3], -w[4]) - w[2], tr, need_r, mp, &er, &erx, &zr);
+            fl |= zr << 2;  // FL_ZERO_GUARD_R_K2, FL_ZERO_BOUND_R_K2
+        }
+    }
+    *vm = cell_value_k2_d(w + 1, 0, el, elx, rl, mp);
+    *vp = cell_value_k2_d(w + 2, 1, er, erx, rr, mp);
+    fl |= (uint32_t(rl & 1) << 2) | (uint32_t(rr & 1) << 4);
+    if (eta_out) *eta_out = el;
+    return fl;
+}
+
 // One field at one face, k = 2.  w[0..5] = cells i-2..i+3 around face i+1/2; v^- from cell i
 // (stencil w[1..3]), v^+ from cell i+1 (stencil w[2..4]); tl, tr: transverse second
 // differences of cells i and i+1 (0 on a line).  Flag bits: 0 switch of cell i, 3 switch of
@@ -452,6 +518,32 @@ __device__ __forceinline__ uint32_t face_point_k2(const R* w, const MethodParams
     return fl;
 }
 
+// face_field<double> for k = 3 (see npw_double.cuh): the weights of both cells, the coefficients once
+__device__ __forceinline__ uint32_t face_field_d(const double* w, const MethodParams& mp, double* vm, double* vp,
+                                                 double* eta_out) {
+    uint32_t fl = 0;
+    const double eta = f64::face_eta(w[1], w[2], w[3], w[4], mp, &fl);
+    if (eta_out) *eta_out = eta;
+    double k[6];
+    f64::face_coefs(eta, mp.rbf, k);
+    const double m0 = f64::dot(k[0], w[2], k[1], w[3], k[2], w[4]), m1 = f64::dot(k[2], w[1], k[1], w[2], k[0], w[3]),
+                 m2 = f64::dot(k[3], w[0], k[4], w[1], k[5], w[2]);
+    const double p0 = f64::dot(k[5], w[3], k[4], w[4], k[3], w[5]), p1 = f64::dot(k[0], w[2], k[1], w[3], k[2], w[4]),
+                 p2 = f64::dot(k[2], w[1], k[1], w[2], k[0], w[3]);
+    if (mp.scheme == NPW_ENO_ || mp.scheme == NPW_RBF_ENO_) {
+        const int rl = eno_choice<double>(w[0], w[1], w[2], w[3], w[4]), rr = eno_choice<double>(w[1], w[2], w[3], w[4], w[5]);
+        *vm = rl == 0 ? m0 : (rl == 1 ? m1 : m2);
+        *vp = rr == 0 ? p0 : (rr == 1 ? p1 : p2);
+        return fl | (uint32_t(rl & 3) << 2) | (uint32_t(rr & 3) << 4);
+    }
+    double a[3], b[3], unused[3];
+    f64::cell_weights(w, mp.eps_weno, a, unused);
+    f64::cell_weights(w + 1, mp.eps_weno, unused, b);
+    *vm = (a[0] * m0 + a[1] * m1) + a[2] * m2;
+    *vp = (b[0] * p0 + b[1] * p1) + b[2] * p2;
+    return fl;
+}
+
 // One field at one face.  w[0..5] = cells i-2..i+3 around face i+1/2.  Returns the flag
 // byte (bit0 switch, bits 2-3 / 4-5 ENO r of the left / right cell, bit 6 / 7 the evaluated eta
 // zeroed by the guard / the bound).
@@ -459,6 +551,8 @@ __device__ __forceinline__ uint32_t face_point_k2(const R* w, const MethodParams
 template <typename R, typename D>
 __device__ __forceinline__ uint32_t face_field(const R* w, const MethodParams& mp, R* vm, R* vp, R tl = R(0.0),
                                                R tr = R(0.0), R* eta_out = nullptr) {
+    if constexpr (sizeof(R) == sizeof(double))
+        return mp.k == 2 ? face_field_k2_d(w, mp, vm, vp, tl, tr, eta_out) : face_field_d(w, mp, vm, vp, eta_out);
     if (mp.k == 2) return face_field_k2<R, D>(w, mp, vm, vp, tl, tr, eta_out);
     uint32_t fl = 0;
     R eta = R(0.0);
@@ -581,14 +675,14 @@ __device__ __forceinline__ void phys_flux(const R* U, const MethodParams& mp, in
         F[0] = R(0.5) * U[0] * U[0];
     } else if (KIND == NPW_FLUX_EULER1D_) {
         const R g = mp_val<R>(mp.gamma, mp.gamma_f);
-        R rho = U[0], u = U[1] / rho, E = U[2];
+        R rho = U[0], u = quotient(U[1], rho), E = U[2];
         R P = (g - R(1.0)) * (E - R(0.5) * rho * u * u);
         F[0] = rho * u;
         F[1] = rho * u * u + P;
         F[2] = (E + P) * u;
     } else {
         const R g = mp_val<R>(mp.gamma, mp.gamma_f);
-        R rho = U[0], u = U[1] / rho, v = U[2] / rho, E = U[3];
+        R rho = U[0], u = quotient(U[1], rho), v = quotient(U[2], rho), E = U[3];
         R P = (g - R(1.0)) * (E - R(0.5) * rho * (u * u + v * v));
         R un = (dir == 0) ? u : v;
         F[0] = rho * un;

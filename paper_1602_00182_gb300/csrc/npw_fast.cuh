@@ -19,6 +19,7 @@
 #pragma once
 #include <cstdint>
 
+#include "npw_bits.cuh"
 #include "npw_device.cuh"
 #include "npw_internal.h"
 
@@ -99,14 +100,6 @@ __device__ __forceinline__ float& lane_of(float& a, int) { return a; }
 __device__ __forceinline__ float lane_of(const float& a, int) { return a; }
 __device__ __forceinline__ float& lane_of(F2& a, int i) { return i ? a.v.y : a.v.x; }
 __device__ __forceinline__ float lane_of(const F2& a, int i) { return i ? a.v.y : a.v.x; }
-
-// reciprocal to about one ulp for a normal argument (subnormal results flushed): one instruction,
-// where a quotient only needs to be an estimate
-__device__ __forceinline__ float rcp_fast(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 
 constexpr float kU = 5.9604645e-08f;  // 2^-24, unit roundoff of float
 constexpr float kE = 6.0f * kU;       // bound factor for short small-integer combinations
@@ -328,12 +321,6 @@ __device__ __forceinline__ bool zero_or_normal(float x) {
     return (t == 0u) | (t - 0x00800000u < 0x7F000000u);
 }
 
-// widen for a zero or normal x (the common case): the exponent field is rebiased in place.
-__device__ __forceinline__ double widen_nz(float x) {
-    const uint32_t b = __float_as_uint(x), t = b & 0x7FFFFFFFu;
-    const uint32_t hi = t != 0u ? (t >> 3) + (896u << 20) : 0u;
-    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
-}
 template <bool NZ>
 __device__ __forceinline__ double widen_as(float x) {
     if constexpr (NZ)
@@ -356,16 +343,6 @@ __device__ __forceinline__ float narrow(double v) {
     uint32_t f = (uint32_t)(m >> 29) - (896u << 23);
     f = E < 897u ? 0u : (E > 1150u ? 0x7F800000u : f);
     return __uint_as_float(f | ((uint32_t)(b >> 32) & 0x80000000u));
-}
-
-// seed_f: a binary64 value whose magnitude lies in [2^-99, 2^99) truncated to binary32
-// (relative error below 2^-23), for a reciprocal seed; false outside that range (zero,
-// subnormal, huge, infinite or NaN), where the caller divides in double instead.
-__device__ __forceinline__ bool seed_f(double v, float* out) {
-    const uint64_t b = (uint64_t)__double_as_longlong(v);
-    const uint32_t E = (uint32_t)(b >> 52) & 0x7FFu;
-    *out = __uint_as_float(((uint32_t)(b >> 29) - (896u << 23)) | ((uint32_t)(b >> 32) & 0x80000000u));
-    return E - 924u < 198u;
 }
 
 

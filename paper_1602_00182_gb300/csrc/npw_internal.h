@@ -92,6 +92,7 @@ struct MethodParams {
     // mixed precision, k = 3: constants of the common path of the shape parameter and of the
     // reconstruction (fast::face_eta, fast::cell_recon)
     float pert_f[6];   // perturbation rows 1 (entries 0..2) and 3 (entries 3..5) of the table; 2 and 0 mirror them
+    int has_guard, has_bound;  // eta_guard > 0, eta_max > 0
     int guard_switch;  // 1: switch variant 0, or no switch (a stencil below the guard needs that switch only)
     float sw24_f, sw12_f, sws_f;       // 24, 12 (with a margin) and the weight of the roundings; 0: switch off
     float guard_hi_f;                  // guard threshold with a margin
@@ -304,11 +305,12 @@ cudaError_t launch_tune_init(R* u, int64_t n, int m, cudaStream_t st);
 
 constexpr int TILE_1D = 1024;     // largest automatic tile of the 1D stage kernels (cells per CTA)
 constexpr int TILE_1D_MIN = 256;  // smallest tile params.tile_1d may choose (sizes the tile tables)
-constexpr int TILE_QUEUE_MIN = 63;  // smallest tile of the work queue and the server (sizes their item tables)
+constexpr int TILE_QUEUE_MIN = 60;  // smallest tile of the work queue and the server (sizes their item tables)
 constexpr int NUM_SMS = 152;      // SMs of the GPU this library is written for (automatic tiles)
 constexpr int RES_GHOST = 3;       // ghost cells on each side of the resident kernel's state arrays
 constexpr size_t RESIDENT_SMEM_MAX = 200 * 1024;  // shared memory a resident CTA may use
 constexpr int THREADS_1D = 256;
+constexpr int CHUNK_D = 30;       // cells per warp of the double 1D body (stage1d_double_body)
 constexpr int TX_2D = 32;      // 2D tile
 constexpr int TY_2D = 8;
 constexpr int TX_WARP = 30;    // tile of the warp-task body (stage2d_warp_body)

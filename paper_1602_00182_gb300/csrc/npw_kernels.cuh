@@ -311,16 +311,29 @@ __global__ void __launch_bounds__(THREADS_1D) alpha_init_kernel(const R* __restr
     if (threadIdx.x == 0) atomicMax(&ctl[td.inst].alpha_next_bits, (unsigned long long)__double_as_longlong(b));
 }
 
+// -(h_right - h_left) / dx with one reciprocal of dx
+struct DivDx {
+    double dx, y;
+    bool ok;
+    __device__ __forceinline__ explicit DivDx(double d) : dx(d) { ok = f64::recip(d, &y); }
+    __device__ __forceinline__ double operator()(double hl, double hr) const {
+        const double dh = hr - hl;
+        return -(ok & f64::num_ok(dh) ? f64::quot(dh, dx, y) : f64::div_any(dh, dx));
+    }
+};
+
 // ---------------------------------------------------------------------------------------
 // The fused stage kernel (1D).  Shared memory: su[(tile + 6) * M] cell-major stage input
 // with 3 ghost cells per side, sh[(tile + 1) * M] face fluxes.
 // ---------------------------------------------------------------------------------------
 // One work item (instance td.inst, tile starting at cell td.start) of one stage; the CTA calls
 // it together.  smem: (a.tile + 6 + a.tile + 1) * M elements of R.
-template <typename R, typename D, int KIND, bool CHAR>
+template <typename R, typename D, int KIND, bool CHAR, int K>
 __device__ __forceinline__ void stage1d_body(const Stage1DArgs& a, const Tile td, const InstDev& in, Ctl* ctl,
                                              unsigned char* smem_raw) {
     constexpr int M = kind_m<KIND>();
+    MethodParams mp = a.mp;
+    mp.k = K;  // a constant: the code of the other order is left out
     __shared__ double red[32];
     __shared__ int redbad[32];
     R* su = reinterpret_cast<R*>(smem_raw);
@@ -337,7 +350,7 @@ __device__ __forceinline__ void stage1d_body(const Stage1DArgs& a, const Tile td
     // memory)
 #pragma unroll
     for (int k = 0; k < M; ++k) {
-        const double inflow_k = a.mp.inflow[k];
+        const double inflow_k = mp.inflow[k];
         for (int j = threadIdx.x; j < span; j += blockDim.x)
             su[j * M + k] = line_get<R>(uin + k * n, n, 1, (int64_t)c0 - 3 + j, in.bc, inflow_k);
     }
@@ -351,15 +364,15 @@ __device__ __forceinline__ void stage1d_body(const Stage1DArgs& a, const Tile td
     for (int q = threadIdx.x; q <= cnt; q += blockDim.x) {
         R vm[M], vp[M], h[M];
         uint32_t fl[M];
-        bool ok = face_all<R, D, KIND, M, CHAR>(su + q * M, a.mp, vm, vp, fl);
-        lf_flux<R, KIND, M>(vm, vp, alpha, a.mp, 0, h);
+        bool ok = face_all<R, D, KIND, M, CHAR>(su + q * M, mp, vm, vp, fl);
+        lf_flux<R, KIND, M>(vm, vp, alpha, mp, 0, h);
 #pragma unroll
         for (int k = 0; k < M; ++k) sh[q * M + k] = ok ? h[k] : R(__longlong_as_double(0x7ff8000000000000ll));
         if (face_owned(q, cnt, last_tile))
 #pragma unroll
-            for (int k = 0; k < M; ++k) ec.face(fl[k], a.mp.k);
+            for (int k = 0; k < M; ++k) ec.face(fl[k], mp.k);
     }
-    flush_counts(ec, ctl, a.mp);
+    flush_counts(ec, ctl, mp);
     __syncthreads();
 
     // cells: eq. PDE1 and the Shu-Osher combination
@@ -388,7 +401,7 @@ __device__ __forceinline__ void stage1d_body(const Stage1DArgs& a, const Tile td
             bad |= !finite_(o);
         }
         if (a.stage == 2) {
-            double s = (double)wave_speed<R, KIND>(U, a.mp, 0);
+            double s = (double)wave_speed<R, KIND>(U, mp, 0);
             bad |= !finite_(s);
             vmax = s > vmax ? s : vmax;
         }
@@ -399,6 +412,120 @@ __device__ __forceinline__ void stage1d_body(const Stage1DArgs& a, const Tile td
             atomicMax(&ctl->alpha_next_bits, (unsigned long long)__double_as_longlong(b));
             __threadfence();
             unsigned prev = atomicAdd(&ctl->tiles_done, 1u);
+            if (prev == (unsigned)in.ntiles - 1u) {
+                __threadfence();
+                finalize_1d(ctl, in);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// One stage of one 1D tile in double, k = 3, component-wise, in chunks of CHUNK_D cells per warp: lane l
+// holds cell e = first - 1 + l of the chunk and the face on its right.  It forms the weights of its cell
+// (both sides from one set of indicators; those of the left value go to the lane before, whose
+// face they serve), the shape parameter, the four candidates of its face (rows 1 and 2 serve both values)
+// and the flux; lanes 1..30 update their cells.  The arithmetic and its order are those of
+// face_field<double>, so the results are the same bits.  Bound by the FP64 pipe (see npw_double.cuh):
+// against the face-by-face body the indicators and weights of a cell are formed once instead of
+// once per face.
+// ---------------------------------------------------------------------------------------
+template <int KIND>
+__device__ __forceinline__ void stage1d_double_body(const Stage1DArgs& a, const Tile td, const InstDev& in, Ctl* ctl,
+                                                    unsigned char* smem_raw) {
+    constexpr int M = kind_m<KIND>();
+    __shared__ double red[32];
+    __shared__ int redbad[32];
+    double* su = reinterpret_cast<double*>(smem_raw);  // [cnt + 6][M]
+    if (*(volatile int32_t*)&ctl->done) return;        // uniform over the CTA
+    const int64_t n = in.n;
+    const int c0 = td.start;
+    const int cnt = (int)((n - c0) < a.tile ? (n - c0) : a.tile);
+    const double* uin = reinterpret_cast<const double*>(a.uin) + in.off;
+    const int span = cnt + 6;
+    for (int j = threadIdx.x; j < span; j += blockDim.x) {
+        const int64_t g = halo_idx(n, (int64_t)c0 - 3 + j, in.bc);
+#pragma unroll
+        for (int k = 0; k < M; ++k) su[j * M + k] = g < 0 ? a.mp.inflow[k] : uin[k * n + g];
+    }
+    const double dt = *(volatile double*)&ctl->dt, alpha = *(volatile double*)&ctl->alpha, dx = in.dx;
+    __syncthreads();
+    EtaCount ec;
+    const bool last_tile = c0 + cnt == n;
+    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    const bool weno = a.mp.scheme == NPW_WENO_JS_ || a.mp.scheme == NPW_RBF_WENO_;
+    double ydx;
+    const bool dx_ok = f64::recip(dx, &ydx);
+    double* uout = reinterpret_cast<double*>(a.uout) + in.off;
+    const double* un = reinterpret_cast<const double*>(a.un) + in.off;
+    double vmax = 0.0;
+    bool bad = false;
+#pragma unroll 1
+    for (int first = (threadIdx.x >> 5) * CHUNK_D; first < cnt; first += nwarps * CHUNK_D) {
+        const int q = first + lane;       // local face on the right of cell q - 1
+        const int e = min(q - 1, cnt);    // local cell (past the tile: its last neighbour)
+        const bool own = (lane < CHUNK_D || q == cnt) && face_owned(q, cnt, last_tile);
+        double vm[M], vp[M], h[M];
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            double c[6];
+#pragma unroll
+            for (int j = 0; j < 6; ++j) c[j] = su[min(e + 1 + j, span - 1) * M + k];
+            uint32_t fl = 0;
+            const double eta = f64::face_eta(c[1], c[2], c[3], c[4], a.mp, &fl);
+            if (own) ec.face_k3(fl);
+            double kc[6];
+            f64::face_coefs(eta, a.mp.rbf, kc);
+            const double r0 = f64::dot(kc[5], c[3], kc[4], c[4], kc[3], c[5]), r1 = f64::dot(kc[0], c[2], kc[1], c[3], kc[2], c[4]),
+                         r2 = f64::dot(kc[2], c[1], kc[1], c[2], kc[0], c[3]), r3 = f64::dot(kc[3], c[0], kc[4], c[1], kc[5], c[2]);
+            if (weno) {
+                double wm[3], wp[3];
+                f64::cell_weights(c, a.mp.eps_weno, wm, wp);
+#pragma unroll
+                for (int r = 0; r < 3; ++r) wp[r] = __shfl_down_sync(0xffffffffu, wp[r], 1);
+                vm[k] = (wm[0] * r1 + wm[1] * r2) + wm[2] * r3;
+                vp[k] = (wp[0] * r0 + wp[1] * r1) + wp[2] * r2;
+            } else {
+                const int rl = eno_choice<double>(c[0], c[1], c[2], c[3], c[4]);
+                const int rr = __shfl_down_sync(0xffffffffu, rl, 1);
+                vm[k] = rl == 0 ? r1 : (rl == 1 ? r2 : r3);
+                vp[k] = rr == 0 ? r0 : (rr == 1 ? r1 : r2);
+            }
+        }
+        lf_flux<double, KIND, M>(vm, vp, alpha, a.mp, 0, h);
+        double U[M];
+        const bool cell = lane >= 1 && lane <= CHUNK_D && q - 1 < cnt;
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const double hl = __shfl_up_sync(0xffffffffu, h[k], 1);
+            if (cell) {
+                const double dh = h[k] - hl;
+                const double L = -(dx_ok & f64::num_ok(dh) ? f64::quot(dh, dx, ydx) : f64::div_any(dh, dx));
+                const double uk = su[(q + 2) * M + k];
+                const int64_t ix = k * n + c0 + q - 1;
+                double o = uk + dt * L;
+                if (a.stage == 1)
+                    o = fma(0.25, o, 0.75 * un[ix]);
+                else if (a.stage == 2)
+                    o = stage3_w1<double>() * un[ix] + stage3_w2<double>() * o;
+                uout[ix] = o;
+                U[k] = o;
+                bad |= !finite_(o);
+            }
+        }
+        if (cell && a.stage == 2) {
+            const double s = wave_speed<double, KIND>(U, a.mp, 0);
+            bad |= !finite_(s);
+            vmax = s > vmax ? s : vmax;
+        }
+    }
+    flush_counts(ec, ctl, a.mp);
+    if (a.stage == 2 && a.advance) {
+        const double b = block_max_nan(vmax, bad, red, redbad);
+        if (threadIdx.x == 0) {
+            atomicMax(&ctl->alpha_next_bits, (unsigned long long)__double_as_longlong(b));
+            __threadfence();
+            const unsigned prev = atomicAdd(&ctl->tiles_done, 1u);
             if (prev == (unsigned)in.ntiles - 1u) {
                 __threadfence();
                 finalize_1d(ctl, in);
@@ -1777,10 +1904,13 @@ __device__ __forceinline__ void gauss_face(const R* S, const R* su, int BX, int 
     for (int k = 0; k < M; ++k) h[k] = R(0.5) * (h1[k] + h[k]);
 }
 
-template <typename R, typename D, int KIND>
+template <typename R, typename D, int KIND, int K>
 __device__ __forceinline__ void stage2d_body(const Stage2DArgs& a, const Inst2D& in, Ctl* ctl, int tile,
                                              unsigned char* smem_raw) {
     constexpr int M = kind_m<KIND>();
+    // the order as a constant: the code (and the registers) of the other one is left out
+    MethodParams mp = a.mp;
+    mp.k = K;
     constexpr int BX = TX_2D + 6, BY = TY_2D + 6;
     R* su = reinterpret_cast<R*>(smem_raw);   // [BY * BX * M]
     R* hx = su + BY * BX * M;                 // [TY * (TX + 1) * M]
@@ -1795,12 +1925,12 @@ __device__ __forceinline__ void stage2d_body(const Stage2DArgs& a, const Inst2D&
     const int64_t nx = in.nx, ny = in.ny, cells = nx * ny;
     const R* uin = reinterpret_cast<const R*>(a.uin) + in.off;
     const int tid = threadIdx.x;
-    const bool gauss = a.mp.k == 2 && a.mp.gauss_2d;
-    const bool cross = gauss || (a.mp.k == 2 && a.mp.cross_2d &&
-                                 (a.mp.scheme == NPW_RBF_ENO_ || a.mp.scheme == NPW_RBF_WENO_));
+    const bool gauss = mp.k == 2 && mp.gauss_2d;
+    const bool cross = gauss || (mp.k == 2 && mp.cross_2d &&
+                                 (mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_));
 #pragma unroll
     for (int k = 0; k < M; ++k) {
-        const double inflow_k = a.mp.inflow[k];
+        const double inflow_k = mp.inflow[k];
         for (int rem = tid; rem < BX * BY; rem += blockDim.x) {
             const int by = rem / BX, bx = rem - by * BX;
             // the corners are read only by the 5-cell cross of k = 2 (transverse differences of
@@ -1833,7 +1963,7 @@ __device__ __forceinline__ void stage2d_body(const Stage2DArgs& a, const Inst2D&
             // mean of the two Lax-Friedrichs fluxes; transverse data of the cells qx-1 (v^-) and qx
             // (v^+) from rows qy-1..qy+1, each with the other as the cell across the face
             R h1[M];
-            gauss_face<R, D, KIND, M>(S, su, BX, qx + 2, qy + 3, 1, BX, ax, a.mp, 0, h, h1, ec,
+            gauss_face<R, D, KIND, M>(S, su, BX, qx + 2, qy + 3, 1, BX, ax, mp, 0, h, h1, ec,
                                       qy < cnt_y && face_owned(qx, cnt_x, last_x));
 #pragma unroll
             for (int k = 0; k < M; ++k) hx[(qy * (TX_2D + 1) + qx) * M + k] = h[k];
@@ -1847,19 +1977,19 @@ __device__ __forceinline__ void stage2d_body(const Stage2DArgs& a, const Inst2D&
 #pragma unroll
                 for (int k = 0; k < M; ++k) {
                     const int bx = qx + 2 + c;
-                    T[c * M + k] = (D(su[((qy + 2) * BX + bx) * M + k]) - D(2.0) * D(su[((qy + 3) * BX + bx) * M + k])) +
-                                   D(su[((qy + 4) * BX + bx) * M + k]);
+                    T[c * M + k] = fma(D(-2.0), D(su[((qy + 3) * BX + bx) * M + k]), D(su[((qy + 2) * BX + bx) * M + k])) +
+                                   D(su[((qy + 4) * BX + bx) * M + k]);  // (2 u is exact)
                 }
-            face_all<R, D, KIND, M, false>(S, a.mp, vm, vp, fl, T);
+            face_all<R, D, KIND, M, false>(S, mp, vm, vp, fl, T);
         } else {
-            face_all<R, D, KIND, M, false>(S, a.mp, vm, vp, fl);
+            face_all<R, D, KIND, M, false>(S, mp, vm, vp, fl);
         }
-        lf_flux<R, KIND, M>(vm, vp, ax, a.mp, 0, h);
+        lf_flux<R, KIND, M>(vm, vp, ax, mp, 0, h);
 #pragma unroll
         for (int k = 0; k < M; ++k) hx[(qy * (TX_2D + 1) + qx) * M + k] = h[k];
         if (qy < cnt_y && face_owned(qx, cnt_x, last_x))
 #pragma unroll
-            for (int k = 0; k < M; ++k) ec.face(fl[k], a.mp.k);
+            for (int k = 0; k < M; ++k) ec.face(fl[k], mp.k);
     }
     // y faces: (qx, qy), qx = 0..TX-1, qy = 0..TY, stencil su[qy .. qy+5][qx+3]
     for (int f = tid; f < TX_2D * (TY_2D + 1); f += blockDim.x) {
@@ -1872,7 +2002,7 @@ __device__ __forceinline__ void stage2d_body(const Stage2DArgs& a, const Inst2D&
             for (int k = 0; k < M; ++k) S[j * M + k] = su[((qy + j) * BX + qx + 3) * M + k];
         if (gauss) {
             R h1[M];
-            gauss_face<R, D, KIND, M>(S, su, BX, qx + 3, qy + 2, BX, 1, ay, a.mp, 1, h, h1, ec,
+            gauss_face<R, D, KIND, M>(S, su, BX, qx + 3, qy + 2, BX, 1, ay, mp, 1, h, h1, ec,
                                       qx < cnt_x && face_owned(qy, cnt_y, last_y));
 #pragma unroll
             for (int k = 0; k < M; ++k) hy[(qy * TX_2D + qx) * M + k] = h[k];
@@ -1886,21 +2016,21 @@ __device__ __forceinline__ void stage2d_body(const Stage2DArgs& a, const Inst2D&
 #pragma unroll
                 for (int k = 0; k < M; ++k) {
                     const int by = qy + 2 + c;
-                    T[c * M + k] = (D(su[(by * BX + qx + 2) * M + k]) - D(2.0) * D(su[(by * BX + qx + 3) * M + k])) +
+                    T[c * M + k] = fma(D(-2.0), D(su[(by * BX + qx + 3) * M + k]), D(su[(by * BX + qx + 2) * M + k])) +
                                    D(su[(by * BX + qx + 4) * M + k]);
                 }
-            face_all<R, D, KIND, M, false>(S, a.mp, vm, vp, fl, T);
+            face_all<R, D, KIND, M, false>(S, mp, vm, vp, fl, T);
         } else {
-            face_all<R, D, KIND, M, false>(S, a.mp, vm, vp, fl);
+            face_all<R, D, KIND, M, false>(S, mp, vm, vp, fl);
         }
-        lf_flux<R, KIND, M>(vm, vp, ay, a.mp, 1, h);
+        lf_flux<R, KIND, M>(vm, vp, ay, mp, 1, h);
 #pragma unroll
         for (int k = 0; k < M; ++k) hy[(qy * TX_2D + qx) * M + k] = h[k];
         if (qx < cnt_x && face_owned(qy, cnt_y, last_y))
 #pragma unroll
-            for (int k = 0; k < M; ++k) ec.face(fl[k], a.mp.k);
+            for (int k = 0; k < M; ++k) ec.face(fl[k], mp.k);
     }
-    flush_counts(ec, ctl, a.mp);
+    flush_counts(ec, ctl, mp);
     __syncthreads();
     R* uout = reinterpret_cast<R*>(a.uout) + in.off;
     const R* un = reinterpret_cast<const R*>(a.un) + in.off;
@@ -1914,8 +2044,13 @@ __device__ __forceinline__ void stage2d_body(const Stage2DArgs& a, const Inst2D&
             R U[M];
 #pragma unroll
             for (int k = 0; k < M; ++k) {
-                R L = -((hx[(qy * (TX_2D + 1) + qx + 1) * M + k] - hx[(qy * (TX_2D + 1) + qx) * M + k]) / dxR);
-                L = L - (hy[((qy + 1) * TX_2D + qx) * M + k] - hy[(qy * TX_2D + qx) * M + k]) / dyR;
+                const R hl = hx[(qy * (TX_2D + 1) + qx) * M + k], hr = hx[(qy * (TX_2D + 1) + qx + 1) * M + k];
+                const R hd = hy[(qy * TX_2D + qx) * M + k], hu = hy[((qy + 1) * TX_2D + qx) * M + k];
+                R L;
+                if constexpr (sizeof(R) == sizeof(double))
+                    L = DivDx(dxR)(hl, hr) + DivDx(dyR)(hd, hu);
+                else
+                    L = -((hr - hl) / dxR) - (hu - hd) / dyR;
                 const R uk = su[((qy + 3) * BX + qx + 3) * M + k];
                 const int64_t gidx = k * cells + gj * nx + gi;
                 R o;
@@ -1931,8 +2066,8 @@ __device__ __forceinline__ void stage2d_body(const Stage2DArgs& a, const Inst2D&
                 bad |= !finite_(o);
             }
             if (a.stage == 2) {
-                double sx = (double)wave_speed<R, KIND>(U, a.mp, 0);
-                double sy = (double)wave_speed<R, KIND>(U, a.mp, 1);
+                double sx = (double)wave_speed<R, KIND>(U, mp, 0);
+                double sy = (double)wave_speed<R, KIND>(U, mp, 1);
                 bad |= !finite_(sx) || !finite_(sy);
                 vmx = sx;
                 vmy = sy;
@@ -1995,11 +2130,18 @@ __global__ void __launch_bounds__(TX_2D * TY_2D) alpha_init_2d_kernel(const R* _
 // One CTA per work item: the per-stage kernels of the 1D runtime (tile table) and of a single
 // 2D instance (blockIdx.x = tile index).
 // ---------------------------------------------------------------------------------------
-template <typename R, typename D, int KIND, bool CHAR>
+template <typename R, typename D, int KIND, bool CHAR, int K>
 __global__ void __launch_bounds__(THREADS_1D) stage1d_kernel(Stage1DArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const Tile td = tile_at(a.tiles, a.tile);
-    stage1d_body<R, D, KIND, CHAR>(a, td, a.inst[td.inst], a.ctl + td.inst, smem_raw);
+    stage1d_body<R, D, KIND, CHAR, K>(a, td, a.inst[td.inst], a.ctl + td.inst, smem_raw);
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(THREADS_1D) stage1d_double_kernel(Stage1DArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const Tile td = tile_at(a.tiles, a.tile);
+    stage1d_double_body<KIND>(a, td, a.inst[td.inst], a.ctl + td.inst, smem_raw);
 }
 
 template <int KIND, int K>
@@ -2021,10 +2163,10 @@ __global__ void __launch_bounds__(THREADS_1D, 4) stage2d_warp_kernel(Stage2DArgs
     stage2d_warp_body<KIND>(a, *a.inst, a.ctl, blockIdx.x, smem_f);
 }
 
-template <typename R, typename D, int KIND>
+template <typename R, typename D, int KIND, int K>
 __global__ void __launch_bounds__(TX_2D * TY_2D) stage2d_kernel(Stage2DArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    stage2d_body<R, D, KIND>(a, *a.inst, a.ctl, blockIdx.x, smem_raw);
+    stage2d_body<R, D, KIND, K>(a, *a.inst, a.ctl, blockIdx.x, smem_raw);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -2047,8 +2189,10 @@ __device__ __forceinline__ void queue_item_1d(const Stage1DArgs& a1, const Tile 
                 step1d_fused_body<KIND>(a1, w, in, ctl, smem);
         } else
             stage1d_fast_body<KIND, K>(a1, w, in, ctl, smem);
-    } else
-        stage1d_body<R, double, KIND, CHAR && KIND == NPW_FLUX_EULER1D_>(a1, w, in, ctl, smem);
+    } else if constexpr (sizeof(R) == sizeof(double) && !CHAR && K == 3)
+        stage1d_double_body<KIND>(a1, w, in, ctl, smem);
+    else
+        stage1d_body<R, double, KIND, CHAR && KIND == NPW_FLUX_EULER1D_, K>(a1, w, in, ctl, smem);
 }
 template <typename R, int K, int KIND>
 __device__ __forceinline__ void queue_item_2d(const Stage2DArgs& a2, const Inst2D& in, Ctl* ctl, int tile,
@@ -2058,7 +2202,7 @@ __device__ __forceinline__ void queue_item_2d(const Stage2DArgs& a2, const Inst2
     else if constexpr (sizeof(R) == sizeof(float))
         stage2d_fast_body<KIND, K>(a2, in, ctl, tile, reinterpret_cast<float*>(smem));
     else
-        stage2d_body<R, double, KIND>(a2, in, ctl, tile, smem);
+        stage2d_body<R, double, KIND, K>(a2, in, ctl, tile, smem);
 }
 
 // CTAs per SM the register allocation aims for: 4 for the specialised mixed-precision k = 3 kernels
@@ -2306,16 +2450,34 @@ struct Launchers {
 
     template <int KIND, bool CHAR>
     static cudaError_t stage_k(const Stage1DArgs& a, cudaStream_t s) {
+        return a.mp.k == 2 ? stage_kk<KIND, CHAR, 2>(a, s) : stage_kk<KIND, CHAR, 3>(a, s);
+    }
+    template <int KIND, bool CHAR, int K>
+    static cudaError_t stage_kk(const Stage1DArgs& a, cudaStream_t s) {
         constexpr int M = kind_m<KIND>();
-        const size_t smem = (size_t)((a.tile + 6) + (a.tile + 1)) * M * sizeof(R);
-        auto kern = stage1d_kernel<R, D, KIND, CHAR>;
-        static bool attr_set = false;
-        if (!attr_set) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-            if (e != cudaSuccess) return e;
-            attr_set = true;
+        if constexpr (sizeof(R) == sizeof(double) && !CHAR && K == 3) {
+            auto kern = stage1d_double_kernel<KIND>;
+            static bool attr_set = false;
+            if (!attr_set) {
+                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+                if (e != cudaSuccess) return e;
+                attr_set = true;
+            }
+            const int chunks = (a.tile + CHUNK_D - 1) / CHUNK_D;
+            kern<<<a.ntiles, cta_threads(chunks * 32), (size_t)(a.tile + 6) * M * sizeof(R), s>>>(a);
+        } else if constexpr (sizeof(R) == sizeof(double) || CHAR) {
+            const size_t smem = (size_t)((a.tile + 6) + (a.tile + 1)) * M * sizeof(R);
+            auto kern = stage1d_kernel<R, D, KIND, CHAR, K>;
+            static bool attr_set = false;
+            if (!attr_set) {
+                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+                if (e != cudaSuccess) return e;
+                attr_set = true;
+            }
+            kern<<<a.ntiles, cta_threads(a.tile + 1), smem, s>>>(a);
+        } else {
+            return cudaErrorInvalidValue;  // float, component-wise: stage_fast
         }
-        kern<<<a.ntiles, cta_threads(a.tile + 1), smem, s>>>(a);
         return cudaGetLastError();
     }
 
@@ -2389,13 +2551,13 @@ struct Launchers {
                 // float cell averages, candidates, weights, flux and update in float
                 switch (kind) {
                     case NPW_FLUX_ADVECTION:
-                        stage2d_kernel<float, double, NPW_FLUX_ADVECTION_><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<1>() * sizeof(float), s>>>(a);
+                        stage2d_kernel<float, double, NPW_FLUX_ADVECTION_, 2><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<1>() * sizeof(float), s>>>(a);
                         break;
                     case NPW_FLUX_BURGERS:
-                        stage2d_kernel<float, double, NPW_FLUX_BURGERS_><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<1>() * sizeof(float), s>>>(a);
+                        stage2d_kernel<float, double, NPW_FLUX_BURGERS_, 2><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<1>() * sizeof(float), s>>>(a);
                         break;
                     case NPW_FLUX_EULER2D:
-                        stage2d_kernel<float, double, NPW_FLUX_EULER2D_><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<4>() * sizeof(float), s>>>(a);
+                        stage2d_kernel<float, double, NPW_FLUX_EULER2D_, 2><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<4>() * sizeof(float), s>>>(a);
                         break;
                     default:
                         return cudaErrorInvalidValue;
@@ -2436,15 +2598,20 @@ struct Launchers {
             }
             return cudaGetLastError();
         }
+        return a.mp.k == 2 ? stage2d_plain<2>(a, tiles, kind, s) : stage2d_plain<3>(a, tiles, kind, s);
+    }
+
+    template <int K>
+    static cudaError_t stage2d_plain(const Stage2DArgs& a, int tiles, int kind, cudaStream_t s) {
         switch (kind) {
             case NPW_FLUX_ADVECTION:
-                stage2d_kernel<R, D, NPW_FLUX_ADVECTION_><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<1>() * sizeof(R), s>>>(a);
+                stage2d_kernel<R, D, NPW_FLUX_ADVECTION_, K><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<1>() * sizeof(R), s>>>(a);
                 break;
             case NPW_FLUX_BURGERS:
-                stage2d_kernel<R, D, NPW_FLUX_BURGERS_><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<1>() * sizeof(R), s>>>(a);
+                stage2d_kernel<R, D, NPW_FLUX_BURGERS_, K><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<1>() * sizeof(R), s>>>(a);
                 break;
             case NPW_FLUX_EULER2D:
-                stage2d_kernel<R, D, NPW_FLUX_EULER2D_><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<4>() * sizeof(R), s>>>(a);
+                stage2d_kernel<R, D, NPW_FLUX_EULER2D_, K><<<tiles, TX_2D * TY_2D, stage2d_smem_elems<4>() * sizeof(R), s>>>(a);
                 break;
             default:
                 return cudaErrorInvalidValue;
