@@ -1102,6 +1102,29 @@ static npw_status single_run(void* u, int64_t n, int32_t m, double dx, double t_
     return NPW_OK;
 }
 
+}  // extern "C"
+namespace {
+int cluster_ctas(const npw_params* p, int64_t n, int m);
+// the run of r by one cluster of ctas CTAs: a solve of `in`, or (single_step) one step of dt
+npw_status cluster_run(const Run1D& r, const npw_instance& in, int ctas, int single_step, double dt, bool* fits) {
+    npw::ResidentArgs a{};
+    a.arena = r.arena;
+    a.carry = reinterpret_cast<float*>(r.ws + r.L.cbuf);
+    a.ctl = reinterpret_cast<npw::Ctl*>(r.ws + r.L.ctl);
+    a.count = 1;
+    a.mp = r.mp;
+    a.one = npw::InstDev{0, in.n, in.dx, in.t_end, in.cfl, in.bc, 0};
+    a.dt_fixed = dt;
+    a.single_step = single_step;
+    auto ev = stage_begin(r.s);
+    const cudaError_t e = r.fp32 ? npw::launch_cluster<float>(a, r.kind, in.n, ctas, r.s, fits)
+                                 : npw::launch_cluster<double>(a, r.kind, in.n, ctas, r.s, fits);
+    stage_end(ev, r.s);
+    return e == cudaSuccess ? NPW_OK : cuda_fail(e, "cluster launch");
+}
+}  // namespace
+extern "C" {
+
 npw_status npweno_rk3_step(void* u, int64_t n, int32_t m, double dx, double dt, int32_t flux_kind, int32_t bc,
                            const npw_params* params, void* workspace, size_t workspace_bytes, double* alpha_out,
                            void* stream) {
@@ -1111,9 +1134,15 @@ npw_status npweno_rk3_step(void* u, int64_t n, int32_t m, double dx, double dt, 
     npw_status st = single_run(u, n, m, dx, 0.0, 0.0, flux_kind, bc, params, workspace, workspace_bytes, s, r, in);
     if (st) return st;
     if (!(dt >= 0.0)) return fail(NPW_EINVAL, "dt must be >= 0");
-    if ((st = setup_1d(r, &in, 1, dt, 2))) return st;
-    if ((st = step_kernels(r, 0))) return st;
-    if ((st = comp_end(r))) return st;
+    bool whole = false;
+    if (const int ctas = cluster_ctas(params, n, m)) {
+        if ((st = cluster_run(r, in, ctas, 1, dt, &whole))) return st;
+    }
+    if (!whole) {
+        if ((st = setup_1d(r, &in, 1, dt, 2))) return st;
+        if ((st = step_kernels(r, 0))) return st;
+        if ((st = comp_end(r))) return st;
+    }
     if (alpha_out) {
         npw::Ctl c;
         if ((st = bounded_sync(s))) return st;
@@ -1124,6 +1153,26 @@ npw_status npweno_rk3_step(void* u, int64_t n, int32_t m, double dx, double dt, 
     return NPW_OK;
 }
 
+// CTAs of the cluster that solves one line whole (solve1d_cluster_kernel), 0: the per-stage kernels.  One
+// slice per CTA of at least 8 cells; 16 CTAs leave 9/10 of the SMs idle, so the line may not be longer
+// than what they work off in the time that the launches of a stage take: float CLUSTER_F32 cells and
+// fields together, double CLUSTER_F64 (an FP64 stage costs tens of float ones).  Against the per-stage
+// launches: FP64 advection N = 200, 100 steps 3.8 -> 2.5 ms and one step 51 -> 35 us (two launches for
+// eight), mixed Burgers N = 5613, 150 steps 2.5 -> 1.26 ms.  A stage of 200 FP64 cells is 8 us of
+// dependent FP64 instructions (about 90 cycles each), whatever the number of SMs.
+}  // extern "C"
+namespace {
+constexpr int64_t CLUSTER_F32 = 40000, CLUSTER_F64 = 1500;
+int cluster_ctas(const npw_params* p, int64_t n, int m) {
+    if (p->k != 3 || p->characteristic) return 0;
+    if (n * m > (p->precision == NPW_FP32_MIXED ? CLUSTER_F32 : CLUSTER_F64)) return 0;
+    int c = (int)(n / 8 < 16 ? n / 8 : 16);
+    while (c > 1 && n - (c - 1) * ((n + c - 1) / c) < npw::RES_GHOST) --c;  // the last slice holds a halo
+    return c < 1 ? 1 : c;
+}
+}  // namespace
+extern "C" {
+
 npw_status npweno_solve(void* u, int64_t n, int32_t m, double dx, double t_end, double cfl, int32_t flux_kind,
                         int32_t bc, const npw_params* params, void* workspace, size_t workspace_bytes,
                         npw_solve_stats* out, void* stream) {
@@ -1133,6 +1182,11 @@ npw_status npweno_solve(void* u, int64_t n, int32_t m, double dx, double t_end, 
     npw_status st = single_run(u, n, m, dx, t_end, cfl, flux_kind, bc, params, workspace, workspace_bytes, s, r, in);
     if (st) return st;
     if (!(cfl > 0.0)) return fail(NPW_EINVAL, "cfl must be > 0");
+    if (const int ctas = cluster_ctas(params, n, m)) {
+        bool fits = false;
+        if ((st = cluster_run(r, in, ctas, 0, 0.0, &fits))) return st;
+        if (fits) return collect_stats(r, out);
+    }
     if ((st = setup_1d(r, &in, 1, 0.0, 1))) return st;
     return run_to_end(r, out);
 }

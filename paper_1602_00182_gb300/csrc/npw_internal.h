@@ -200,6 +200,10 @@ struct ResidentArgs {
     const int32_t* list;     // instance indices handled by this launch, one per CTA
     int32_t count;
     MethodParams mp;
+    // solve1d_cluster_kernel: its one line, and a single step of dt_fixed instead of a solve
+    InstDev one;
+    double dt_fixed;
+    int32_t single_step;
 };
 
 struct Stage2DArgs {
@@ -281,6 +285,10 @@ template <typename R>
 cudaError_t launch_queue_alpha(const QueueArgs& q, cudaStream_t s);
 template <typename R>
 size_t queue_smem_bytes(int tile, bool has1d, int m1d, bool has2d, int m2d, bool characteristic, int k);
+// whole solve of one line by one cluster of `ctas` CTAs; *fits = false (nothing launched) where such a
+// cluster does not fit the GPU
+template <typename R>
+cudaError_t launch_cluster(const ResidentArgs& a, int kind, int64_t n, int ctas, cudaStream_t s, bool* fits);
 // resident whole-solve launch (float state only); max_n = largest n in the list
 cudaError_t launch_resident_f32(const ResidentArgs& a, int m, int kind, int64_t max_n, int threads, cudaStream_t s);
 size_t resident_smem_bytes(int64_t n, int m);

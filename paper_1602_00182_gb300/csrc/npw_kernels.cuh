@@ -7,9 +7,11 @@
 // the flux difference of eq. PDE1 and the Shu-Osher stage combination -- and, in stage 3,
 // the block reduction of the next Lax-Friedrichs alpha and the per-instance time control.
 #pragma once
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <mutex>
 #include <type_traits>
 
 #include "npw_device.cuh"
@@ -421,15 +423,59 @@ __device__ __forceinline__ void stage1d_body(const Stage1DArgs& a, const Tile td
 }
 
 // ---------------------------------------------------------------------------------------
-// One stage of one 1D tile in double, k = 3, component-wise, in chunks of CHUNK_D cells per warp: lane l
-// holds cell e = first - 1 + l of the chunk and the face on its right.  It forms the weights of its cell
-// (both sides from one set of indicators; those of the left value go to the lane before, whose
-// face they serve), the shape parameter, the four candidates of its face (rows 1 and 2 serve both values)
-// and the flux; lanes 1..30 update their cells.  The arithmetic and its order are those of
-// face_field<double>, so the results are the same bits.  Bound by the FP64 pipe (see npw_double.cuh):
-// against the face-by-face body the indicators and weights of a cell are formed once instead of
-// once per face.
+// One chunk of CHUNK_D cells of a line of cnt cells in double, k = 3, component-wise, by one warp: lane l
+// holds cell first - 1 + l and the face on its right.  It forms the weights of its cell (both sides
+// from one set of indicators; those of the left value go to the lane before, whose face they serve),
+// the shape parameter, the four candidates of its face (rows 1 and 2 serve both values) and the flux;
+// lanes 1..30 update their cells, upd(j, flux of face j, flux of face j + 1).  X(k, i): the stage input,
+// i in -3..cnt + 2; last: the line's last face is counted here.  The arithmetic and its order are those
+// of face_field<double>, so the results are the same bits.  Bound by the FP64 pipe (see
+// npw_double.cuh): against the face-by-face body the indicators and weights of a cell are formed once
+// instead of once per face.
 // ---------------------------------------------------------------------------------------
+template <int KIND, typename LoadX, typename Upd>
+__device__ __forceinline__ void warp_chunk_d(int first, int cnt, bool last, int lane, const MethodParams& mp, double alpha,
+                                             LoadX X, Upd upd, EtaCount& ec) {
+    constexpr int M = kind_m<KIND>();
+    const bool weno = mp.scheme == NPW_WENO_JS_ || mp.scheme == NPW_RBF_WENO_;
+    const int q = first + lane;     // face on the right of cell q - 1
+    const int e = min(q - 1, cnt);  // (past the line: its last neighbour)
+    const bool own = (lane < CHUNK_D || q == cnt) && face_owned(q, cnt, last);
+    double vm[M], vp[M], h[M], hl[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        double c[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) c[j] = X(k, min(e - 2 + j, cnt + 2));
+        uint32_t fl = 0;
+        const double eta = f64::face_eta(c[1], c[2], c[3], c[4], mp, &fl);
+        if (own) ec.face_k3(fl);
+        double kc[6];
+        f64::face_coefs(eta, mp.rbf, kc);
+        const double r0 = f64::dot(kc[5], c[3], kc[4], c[4], kc[3], c[5]), r1 = f64::dot(kc[0], c[2], kc[1], c[3], kc[2], c[4]),
+                     r2 = f64::dot(kc[2], c[1], kc[1], c[2], kc[0], c[3]), r3 = f64::dot(kc[3], c[0], kc[4], c[1], kc[5], c[2]);
+        if (weno) {
+            double wm[3], wp[3];
+            f64::cell_weights(c, mp.eps_weno, wm, wp);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) wp[r] = __shfl_down_sync(0xffffffffu, wp[r], 1);
+            vm[k] = (wm[0] * r1 + wm[1] * r2) + wm[2] * r3;
+            vp[k] = (wp[0] * r0 + wp[1] * r1) + wp[2] * r2;
+        } else {
+            const int rl = eno_choice<double>(c[0], c[1], c[2], c[3], c[4]);
+            const int rr = __shfl_down_sync(0xffffffffu, rl, 1);
+            vm[k] = rl == 0 ? r1 : (rl == 1 ? r2 : r3);
+            vp[k] = rr == 0 ? r0 : (rr == 1 ? r1 : r2);
+        }
+    }
+    lf_flux<double, KIND, M>(vm, vp, alpha, mp, 0, h);
+#pragma unroll
+    for (int k = 0; k < M; ++k) hl[k] = __shfl_up_sync(0xffffffffu, h[k], 1);
+    if (lane >= 1 && lane <= CHUNK_D && q - 1 < cnt) upd(q - 1, hl, h);
+}
+
+// One stage of one 1D tile in double, k = 3, component-wise: the tile's cells in shared memory, a chunk
+// per warp.
 template <int KIND>
 __device__ __forceinline__ void stage1d_double_body(const Stage1DArgs& a, const Tile td, const InstDev& in, Ctl* ctl,
                                                     unsigned char* smem_raw) {
@@ -453,72 +499,36 @@ __device__ __forceinline__ void stage1d_double_body(const Stage1DArgs& a, const 
     EtaCount ec;
     const bool last_tile = c0 + cnt == n;
     const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    const bool weno = a.mp.scheme == NPW_WENO_JS_ || a.mp.scheme == NPW_RBF_WENO_;
-    double ydx;
-    const bool dx_ok = f64::recip(dx, &ydx);
+    const DivDx dxq(dx);
     double* uout = reinterpret_cast<double*>(a.uout) + in.off;
     const double* un = reinterpret_cast<const double*>(a.un) + in.off;
     double vmax = 0.0;
     bool bad = false;
-#pragma unroll 1
-    for (int first = (threadIdx.x >> 5) * CHUNK_D; first < cnt; first += nwarps * CHUNK_D) {
-        const int q = first + lane;       // local face on the right of cell q - 1
-        const int e = min(q - 1, cnt);    // local cell (past the tile: its last neighbour)
-        const bool own = (lane < CHUNK_D || q == cnt) && face_owned(q, cnt, last_tile);
-        double vm[M], vp[M], h[M];
-#pragma unroll
-        for (int k = 0; k < M; ++k) {
-            double c[6];
-#pragma unroll
-            for (int j = 0; j < 6; ++j) c[j] = su[min(e + 1 + j, span - 1) * M + k];
-            uint32_t fl = 0;
-            const double eta = f64::face_eta(c[1], c[2], c[3], c[4], a.mp, &fl);
-            if (own) ec.face_k3(fl);
-            double kc[6];
-            f64::face_coefs(eta, a.mp.rbf, kc);
-            const double r0 = f64::dot(kc[5], c[3], kc[4], c[4], kc[3], c[5]), r1 = f64::dot(kc[0], c[2], kc[1], c[3], kc[2], c[4]),
-                         r2 = f64::dot(kc[2], c[1], kc[1], c[2], kc[0], c[3]), r3 = f64::dot(kc[3], c[0], kc[4], c[1], kc[5], c[2]);
-            if (weno) {
-                double wm[3], wp[3];
-                f64::cell_weights(c, a.mp.eps_weno, wm, wp);
-#pragma unroll
-                for (int r = 0; r < 3; ++r) wp[r] = __shfl_down_sync(0xffffffffu, wp[r], 1);
-                vm[k] = (wm[0] * r1 + wm[1] * r2) + wm[2] * r3;
-                vp[k] = (wp[0] * r0 + wp[1] * r1) + wp[2] * r2;
-            } else {
-                const int rl = eno_choice<double>(c[0], c[1], c[2], c[3], c[4]);
-                const int rr = __shfl_down_sync(0xffffffffu, rl, 1);
-                vm[k] = rl == 0 ? r1 : (rl == 1 ? r2 : r3);
-                vp[k] = rr == 0 ? r0 : (rr == 1 ? r1 : r2);
-            }
-        }
-        lf_flux<double, KIND, M>(vm, vp, alpha, a.mp, 0, h);
+    auto X = [&](int k, int i) { return su[(i + 3) * M + k]; };
+    auto upd = [&](int j, const double* hl, const double* hr) {
         double U[M];
-        const bool cell = lane >= 1 && lane <= CHUNK_D && q - 1 < cnt;
 #pragma unroll
         for (int k = 0; k < M; ++k) {
-            const double hl = __shfl_up_sync(0xffffffffu, h[k], 1);
-            if (cell) {
-                const double dh = h[k] - hl;
-                const double L = -(dx_ok & f64::num_ok(dh) ? f64::quot(dh, dx, ydx) : f64::div_any(dh, dx));
-                const double uk = su[(q + 2) * M + k];
-                const int64_t ix = k * n + c0 + q - 1;
-                double o = uk + dt * L;
-                if (a.stage == 1)
-                    o = fma(0.25, o, 0.75 * un[ix]);
-                else if (a.stage == 2)
-                    o = stage3_w1<double>() * un[ix] + stage3_w2<double>() * o;
-                uout[ix] = o;
-                U[k] = o;
-                bad |= !finite_(o);
-            }
+            const double uk = X(k, j);
+            const int64_t ix = k * n + c0 + j;
+            double o = uk + dt * dxq(hl[k], hr[k]);
+            if (a.stage == 1)
+                o = fma(0.25, o, 0.75 * un[ix]);
+            else if (a.stage == 2)
+                o = stage3_w1<double>() * un[ix] + stage3_w2<double>() * o;
+            uout[ix] = o;
+            U[k] = o;
+            bad |= !finite_(o);
         }
-        if (cell && a.stage == 2) {
+        if (a.stage == 2) {
             const double s = wave_speed<double, KIND>(U, a.mp, 0);
             bad |= !finite_(s);
             vmax = s > vmax ? s : vmax;
         }
-    }
+    };
+#pragma unroll 1
+    for (int first = (threadIdx.x >> 5) * CHUNK_D; first < cnt; first += nwarps * CHUNK_D)
+        warp_chunk_d<KIND>(first, cnt, last_tile, lane, a.mp, alpha, X, upd, ec);
     flush_counts(ec, ctl, a.mp);
     if (a.stage == 2 && a.advance) {
         const double b = block_max_nan(vmax, bad, red, redbad);
@@ -598,8 +608,8 @@ __device__ __forceinline__ void warp_line_pass(int lo, int hi, int n, int lane, 
 // ---------------------------------------------------------------------------------------
 constexpr int BLOCK_CELLS = 62;
 template <int KIND, int M, typename LoadX, typename Upd>
-__device__ __forceinline__ void warp_block_pass(int b0, int n, int lane, const fast::FParams& fp, const MethodParams& mp,
-                                                float alpha, LoadX X, Upd upd, EtaCount& ec) {
+__device__ __forceinline__ void warp_block_pass(int b0, int n, bool last, int lane, const fast::FParams& fp,
+                                                const MethodParams& mp, float alpha, LoadX X, Upd upd, EtaCount& ec) {
     using fast::F2;
     auto before = [lane](F2 v) {  // the position before (p = 0 gets its own value)
         const float xe = __shfl_sync(0xffffffffu, v.v.x, 31);
@@ -617,10 +627,10 @@ __device__ __forceinline__ void warp_block_pass(int b0, int n, int lane, const f
         for (int q = 0; q < 5; ++q) c[q] = F2{make_float2(X(k, ix - 2 + q), X(k, iy - 2 + q))};
         const F2 w[1][4] = {{c[1], c[2], c[3], c[4]}};
         fast::face_eta_n<F2, 1>(w, fp, eta, fl);
-        // face b0 + p, counted by this block for p < 62, and face n wherever it falls
-        if (b0 + lane <= n) ec.face_k3(fl[0][0]);
+        // face b0 + p, counted by this block for p < 62, and face n wherever it falls if `last`
+        if (face_owned(b0 + lane, n, last)) ec.face_k3(fl[0][0]);
         const int f = b0 + 32 + lane;
-        if (f <= n && (lane < 30 || (lane == 30 && f == n))) ec.face_k3(fl[0][1]);
+        if ((lane < 30 || f == n) && face_owned(f, n, last)) ec.face_k3(fl[0][1]);
         fast::cell_recon<F2>(c, eta[0], before(eta[0]), fp, &vm, &vp);
         const F2 vl = before(vm);
         ax[k] = vl.v.x;
@@ -1325,7 +1335,7 @@ __global__ void __launch_bounds__(K == 3 ? 512 : 1024) solve1d_resident_kernel(R
                 if constexpr (K == 3) {
 #pragma unroll 1
                     for (int b0 = warp * BLOCK_CELLS; b0 < n; b0 += nwarps * BLOCK_CELLS)
-                        warp_block_pass<KIND, M>(b0, n, lane, fp, a.mp, alphaf, X, upd, ec);
+                        warp_block_pass<KIND, M>(b0, n, true, lane, fp, a.mp, alphaf, X, upd, ec);
                 } else {
                     warp_line_pass<KIND, M>(lo, hi, n, lane, fp, a.mp, alphaf, X, upd, ec);
                 }
@@ -1378,6 +1388,342 @@ __global__ void __launch_bounds__(K == 3 ? 512 : 1024) solve1d_resident_kernel(R
         ctl->steps = steps;
         ctl->status = status;
         ctl->done = 1;
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// Whole solve of one line by one thread-block cluster, k = 3, component-wise, either state type: the line
+// is cut into one slice per CTA, whose stage arrays live in that CTA's shared memory with RES_GHOST ghost
+// cells on each side.  A boundary cell is stored into the neighbour's ghost cells as well, through
+// distributed shared memory, and one cluster barrier ends each stage.  In the last stage every CTA
+// also stores its largest wave speed into a slot of every other, so that each advances t, alpha and dt
+// by itself to the same values.  Float: the increment form of the resident kernel (un, d1 / new state,
+// d2; carry in global memory); double: the Shu-Osher form of the per-stage kernel (un, u1, u2).  The
+// arithmetic per cell is theirs, so the results are the same bits.
+// For a single instance this replaces three launches per step, each with too few cells to fill the
+// GPU, by three barriers of a microsecond or less; it uses 16 SMs, so long lines stay with the
+// per-stage kernels (see cluster_ctas).
+// ---------------------------------------------------------------------------------------
+constexpr int MAX_CLUSTER = 16;
+template <typename R, int KIND>
+__global__ void __launch_bounds__(512) solve1d_cluster_kernel(ResidentArgs a) {
+    namespace cg = cooperative_groups;
+    constexpr int M = kind_m<KIND>();
+    constexpr bool F32 = sizeof(R) == sizeof(float);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red_d[32];
+    __shared__ float red_f[32];
+    __shared__ int redbad[32];
+    __shared__ double s_slot[MAX_CLUSTER];  // wave speeds of the slices
+    __shared__ double s_alpha, s_dt;
+    __shared__ float s_lam;
+    __shared__ int s_done;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const InstDev in = a.one;
+    Ctl* ctl = a.ctl;
+    const int n = (int)in.n, per = (n + C - 1) / C;
+    const int s0 = rank * per, cnt = min(per, n - s0);  // every slice has at least RES_GHOST cells (cluster_ctas)
+    const bool periodic = in.bc == NPW_BC_PERIODIC, last_slice = rank == C - 1;
+    const int NS = per + 2 * RES_GHOST;
+    R* const base = reinterpret_cast<R*>(smem_raw);
+    R* un = base;             // [M][NS]
+    R* uA = un + M * NS;      // float: d1, then the new state; double: u1
+    R* uB = uA + M * NS;      // float: d2; double: u2
+    // neighbours' arrays and the places of their ghost cells (periodic ends meet)
+    const int rl = rank > 0 ? rank - 1 : C - 1, rr = last_slice ? 0 : rank + 1;
+    R* const left = cluster.map_shared_rank(base, rl);
+    R* const right = cluster.map_shared_rank(base, rr);
+    const int cnt_l = min(per, n - rl * per);
+    const bool to_left = rank > 0 || periodic, to_right = !last_slice || periodic;
+    R inflow[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) inflow[k] = mp_val<R>(a.mp.inflow[k], a.mp.inflow_f[k]);
+    // cell i of field k of the array at p, with the ghost cells that copy it
+    auto store = [&](R* p, int k, int i, R v, R inflow_ghost) {
+        const int at = (int)(p - base) + k * NS + RES_GHOST;
+        base[at + i] = v;
+        if (i < RES_GHOST) {
+            if (to_left) left[at + cnt_l + i] = v;
+            if (i == 0 && !to_left) {
+                const R g = in.bc == NPW_BC_INFLOW ? inflow_ghost : v;
+#pragma unroll
+                for (int j = 1; j <= RES_GHOST; ++j) base[at - j] = g;
+            }
+        }
+        if (i >= cnt - RES_GHOST) {
+            if (to_right) right[at + i - cnt] = v;
+            if (i == cnt - 1 && !to_right) {
+#pragma unroll
+                for (int j = 0; j < RES_GHOST; ++j) base[at + cnt + j] = v;
+            }
+        }
+    };
+    R* g = reinterpret_cast<R*>(a.arena) + in.off;
+    float* cr = F32 ? a.carry + in.off : nullptr;
+    for (int i = (int)threadIdx.x - RES_GHOST; i < cnt + RES_GHOST; i += blockDim.x) {
+        const int c = res_map(s0 + i, n, in.bc);
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            un[k * NS + RES_GHOST + i] = c < 0 ? inflow[k] : g[(int64_t)k * n + c];
+            if (F32 && i >= 0 && i < cnt) cr[(int64_t)k * n + s0 + i] = 0.0f;
+        }
+    }
+    const fast::FParams fp = fast::fparams(a.mp);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    EtaCount ec;
+    R vmax = R(0.0);
+    bool bad = false;
+    __syncthreads();
+    for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+        R U[M];
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            U[k] = un[k * NS + RES_GHOST + i];
+            bad |= !finite_(U[k]);
+        }
+        const R sp = wave_speed<R, KIND>(U, a.mp, 0);
+        bad |= !finite_(sp);
+        vmax = sp > vmax ? sp : vmax;
+    }
+    // the largest wave speed of the line in thread 0 of every CTA (NaN: not finite)
+    auto line_max = [&]() {
+        double b;
+        if constexpr (F32)
+            b = block_max_nan_f(vmax, bad, red_f, redbad);
+        else
+            b = block_max_nan(vmax, bad, red_d, redbad);
+        if (threadIdx.x == 0)
+            for (int r = 0; r < C; ++r) *cluster.map_shared_rank(s_slot + rank, r) = b;
+        cluster.sync();
+        double m = 0.0;
+        if (threadIdx.x == 0) {
+            bool nan = false;
+            for (int r = 0; r < C; ++r) {
+                const double v = s_slot[r];
+                nan |= !(v - v == 0.0);
+                m = v > m ? v : m;
+            }
+            if (nan) m = __longlong_as_double(0x7ff8000000000000ll);
+        }
+        return m;
+    };
+    double t = 0.0, dt = 0.0, alpha = 0.0, alpha_max = 0.0;  // thread 0's copies
+    int64_t steps = 0, cap = 0;
+    int last = 0, status = 0;
+    auto next_step = [&](double b) {  // thread 0: dt of the next step
+        const double rate = b / in.dx;
+        dt = (rate > 0.0) ? in.cfl / rate : in.t_end - t;
+        if (t + dt * (1.0 + 1e-10) >= in.t_end) {
+            dt = in.t_end - t;
+            last = 1;
+        }
+        s_lam = (float)(dt / in.dx);
+        s_alpha = alpha;
+        s_dt = dt;
+    };
+    if (rank == 0 && threadIdx.x == 0) memset(ctl, 0, sizeof(Ctl));
+    cluster.sync();  // every CTA of the cluster has started: its shared memory may be written
+    {
+        const double b = line_max();
+        if (threadIdx.x == 0) {
+            s_done = 0;
+            if (!(b - b == 0.0)) {
+                status = NPW_ENONFINITE;
+                s_done = 1;
+            } else {
+                alpha = alpha_max = b;
+                if (a.single_step) {
+                    dt = a.dt_fixed;
+                    s_lam = (float)(dt / in.dx);
+                    s_alpha = alpha;
+                    s_dt = dt;
+                } else {
+                    s_done = !(t < in.t_end);
+                    next_step(b);
+                    cap = step_cap(in.t_end - t, dt, a.mp.max_steps);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    const DivDx dxq(F32 ? 1.0 : in.dx);
+    while (!s_done) {
+        const float lam = s_lam;
+        const R alphaR = R(s_alpha), dtR = R(s_dt);
+        vmax = R(0.0);
+        bad = false;
+#pragma unroll 1
+        for (int stage = 0; stage < 3; ++stage) {
+            const R* D = stage == 1 ? uA : uB;
+            auto upd_speed = [&](const R* U) {
+                const R sp = wave_speed<R, KIND>(U, a.mp, 0);
+                bad |= !finite_(sp);
+                vmax = sp > vmax ? sp : vmax;
+            };
+            if constexpr (F32) {
+                auto X = [&](int k, int i) {
+                    const int ix = k * NS + RES_GHOST + i;
+                    return stage == 0 ? un[ix] : un[ix] + D[ix];
+                };
+                auto upd = [&](int j, const float* hl, const float* hr) {
+                    float U[M];
+#pragma unroll
+                    for (int k = 0; k < M; ++k) {
+                        const float du = lam * (hl[k] - hr[k]);
+                        const int ix = k * NS + RES_GHOST + j;
+                        if (stage == 0) {
+                            store(uA, k, j, du, -0.0f);
+                            U[k] = du;
+                        } else if (stage == 1) {
+                            const float v = 0.25f * (uA[ix] + du);
+                            store(uB, k, j, v, -0.0f);
+                            U[k] = v;
+                        } else {
+                            const int64_t gx = (int64_t)k * n + s0 + j;
+                            const float base_u = un[ix];
+                            const float y = kTwoThirdsF * (uB[ix] + du) + cr[gx];
+                            const float tn = base_u + y;
+                            cr[gx] = y - (tn - base_u);
+                            store(uA, k, j, tn, inflow[k]);
+                            U[k] = tn;
+                        }
+                        bad |= !finite_(U[k]);
+                    }
+                    if (stage == 2) upd_speed(U);
+                };
+#pragma unroll 1
+                for (int b0 = warp * BLOCK_CELLS; b0 < cnt; b0 += nwarps * BLOCK_CELLS)
+                    warp_block_pass<KIND, M>(b0, cnt, last_slice, lane, fp, a.mp, alphaR, X, upd, ec);
+            } else {
+                const R* in_ = stage == 0 ? un : D;
+                R* out_ = stage == 0 ? uA : (stage == 1 ? uB : un);
+                auto X = [&](int k, int i) { return in_[k * NS + RES_GHOST + i]; };
+                auto upd = [&](int j, const double* hl, const double* hr) {
+                    double U[M];
+#pragma unroll
+                    for (int k = 0; k < M; ++k) {
+                        const int ix = k * NS + RES_GHOST + j;
+                        double o = in_[ix] + dtR * dxq(hl[k], hr[k]);
+                        if (stage == 1)
+                            o = fma(0.25, o, 0.75 * un[ix]);
+                        else if (stage == 2)
+                            o = stage3_w1<double>() * un[ix] + stage3_w2<double>() * o;
+                        store(out_, k, j, o, inflow[k]);
+                        U[k] = o;
+                        bad |= !finite_(o);
+                    }
+                    if (stage == 2) upd_speed(U);
+                };
+#pragma unroll 1
+                for (int first = warp * CHUNK_D; first < cnt; first += nwarps * CHUNK_D)
+                    warp_chunk_d<KIND>(first, cnt, last_slice, lane, a.mp, alphaR, X, upd, ec);
+            }
+            if (stage < 2) cluster.sync();
+        }
+        if constexpr (F32) {  // the new state (in uA) becomes u^n
+            R* tmp = un;
+            un = uA;
+            uA = tmp;
+        }
+        if (a.single_step) {
+            cluster.sync();  // no CTA leaves while a neighbour stores into its ghost cells
+            break;
+        }
+        const double b = line_max();  // (its cluster barrier ends the stage)
+        if (threadIdx.x == 0) {
+            steps += 1;
+            t = last ? in.t_end : t + dt;
+            if (!(b - b == 0.0)) {
+                status = NPW_ENONFINITE;
+                s_done = 1;
+            } else {
+                alpha = b;
+                alpha_max = b > alpha_max ? b : alpha_max;
+                if (last) {
+                    s_done = 1;
+                } else {
+                    next_step(b);
+                    if (steps >= cap || !(t + dt > t)) {  // step limit, or time stopped advancing
+                        status = NPW_ETIMEOUT;
+                        s_done = 1;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < cnt; i += blockDim.x)
+#pragma unroll
+        for (int k = 0; k < M; ++k) g[(int64_t)k * n + s0 + i] = un[k * NS + RES_GHOST + i];
+    flush_counts(ec, ctl, a.mp);
+    if (rank == 0 && threadIdx.x == 0) {
+        ctl->t = t;
+        ctl->dt = dt;
+        ctl->alpha = alpha;
+        ctl->alpha_max = alpha_max;
+        ctl->steps = steps;
+        ctl->status = status;
+        ctl->done = 1;
+    }
+}
+
+// bytes of shared memory of a slice of `per` cells
+template <typename R>
+constexpr size_t cluster_smem(int64_t per, int m) {
+    return (size_t)m * 3 * (size_t)(per + 2 * RES_GHOST) * sizeof(R);
+}
+template <typename R, int KIND>
+cudaError_t launch_cluster_k(const ResidentArgs& a, int64_t n, int ctas, cudaStream_t s, bool* fits) {
+    auto kern = solve1d_cluster_kernel<R, KIND>;
+    const int64_t per = (n + ctas - 1) / ctas;
+    const int unit = sizeof(R) == sizeof(float) ? BLOCK_CELLS : CHUNK_D;
+    const int warps = (int)((per + unit - 1) / unit);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)(warps > 16 ? 512 : warps * 32));
+    cfg.dynamicSmemBytes = cluster_smem<R>(per, kind_m<KIND>());
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    // the attributes, and whether the largest slice's cluster of this size fits, once per device
+    static std::mutex mu;
+    static signed char known[64][MAX_CLUSTER + 1];  // 0 not asked, 1 fits, -1 does not
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || ctas > MAX_CLUSTER) return cudaErrorInvalidValue;
+    {
+        std::lock_guard<std::mutex> g(mu);
+        signed char& k = known[dev][ctas];
+        if (k == 0) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RESIDENT_SMEM_MAX);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            int clusters = 0;
+            cudaLaunchConfig_t most = cfg;
+            most.blockDim = dim3(512);
+            most.dynamicSmemBytes = RESIDENT_SMEM_MAX;
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kern, &most);
+            if (e != cudaSuccess) return e;
+            k = clusters > 0 ? 1 : -1;
+        }
+        *fits = k > 0;
+    }
+    return *fits ? cudaLaunchKernelEx(&cfg, kern, a) : cudaSuccess;
+}
+template <typename R>
+cudaError_t launch_cluster_r(const ResidentArgs& a, int kind, int64_t n, int ctas, cudaStream_t s, bool* fits) {
+    *fits = false;
+    if (cluster_smem<R>((n + ctas - 1) / ctas, kind == NPW_FLUX_EULER1D ? 3 : 1) > RESIDENT_SMEM_MAX) return cudaSuccess;
+    switch (kind) {
+        case NPW_FLUX_ADVECTION: return launch_cluster_k<R, NPW_FLUX_ADVECTION_>(a, n, ctas, s, fits);
+        case NPW_FLUX_BURGERS: return launch_cluster_k<R, NPW_FLUX_BURGERS_>(a, n, ctas, s, fits);
+        case NPW_FLUX_EULER1D: return launch_cluster_k<R, NPW_FLUX_EULER1D_>(a, n, ctas, s, fits);
+        default: return cudaErrorInvalidValue;
     }
 }
 
