@@ -163,7 +163,8 @@ __device__ __forceinline__ int switch_v0_cert(float d0, float d1, float d2) {
         const float eG = 2.f * (aA * eC + aC * eA + 3.f * eA * eC) + 3.f * (2.f * aB * eB + 3.f * eB * eB) +
                          kE * (2.f * aA * aC + 3.f * aB * aB);
         const int sG = csign(G, eG);
-        if (sG == kUncertain) return -1;
+        // (below 2^-120 the products may have underflowed, G and its bound to 0 alike)
+        if (sG == kUncertain || !(eG > 0x1p-120f)) return -1;
         const int sV = sG * sA;
         neg = neg || sV < 0;
         pos = pos || sV > 0;
