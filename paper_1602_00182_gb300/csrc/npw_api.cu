@@ -125,6 +125,7 @@ npw::MethodParams method(const npw_params* p) {
     const float ga_rows[6] = {float(2.0 / 3.0), float(-1.0 / 3.0), float(-1.0 / 3.0), 0.0f, 3.0f, -3.0f};
     const float mq_rows[6] = {float(5.0 / 6.0), float(-2.0 / 3.0), float(-1.0 / 6.0), -1.5f, 6.0f, -4.5f};
     for (int k = 0; k < 6; ++k) mp.pert_f[k] = ga ? ga_rows[k] : mq_rows[k];
+    mp.tie_tol_f = (float)mp.tie_tol;
     mp.has_guard = mp.eta_guard > 0.0;
     mp.has_bound = mp.eta_max > 0.0;
     const float margin = 1.0f + 0x1p-16f;

@@ -628,11 +628,9 @@ __device__ __forceinline__ bool switch_v0_near(const double* w, double tol) {
     }
     return near;
 }
-template <typename R>
-__device__ __forceinline__ bool face_near_tie(const R* wr, const MethodParams& mp, double tol) {
-    double w[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) w[j] = (double)wr[j];
+static __device__ __noinline__ bool face_near_tie_d(double w1, double w2, double w3, double w4, const MethodParams& mp,
+                                                    double tol) {
+    const double w[6] = {0.0, w1, w2, w3, w4, 0.0};  // (both orders use cells i-1..i+2)
     const bool rbf = mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_;
     bool near = false;
     if (mp.k == 2) {
@@ -662,6 +660,62 @@ __device__ __forceinline__ bool face_near_tie(const R* wr, const MethodParams& m
             near = near || tie_rel(fabs(eta_num<double>(w[1], w[2], w[3], w[4]) / (den0 + mp.eps_M)), mp.eta_max, tol);
     }
     return near;
+}
+
+// Certainly no near tie at a k = 3 face (switch variant 0), in float: every quantity compared by
+// face_near_tie lies further from its threshold than tol and the bounds here together.  A, B, C of
+// switch_v0_cert from the neighbour differences truncated or rounded to float, e bounds their errors (as
+// in fast::switch_level2, f64::switch_v0; a sixty-fourth of that of E = 24 A + C).  Nearly every face
+// passes; the rest takes the FP64 expressions, some 60 FP64-pipe instructions, which bounded
+// npweno_reconstruct before.
+__device__ __forceinline__ bool far_from_ties(float d0, float d1, float d2, float a1, float a2, float unit, float abs_err,
+                                              const MethodParams& mp, float tol) {
+    const float t02 = d0 + d2, s = fabsf(d0) + fabsf(d2);
+    const float A = fmaf(-2.f, d1, t02), B = d2 - d0, C = fmaf(14.f, d1, -t02);
+    const float aA = fabsf(A), aB = fabsf(B), aC = fabsf(C);
+    const float e = fmaf(unit, s + aC, abs_err * (a1 + a2));
+    const float mag = 2.f * (a1 + a2) + s;  // at least |w0| + .. + |w3|
+    if (!((s < 0x1p50f) & (aC < 0x1p50f) & (s + aC > 0x1p-40f))) return false;
+    bool far_ = true;
+    if (mp.monotone_switch) {
+        const float lim = 100.f * tol * mag, E = fmaf(24.f, A, C), aE = fabsf(E), eE = fmaf(64.f, e, lim), b12 = 12.f * aB;
+        far_ = fabsf(b12 - aE) > eE + 0x1p-20f * (b12 + aE);  // both ends
+        const float a4 = 4.f * aA;
+        const bool inside = aB < a4 * (1.f - 0x1p-10f) - 8.f * e, outside = aB > fmaf(a4, 1.f + 0x1p-10f, 8.f * e);
+        const float G = fmaf(2.f * A, C, -3.f * B * B);
+        far_ = far_ & (outside | (inside & (fabsf(G) > fmaf(40.f * e, aA + aB + aC + e, 2.5f * aA * lim))));
+    }
+    if (mp.has_guard) {
+        const float g = mp.eta_guard_f * (fabsf(a1) * 16.f + fabsf(a2) * 16.f);  // (the magnitudes, within s + ...)
+        const float gm = mp.eta_guard_f * s;
+        far_ = far_ & ((aC > g * 1.01f + 2.f * gm + 64.f * e) | (aC < g * 0.85f - 2.f * gm - 64.f * e));
+    }
+    if (mp.has_bound) {
+        const float x = mp.eta_max_f * aC, m = fmaf(mp.eta_max_f, fabsf(mp.eps_M_f) + 64.f * e, 64.f * e);
+        far_ = far_ & (fabsf(aA - x) > 0x1p-10f * (aA + x) + m);
+    }
+    return far_;
+}
+
+template <typename R>
+__device__ __forceinline__ bool face_near_tie(const R* wr, const MethodParams& mp, double tol) {
+    if (mp.k == 3 && (mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_) && mp.guard_switch && mp.tie_tol_f <= 0x1p-14f) {
+        // a constant stencil: monotone, its denominator and eta exactly 0 against positive thresholds
+        if (wr[1] == wr[2] && wr[2] == wr[3] && wr[3] == wr[4]) return false;
+        bool ok = true;
+        if constexpr (sizeof(R) == sizeof(float))
+            ok = far_from_ties(wr[2] - wr[1], wr[3] - wr[2], wr[4] - wr[3], fabsf(wr[2]), fabsf(wr[3]), 0x1p-19f, 0.0f, mp,
+                               mp.tie_tol_f);
+        else {
+            const float d0 = f64::to_f(wr[2] - wr[1], &ok), d1 = f64::to_f(wr[3] - wr[2], &ok),
+                        d2 = f64::to_f(wr[4] - wr[3], &ok), a1 = fabsf(f64::to_f(wr[2], &ok)),
+                        a2 = fabsf(f64::to_f(wr[3], &ok));
+            ok = ok && far_from_ties(d0, d1, d2, a1, a2, 0x1p-18f, 0x1p-40f, mp, mp.tie_tol_f);
+        }
+        if (ok) return false;
+    }
+    if (mp.scheme != NPW_RBF_ENO_ && mp.scheme != NPW_RBF_WENO_) return false;
+    return face_near_tie_d((double)wr[1], (double)wr[2], (double)wr[3], (double)wr[4], mp, tol);
 }
 
 // ---------------------------------------------------------------------------------------

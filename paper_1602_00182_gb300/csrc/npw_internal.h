@@ -92,6 +92,7 @@ struct MethodParams {
     // mixed precision, k = 3: constants of the common path of the shape parameter and of the
     // reconstruction (fast::face_eta, fast::cell_recon)
     float pert_f[6];   // perturbation rows 1 (entries 0..2) and 3 (entries 3..5) of the table; 2 and 0 mirror them
+    float tie_tol_f;   // tie_tol
     int has_guard, has_bound;  // eta_guard > 0, eta_max > 0
     int guard_switch;  // 1: switch variant 0, or no switch (a stencil below the guard needs that switch only)
     float sw24_f, sw12_f, sws_f;       // 24, 12 (with a margin) and the weight of the roundings; 0: switch off

@@ -217,7 +217,8 @@ __device__ __forceinline__ void finalize_2d(Ctl* c, const Inst2D& in) {
 // fields), and eta (optional) the shape parameters as used.
 // ---------------------------------------------------------------------------------------
 template <typename R, typename D, int M, bool CHAR>
-__global__ void reconstruct_kernel(const R* __restrict__ u, int64_t n, int bc, MethodParams mp, R* __restrict__ vm,
+__global__ void reconstruct_kernel(const R* __restrict__ u, int64_t n, int bc, const __grid_constant__ MethodParams mp,
+                                   R* __restrict__ vm,
                                    R* __restrict__ vp, uint8_t* __restrict__ flags, R* __restrict__ eta) {
     int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (f > n) return;
