@@ -849,8 +849,8 @@ __device__ __forceinline__ int eno2_choice_f(float c0, float c1, float c2) {
 
 // value of cell i (c[0..2] = cells i-1..i+1) at its right (side 0) or left (side 1) face;
 // eta_c for the central row, eta_x for the extrapolating ones
-__device__ __forceinline__ float cell_value_k2_f(const float* c, int side, float eta_c, float eta_x, const FParams& fp,
-                                                 int* r_out) {
+__device__ __forceinline__ float cell_value_k2_f(const float* c, int side, float eta_c, float eta_x, int r,
+                                                 const FParams& fp) {
     float cand[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
@@ -860,13 +860,8 @@ __device__ __forceinline__ float cell_value_k2_f(const float* c, int side, float
         const float k1 = fmaf(pert2_coef<float>(fp.rbf, row + 1, 1), eta, poly2_coef<float>(row + 1, 1));
         cand[r] = fmaf(k0, c[1 - r], k1 * c[2 - r]);
     }
-    if (fp.scheme == NPW_ENO_ || fp.scheme == NPW_RBF_ENO_) {
-        const int r = eno2_choice_f(c[0], c[1], c[2]);
-        *r_out = r;
-        return r == 0 ? cand[0] : cand[1];
-    }
-    *r_out = 0;
-    constexpr float kBeMax = 1e18f;  // keeps the fast division in range (see cell_recon)
+    if (fp.scheme == NPW_ENO_ || fp.scheme == NPW_RBF_ENO_) return r == 0 ? cand[0] : cand[1];
+    constexpr float kBeMax = 1e18f;  // keeps the fast division in range
     const float g0 = c[2] - c[1], g1 = c[1] - c[0];
     const float be0 = fminf(fmaf(g0, g0, fp.eps_weno), kBeMax), be1 = fminf(fmaf(g1, g1, fp.eps_weno), kBeMax);
     const float a0 = __fdividef(side == 0 ? 2.f / 3.f : 1.f / 3.f, be0 * be0);
@@ -892,45 +887,63 @@ __device__ __forceinline__ float cell_value_k2_f(const float* c, int side, float
 //   * The factor 2 of the multiquadric row is applied to the rounded float value (exact).
 // FP64-pipe instructions per face value: 5 for numerator and denominator, 1 for e and 2 per
 // quotient (on the cross, 2 more for the two numerators and 2 for the second quotient).
+//   * need: bit 0 the central, bit 1 the extrapolating one is used (an ENO value takes one of them).  The
+//     other differs from it by 3/8 trans / den; it is formed only where that might pass the bound,
+//     since its flag counts.
 template <bool NZ>
-__device__ __forceinline__ void eta_k2_quot(float af, float bf, float df, double trans, const FParams& fp, float* ec,
-                                            float* ex, uint32_t* fl) {
+__device__ __forceinline__ void eta_k2_quot(float af, float bf, float df, double trans, int need, const FParams& fp,
+                                            float* ec, float* ex, uint32_t* fl) {
     const double a = widen_as<NZ>(af), b = widen_as<NZ>(bf), d = widen_as<NZ>(df);
     const double base = fma(2.0, b, -(a + d));
     const double den = fma(5.0, b, fma(2.0, d, -a)) + fp.eps_M;
-    float denf, vc, vx;
+    const float bound = fp.eta_max;
+    if (trans == 0.0) need = 1;
+    float denf, vc = 0.0f, vx = 0.0f;
     if (seed_f(den, &denf)) {
-        const double r0 = widen_nz(__fdividef(1.0f, denf));
+        const float rf = __fdividef(1.0f, denf);
+        const double r0 = widen_nz(rf);
         const double e = fma(-den, r0, 1.0);
-        const double nc = trans == 0.0 ? base : fma(-0.25, trans, base);
-        const double qc = nc * r0;
-        vc = narrow(fma(qc, e, qc));
-        if (trans == 0.0) {
-            vx = vc;
-        } else {
-            const double qx = fma(0.125, trans, base) * r0;
-            vx = narrow(fma(qx, e, qx));
+        auto value = [&](double num) {
+            const double q = num * r0;
+            return narrow(fma(q, e, q));
+        };
+        if (need & 1) vc = value(trans == 0.0 ? base : fma(-0.25, trans, base));
+        if (need & 2) vx = value(fma(0.125, trans, base));
+        if (bound > 0.0f && need != 3 && trans != 0.0) {
+            const float span = 0.376f * fabsf(narrow(trans) * rf) * (fp.rbf == NPW_RBF_GA_ ? 1.0f : 2.0f);
+            const float have = fabsf((need & 1) ? vc : vx) * (fp.rbf == NPW_RBF_GA_ ? 1.0f : 2.0f);
+            if (!((have + span) * (1.0f + 0x1p-10f) < bound)) {
+                if (need & 1)
+                    vx = value(fma(0.125, trans, base));
+                else
+                    vc = value(fma(-0.25, trans, base));
+            }
         }
     } else {
         vc = div_rn_f(fma(-0.25, trans, base), den);
         vx = trans == 0.0 ? vc : div_rn_f(fma(0.125, trans, base), den);
     }
+    if (trans == 0.0) vx = vc;
     if (fp.rbf != NPW_RBF_GA_) {
         vc *= 2.0f;
         vx *= 2.0f;
     }
-    const float bound = fp.eta_max;
     const bool zc = bound > 0.0f && fabsf(vc) > bound, zx = bound > 0.0f && fabsf(vx) > bound;
     *ec = zc ? 0.0f : vc;
     *ex = zx ? 0.0f : vx;
     if (zc | zx) *fl |= FL_ZERO_BOUND;
 }
-static __device__ __noinline__ void eta_k2_quot_any(float af, float bf, float df, double trans, const FParams& fp,
-                                                    float* ec, float* ex, uint32_t* fl) {
-    eta_k2_quot<false>(af, bf, df, trans, fp, ec, ex, fl);
+// (out of line: by value what it reads)
+static __device__ __noinline__ void eta_k2_quot_any(float af, float bf, float df, double trans, double eps_M, float eta_max,
+                                                    int rbf, float* ec, float* ex, uint32_t* fl) {
+    FParams fp;
+    fp.eps_M = eps_M;
+    fp.eta_max = eta_max;
+    fp.rbf = rbf;
+    eta_k2_quot<false>(af, bf, df, trans, 3, fp, ec, ex, fl);
 }
 // fl: FL_ZERO_GUARD / FL_ZERO_BOUND where the guard / the bound set a shape parameter to 0
-__device__ __forceinline__ void eta_k2_pair(const float* cf, int side, double trans, const MethodParams& mp,
+__device__ __forceinline__ void eta_k2_pair(const float* cf, int side, double trans, int need, const MethodParams& mp,
                                             const FParams& fp, float* ec, float* ex, uint32_t* fl) {
     const float af = side == 0 ? cf[0] : cf[2], bf = cf[1], df = side == 0 ? cf[2] : cf[0];
     *ec = *ex = 0.0f;
@@ -951,10 +964,13 @@ __device__ __forceinline__ void eta_k2_pair(const float* cf, int side, double tr
         }
     }
     if (zero_or_normal(af) & zero_or_normal(bf) & zero_or_normal(df))
-        eta_k2_quot<true>(af, bf, df, trans, fp, ec, ex, fl);
+        eta_k2_quot<true>(af, bf, df, trans, need, fp, ec, ex, fl);
     else
-        eta_k2_quot_any(af, bf, df, trans, fp, ec, ex, fl);
+        eta_k2_quot_any(af, bf, df, trans, fp.eps_M, fp.eta_max, fp.rbf, ec, ex, fl);
 }
+// the shape parameters of a k = 2 face value that are used (bit 0 central, bit 1 extrapolating): an ENO
+// value with stencil r takes row r on the right face, r - 1 on the left one
+__device__ __forceinline__ int k2_need(bool eno, int side, int r) { return eno ? (r == side ? 1 : 2) : 3; }
 
 // Decisions of a k = 2 cell, as returned by cell_recon_k2: FL_SWITCH (the cell's switch fired:
 // both its shape parameters are 0), FL_ZERO_GUARD / FL_ZERO_BOUND for the side-0 (v^-) value and
@@ -969,18 +985,19 @@ __device__ __forceinline__ uint32_t cell_recon_k2(const float* c3, double trans,
                                                   const FParams& fp, float* vm, float* vp) {
     float e0c = 0.0f, e0x = 0.0f, e1c = 0.0f, e1x = 0.0f;
     uint32_t d = 0, f0 = 0, f1 = 0;
+    const bool eno = fp.scheme == NPW_ENO_ || fp.scheme == NPW_RBF_ENO_;
+    const int r = eno ? eno2_choice_f(c3[0], c3[1], c3[2]) : 0;
     if (fp.scheme == NPW_RBF_ENO_ || fp.scheme == NPW_RBF_WENO_) {
         if (fp.monotone_switch && switch_k2_f(c3[0], c3[1], c3[2])) {
             d = FL_SWITCH;
         } else {
-            eta_k2_pair(c3, 0, trans, mp0, fp, &e0c, &e0x, &f0);
-            eta_k2_pair(c3, 1, trans, mp0, fp, &e1c, &e1x, &f1);
+            eta_k2_pair(c3, 0, trans, k2_need(eno, 0, r), mp0, fp, &e0c, &e0x, &f0);
+            eta_k2_pair(c3, 1, trans, k2_need(eno, 1, r), mp0, fp, &e1c, &e1x, &f1);
             d = K2_EVAL | f0 | (f1 << K2_SIDE1);
         }
     }
-    int r;
-    *vm = cell_value_k2_f(c3, 0, e0c, e0x, fp, &r);
-    *vp = cell_value_k2_f(c3, 1, e1c, e1x, fp, &r);
+    *vm = cell_value_k2_f(c3, 0, e0c, e0x, r, fp);
+    *vp = cell_value_k2_f(c3, 1, e1c, e1x, r, fp);
     return d;
 }
 
@@ -1000,21 +1017,22 @@ __device__ __forceinline__ uint32_t face_field_k2(const float* w, const MethodPa
     const FParams fp = fparams(mp0);
     uint32_t fl = 0;
     float el = 0.0f, er = 0.0f, elx = 0.0f, erx = 0.0f;
+    const bool eno = fp.scheme == NPW_ENO_ || fp.scheme == NPW_RBF_ENO_;
+    const int rl = eno ? eno2_choice_f(w[1], w[2], w[3]) : 0, rr = eno ? eno2_choice_f(w[2], w[3], w[4]) : 0;
     if (fp.scheme == NPW_RBF_ENO_ || fp.scheme == NPW_RBF_WENO_) {
         if (fp.monotone_switch && switch_k2_f(w[1], w[2], w[3]))
             fl |= FL_SWITCH;
         else
-            eta_k2_pair(w + 1, 0, tl, mp0, fp, &el, &elx, &fl);
+            eta_k2_pair(w + 1, 0, tl, k2_need(eno, 0, rl) | (eta_out ? 1 : 0), mp0, fp, &el, &elx, &fl);
         uint32_t zr = 0;
         if (fp.monotone_switch && switch_k2_f(w[2], w[3], w[4]))
             fl |= FL_SWITCH_R_K2;
         else
-            eta_k2_pair(w + 2, 1, tr, mp0, fp, &er, &erx, &zr);
+            eta_k2_pair(w + 2, 1, tr, k2_need(eno, 1, rr), mp0, fp, &er, &erx, &zr);
         fl |= zr << 2;  // FL_ZERO_GUARD_R_K2, FL_ZERO_BOUND_R_K2
     }
-    int rl = 0, rr = 0;
-    *vm = cell_value_k2_f(w + 1, 0, el, elx, fp, &rl);
-    *vp = cell_value_k2_f(w + 2, 1, er, erx, fp, &rr);
+    *vm = cell_value_k2_f(w + 1, 0, el, elx, rl, fp);
+    *vp = cell_value_k2_f(w + 2, 1, er, erx, rr, fp);
     if (eta_out) *eta_out = el;
     return fl | (uint32_t(rl & 1) << 2) | (uint32_t(rr & 1) << 4);
 }

@@ -1893,7 +1893,7 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
             own_l = cx >= 0 && own_x(cx, qy);
             own_r = cx < TX_2D && own_x(cx + 1, qy);
             if (cross)
-                trans = (fast::widen(NPW_SU(cx + 3, qy + 2, k)) - 2.0 * fast::widen(NPW_SU(cx + 3, qy + 3, k))) +
+                trans = fma(-2.0, fast::widen(NPW_SU(cx + 3, qy + 3, k)), fast::widen(NPW_SU(cx + 3, qy + 2, k))) +
                         fast::widen(NPW_SU(cx + 3, qy + 4, k));
         } else {
             // consecutive threads take consecutive columns of one row (no shared-memory bank
@@ -1907,7 +1907,7 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
             own_l = cy >= 0 && own_y(qx, cy);
             own_r = cy < TY_2D && own_y(qx, cy + 1);
             if (cross)
-                trans = (fast::widen(NPW_SU(qx + 2, cy + 3, k)) - 2.0 * fast::widen(NPW_SU(qx + 3, cy + 3, k))) +
+                trans = fma(-2.0, fast::widen(NPW_SU(qx + 3, cy + 3, k)), fast::widen(NPW_SU(qx + 2, cy + 3, k))) +
                         fast::widen(NPW_SU(qx + 4, cy + 3, k));
         }
         float vm, vp;
