@@ -1008,6 +1008,7 @@ __device__ __forceinline__ void step1d_fused_warp_body(const Stage1DArgs& a, con
     float* cr = a.c + in.off;
     const bool periodic = in.bc == NPW_BC_PERIODIC;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll 2
     for (int j = threadIdx.x; j < span; j += blockDim.x) {
         int g = c0 - H + j;
         bool inflow = false;
@@ -1083,9 +1084,14 @@ __device__ __forceinline__ void step1d_fused_warp_body(const Stage1DArgs& a, con
 #pragma unroll 1
         for (int b = L + warp * 31; b < R; b += NW * 31) {
             const int e = b + lane;
-            float vl[M], vr[M], hl[M], hr[M];
+            const int g = c0 - H + e;
+            const bool skip = lane == 31 || e >= R || (!periodic && (g < 0 || g >= n));  // (a ghost: filled below)
+            float vl[M], vr[M], hl[M], hr[M], carry[M];
 #pragma unroll
             for (int k = 0; k < M; ++k) hl[k] = 0.0f;
+            if (st == 2 && !skip)
+#pragma unroll
+                for (int k = 0; k < M; ++k) carry[k] = cr[(int64_t)k * n + g];
             if (e <= R) {
 #pragma unroll
                 for (int k = 0; k < M; ++k) {
@@ -1096,8 +1102,7 @@ __device__ __forceinline__ void step1d_fused_warp_body(const Stage1DArgs& a, con
             }
 #pragma unroll
             for (int k = 0; k < M; ++k) hr[k] = __shfl_down_sync(0xffffffffu, hl[k], 1);
-            const int g = c0 - H + e;
-            if (lane == 31 || e >= R || (!periodic && (g < 0 || g >= n))) continue;  // (a ghost: filled below)
+            if (skip) continue;
             if (st < 2) {
 #pragma unroll
                 for (int k = 0; k < M; ++k) {
@@ -1113,7 +1118,7 @@ __device__ __forceinline__ void step1d_fused_warp_body(const Stage1DArgs& a, con
                     const float du = lam * (hl[k] - hr[k]);
                     const int64_t ix = (int64_t)k * n + g;
                     const float base = su0[k * S + e];
-                    const float y = kTwoThirdsF * (sd[k * S + e] + du) + cr[ix];
+                    const float y = kTwoThirdsF * (sd[k * S + e] + du) + carry[k];
                     const float t = base + y;
                     cr[ix] = y - (t - base);
                     uout[ix] = t;
@@ -2060,20 +2065,32 @@ __device__ __forceinline__ void stage2d_warp_body(const Stage2DArgs& a, const In
         };
         const int x0 = map(tx0 - 3 + min(lane, cols + 5), nx, in.bc), x1 = map(tx0 - 3 + min(lane + 32, cols + 5), nx, in.bc);
         const bool in0 = lane < cols + 6, in1 = lane + 32 < cols + 6;
-#pragma unroll 1
-        for (int by = warp; by < rows + 6; by += NW) {
+        // all of a warp's rows are fetched before the first is stored: one wait for global memory
+        constexpr int NB = (BY + NW - 1) / NW;
+        float v0[NB][M], v1[NB][M];
+#pragma unroll
+        for (int r = 0; r < NB; ++r) {
+            const int by = min(warp + r * NW, rows + 5);
             const int y = map(ty0 - 3 + by, ny, in.bc_y);
             const float* row = uin + (int64_t)max(y, 0) * nx;
-            V* to = su + by * BX + lane;
 #pragma unroll
             for (int k = 0; k < M; ++k) {
                 const float* at = row + k * cells;
-                float v0 = at[max(x0, 0)], v1 = 0.0f;
-                if (in1) v1 = at[max(x1, 0)];
-                if ((x0 | y) < 0) v0 = a.mp.inflow_f[k];
-                if ((x1 | y) < 0) v1 = a.mp.inflow_f[k];
-                if (in0) fast::lane_of(to[k / W * BY * BX], k % W) = v0;
-                if (in1) fast::lane_of(to[k / W * BY * BX + 32], k % W) = v1;
+                v0[r][k] = at[max(x0, 0)];
+                v1[r][k] = in1 ? at[max(x1, 0)] : 0.0f;
+                if ((x0 | y) < 0) v0[r][k] = a.mp.inflow_f[k];
+                if ((x1 | y) < 0) v1[r][k] = a.mp.inflow_f[k];
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < NB; ++r) {
+            const int by = warp + r * NW;
+            if (by >= rows + 6) break;
+            V* to = su + by * BX + lane;
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+                if (in0) fast::lane_of(to[k / W * BY * BX], k % W) = v0[r][k];
+                if (in1) fast::lane_of(to[k / W * BY * BX + 32], k % W) = v1[r][k];
             }
         }
     }
@@ -2156,16 +2173,27 @@ __device__ __forceinline__ void stage2d_warp_body(const Stage2DArgs& a, const In
             for (int k = 0; k < M; ++k) fast::lane_of(ef[k / W * NR * 32 + f], k % W) = h[k];
         }
     }
-    __syncthreads();
-    // U: task = row, lane = column
+    // U: task = row, lane = column; u^n is fetched while the other warps finish the fluxes
     float* uout = reinterpret_cast<float*>(a.uout) + in.off;
     const float* un = reinterpret_cast<const float*>(a.un) + in.off;
+    constexpr int NU = (TY_WARP + NW - 1) / NW;
+    float u0[NU][M];
+    if (a.stage != 0 && lane < cols) {
+#pragma unroll
+        for (int r = 0; r < NU; ++r) {
+            const int64_t at = (int64_t)(ty0 + min(warp + r * NW, rows - 1)) * nx + tx0 + lane;
+#pragma unroll
+            for (int k = 0; k < M; ++k) u0[r][k] = un[k * cells + at];
+        }
+    }
+    __syncthreads();
     const float dtR = s_par[2], idxR = s_par[3], idyR = s_par[4];
     float vmx = 0.0f, vmy = 0.0f;
     bool bad = false;
-#pragma unroll 1
-    for (int q = warp; q < rows; q += NW) {
-        if (lane >= cols) continue;
+#pragma unroll
+    for (int r = 0; r < NU; ++r) {
+        const int q = warp + r * NW;
+        if (q >= rows || lane >= cols) break;
         float U[M];
         const int64_t at = (int64_t)(ty0 + q) * nx + tx0 + lane;
 #pragma unroll
@@ -2180,9 +2208,9 @@ __device__ __forceinline__ void stage2d_warp_body(const Stage2DArgs& a, const In
             if (a.stage == 0)
                 o = uk + dtR * L;
             else if (a.stage == 1)
-                o = 0.75f * un[gidx] + 0.25f * (uk + dtR * L);
+                o = 0.75f * u0[r][k] + 0.25f * (uk + dtR * L);
             else
-                o = stage3_w1<float>() * un[gidx] + stage3_w2<float>() * (uk + dtR * L);
+                o = stage3_w1<float>() * u0[r][k] + stage3_w2<float>() * (uk + dtR * L);
             uout[gidx] = o;
             U[k] = o;
             bad |= !finite_(o);
