@@ -2581,10 +2581,12 @@ __device__ __forceinline__ void queue_item_2d(const Stage2DArgs& a2, const Inst2
 }
 
 // CTAs per SM the register allocation aims for: 4 for the specialised mixed-precision k = 3 kernels
-// (64 registers a thread for the f32x2 pairs; their shared memory allows as many), else no bound
+// (64 registers a thread for the f32x2 pairs; their shared memory allows as many), 3 for the
+// characteristic one (it takes 116 registers when left alone, and two CTAs are too few warps to hide its
+// long chains), else no bound
 template <typename R, int K, bool CHAR, int SHAPE>
 constexpr int queue_min_blocks() {
-    return sizeof(R) == sizeof(float) && K == 3 && !CHAR && SHAPE != QS_ANY ? 4 : 1;
+    return sizeof(R) == sizeof(float) && K == 3 && SHAPE != QS_ANY ? (CHAR ? 3 : 4) : 1;
 }
 
 template <typename R, int K, bool CHAR, int SHAPE>
@@ -2667,13 +2669,17 @@ __device__ __forceinline__ void queue_stage_body(const QueueArgs& q) {
 }
 
 
-// the kernels: one without a register bound, one bounded at 4 CTAs per SM (see queue_min_blocks)
+// the kernels: one without a register bound, one bounded at 4 and one at 3 CTAs per SM (see queue_min_blocks)
 template <typename R, int K, bool CHAR, int SHAPE>
 __global__ void __launch_bounds__(THREADS_1D) queue_stage_kernel(QueueArgs q) {
     queue_stage_body<R, K, CHAR, SHAPE>(q);
 }
 template <typename R, int K, bool CHAR, int SHAPE>
 __global__ void __launch_bounds__(THREADS_1D, 4) queue_stage_kernel_b4(QueueArgs q) {
+    queue_stage_body<R, K, CHAR, SHAPE>(q);
+}
+template <typename R, int K, bool CHAR, int SHAPE>
+__global__ void __launch_bounds__(THREADS_1D, 3) queue_stage_kernel_b3(QueueArgs q) {
     queue_stage_body<R, K, CHAR, SHAPE>(q);
 }
 
