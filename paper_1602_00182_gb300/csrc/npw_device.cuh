@@ -84,13 +84,6 @@ __device__ __forceinline__ T pert_coef(int rbf, int row, int j) {
     }
 }
 
-// linear weights for v^-_{i+1/2} (d_r, r = cells to the left) and mirrored for v^+_{i-1/2}
-template <typename T>
-__device__ __forceinline__ T lin_weight(int side, int r) {
-    if (side == 0) return r == 0 ? T(3.0 / 10.0) : (r == 1 ? T(3.0 / 5.0) : T(1.0 / 10.0));
-    return r == 0 ? T(1.0 / 10.0) : (r == 1 ? T(3.0 / 5.0) : T(3.0 / 10.0));
-}
-
 // ---------------------------------------------------------------------------------------
 // Shape parameter (Table k3): eta = (w0 - 3 w1 + 3 w2 - w3) / (w0 - 15 w1 + 15 w2 - w3 + eps_M)
 // with w = cells i-1..i+2 of face i+1/2.
@@ -164,62 +157,6 @@ __device__ __forceinline__ int eno_choice(D c0, D c1, D c2, D c3, D c4) {
     return (ddl < ddr) ? 1 : 0;
 }
 
-// Jiang-Shu smoothness indicators (cited in Sec. 2): beta[r] of stencil i-r..i-r+2.
-template <typename D>
-__device__ __forceinline__ void beta_k3(D c0, D c1, D c2, D c3, D c4, D beta[3]) {
-    D a, b;
-    a = c2 - D(2.0) * c3 + c4;
-    b = D(3.0) * c2 - D(4.0) * c3 + c4;
-    beta[0] = D(13.0 / 12.0) * a * a + D(0.25) * b * b;
-    a = c1 - D(2.0) * c2 + c3;
-    b = c1 - c3;
-    beta[1] = D(13.0 / 12.0) * a * a + D(0.25) * b * b;
-    a = c0 - D(2.0) * c1 + c2;
-    b = c0 - D(4.0) * c1 + D(3.0) * c2;
-    beta[2] = D(13.0 / 12.0) * a * a + D(0.25) * b * b;
-}
-
-// ---------------------------------------------------------------------------------------
-// Value of cell i at its right face (side 0: v^-_{i+1/2}, rows r) or left face (side 1:
-// v^+_{i-1/2}, rows r - 1).  c[0..4] = cells i-2..i+2; eta is the face's shape parameter
-// (already rounded to R).  forced_r >= 0 replays a stencil choice.
-// ---------------------------------------------------------------------------------------
-template <typename R, typename D>
-__device__ __forceinline__ R cell_face_value(const R* c, int side, R eta, const MethodParams& mp, int* r_out) {
-    R cand[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        const int row = (side == 0) ? r : r - 1;
-        R s = R(0.0);
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            R coef = poly_coef<R>(row + 1, j) + pert_coef<R>(mp.rbf, row + 1, j) * eta;
-            s += coef * c[2 - r + j];
-        }
-        cand[r] = s;
-    }
-    if (mp.scheme == NPW_ENO_ || mp.scheme == NPW_RBF_ENO_) {
-        int r = eno_choice<D>(D(c[0]), D(c[1]), D(c[2]), D(c[3]), D(c[4]));
-        *r_out = r;
-        return r == 0 ? cand[0] : (r == 1 ? cand[1] : cand[2]);
-    }
-    *r_out = 0;
-    D beta[3];
-    beta_k3<D>(D(c[0]), D(c[1]), D(c[2]), D(c[3]), D(c[4]), beta);
-    R alpha[3];
-    R asum = R(0.0);
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        R den = R(D(mp.eps_weno) + beta[r]);
-        alpha[r] = lin_weight<R>(side, r) / (den * den);
-        asum += alpha[r];
-    }
-    R v = R(0.0);
-#pragma unroll
-    for (int r = 0; r < 3; ++r) v += (alpha[r] / asum) * cand[r];
-    return v;
-}
-
 // ---------------------------------------------------------------------------------------
 // k = 2.  Table k2: row = r + 1 for r = -1, 0, 1; row r gives the value at x_{i+1/2} from the
 // cells i-r, i-r+1.  A cell i has the stencil c[0..2] = cells i-1, i, i+1; its two face
@@ -267,34 +204,6 @@ template <typename T>
 __device__ __forceinline__ T lin_weight2(int side, int r) {
     if (side == 0) return r == 0 ? T(2.0 / 3.0) : T(1.0 / 3.0);
     return r == 0 ? T(1.0 / 3.0) : T(2.0 / 3.0);
-}
-
-// shape parameter of a cell, side 0 / 1 (MQ: 2 num / (den + eps_M); Gaussian: half), with the
-// optional guard and bound of the k = 3 path (magnitudes of the denominator's terms).  On the
-// 5-cell cross of Sec. 6 (2D) the numerator also carries the transverse second difference
-// trans of the cell, with weight -1/4 for the stencil of the two cells at the face (central)
-// and 1/8 for the extrapolating one: the terms that cancel the transverse curvature of the
-// cell averages at the face midpoint.
-// *zr receives FL_ZERO_GUARD / FL_ZERO_BOUND where the guard / the bound set eta to 0
-template <typename D>
-__device__ __forceinline__ D eta_k2_cross(const D* c, int side, bool central, D trans, const MethodParams& mp,
-                                          uint32_t* zr) {
-    const D a = side == 0 ? c[0] : c[2];
-    const D b = c[1];
-    const D d = side == 0 ? c[2] : c[0];
-    const D num = -a + D(2.0) * b - d + (central ? D(-0.25) : D(0.125)) * trans;
-    const D den0 = -a + D(5.0) * b + D(2.0) * d;
-    const D mag = fabs(a) + D(5.0) * fabs(b) + D(2.0) * fabs(d);
-    if (mp.eta_guard > 0.0 && fabs(den0) <= D(mp.eta_guard) * mag) {
-        *zr |= FL_ZERO_GUARD;
-        return D(0.0);
-    }
-    const D e = (mp.rbf == NPW_RBF_GA_ ? D(1.0) : D(2.0)) * num / (den0 + D(mp.eps_M));
-    if (mp.eta_max > 0.0 && fabs(e) > D(mp.eta_max)) {
-        *zr |= FL_ZERO_BOUND;
-        return D(0.0);
-    }
-    return e;
 }
 
 // value of cell i at its right (side 0) or left (side 1) face, k = 2; c[0..2] = cells i-1..i+1;
@@ -358,7 +267,12 @@ __device__ __forceinline__ double cell_value_k2_d(const double* c, int side, dou
     return f64::div(a0, sum) * cand(0) + f64::div(a1, sum) * cand(1);
 }
 
-// face_field_k2<double> with fewer FP64-pipe instructions and the same bits (see npw_double.cuh)
+// One field at one face, k = 2.  w[0..5] = cells i-2..i+3 around face i+1/2; v^- from cell i
+// (stencil w[1..3]), v^+ from cell i+1 (stencil w[2..4]); tl, tr: transverse second
+// differences of cells i and i+1 (0 on a line).  Flag bits: 0 switch of cell i, 3 switch of
+// cell i+1, 2 / 4 ENO r of cell i / i+1, 6 / 7 an eta of v^- zeroed by the guard / the bound,
+// 8 / 9 the same for v^+.
+// Arithmetic of npw_double.cuh; eta of v^- and v^+ from f64::eta_k2_pair.
 __device__ __forceinline__ uint32_t face_field_k2_d(const double* w, const MethodParams& mp, double* vm, double* vp,
                                                     double tl, double tr, double* eta_out) {
     uint32_t fl = 0;
@@ -389,42 +303,6 @@ __device__ __forceinline__ uint32_t face_field_k2_d(const double* w, const Metho
     }
     *vm = cell_value_k2_d(w + 1, 0, el, elx, rl, mp);
     *vp = cell_value_k2_d(w + 2, 1, er, erx, rr, mp);
-    fl |= (uint32_t(rl & 1) << 2) | (uint32_t(rr & 1) << 4);
-    if (eta_out) *eta_out = el;
-    return fl;
-}
-
-// One field at one face, k = 2.  w[0..5] = cells i-2..i+3 around face i+1/2; v^- from cell i
-// (stencil w[1..3]), v^+ from cell i+1 (stencil w[2..4]); tl, tr: transverse second
-// differences of cells i and i+1 (0 on a line).  Flag bits: 0 switch of cell i, 3 switch of
-// cell i+1, 2 / 4 ENO r of cell i / i+1, 6 / 7 an eta of v^- zeroed by the guard / the bound,
-// 8 / 9 the same for v^+.
-template <typename R, typename D>
-__device__ __forceinline__ uint32_t face_field_k2(const R* w, const MethodParams& mp, R* vm, R* vp, R tl, R tr,
-                                                  R* eta_out) {
-    uint32_t fl = 0;
-    R el = R(0.0), er = R(0.0), elx = R(0.0), erx = R(0.0);
-    if (mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_) {
-        const D cl[3] = {D(w[1]), D(w[2]), D(w[3])};
-        const D cr[3] = {D(w[2]), D(w[3]), D(w[4])};
-        if (mp.monotone_switch && k2_ratio_fires<D>(cl[0], cl[1], cl[2])) {
-            fl |= FL_SWITCH;
-        } else {
-            el = R(eta_k2_cross<D>(cl, 0, true, D(tl), mp, &fl));
-            elx = tl == R(0.0) ? el : R(eta_k2_cross<D>(cl, 0, false, D(tl), mp, &fl));
-        }
-        if (mp.monotone_switch && k2_ratio_fires<D>(cr[0], cr[1], cr[2])) {
-            fl |= FL_SWITCH_R_K2;
-        } else {
-            uint32_t zr = 0;
-            er = R(eta_k2_cross<D>(cr, 1, true, D(tr), mp, &zr));
-            erx = tr == R(0.0) ? er : R(eta_k2_cross<D>(cr, 1, false, D(tr), mp, &zr));
-            fl |= zr << 2;  // FL_ZERO_GUARD_R_K2, FL_ZERO_BOUND_R_K2
-        }
-    }
-    int rl = 0, rr = 0;
-    *vm = cell_face_value_k2<R, D>(w + 1, 0, el, elx, mp, &rl);
-    *vp = cell_face_value_k2<R, D>(w + 2, 1, er, erx, mp, &rr);
     fl |= (uint32_t(rl & 1) << 2) | (uint32_t(rr & 1) << 4);
     if (eta_out) *eta_out = el;
     return fl;
@@ -518,7 +396,8 @@ __device__ __forceinline__ uint32_t face_point_k2(const R* w, const MethodParams
     return fl;
 }
 
-// face_field<double> for k = 3 (see npw_double.cuh): the weights of both cells, the coefficients once
+// One field at one face, k = 3 (arguments and flags as face_field): the weights of both cells, the
+// coefficients once; arithmetic of npw_double.cuh
 __device__ __forceinline__ uint32_t face_field_d(const double* w, const MethodParams& mp, double* vm, double* vp,
                                                  double* eta_out) {
     uint32_t fl = 0;
@@ -548,41 +427,9 @@ __device__ __forceinline__ uint32_t face_field_d(const double* w, const MethodPa
 // byte (bit0 switch, bits 2-3 / 4-5 ENO r of the left / right cell, bit 6 / 7 the evaluated eta
 // zeroed by the guard / the bound).
 // eta_out (may be NULL): the face's shape parameter as used (k = 2: that of v^-, central row)
-template <typename R, typename D>
-__device__ __forceinline__ uint32_t face_field(const R* w, const MethodParams& mp, R* vm, R* vp, R tl = R(0.0),
-                                               R tr = R(0.0), R* eta_out = nullptr) {
-    if constexpr (sizeof(R) == sizeof(double))
-        return mp.k == 2 ? face_field_k2_d(w, mp, vm, vp, tl, tr, eta_out) : face_field_d(w, mp, vm, vp, eta_out);
-    if (mp.k == 2) return face_field_k2<R, D>(w, mp, vm, vp, tl, tr, eta_out);
-    uint32_t fl = 0;
-    R eta = R(0.0);
-    if (mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_) {
-        const D w1 = D(w[1]), w2 = D(w[2]), w3 = D(w[3]), w4 = D(w[4]);
-        bool fires = mp.monotone_switch ? switch_fires<D>(w1, w2, w3, w4, mp.switch_variant) : false;
-        if (fires) {
-            fl |= FL_SWITCH;
-        } else {
-            D den0 = eta_den<D>(w1, w2, w3, w4);
-            bool unresolved = mp.eta_guard > 0.0 &&
-                              fabs(den0) <= D(mp.eta_guard) * (fabs(w1) + D(15.0) * fabs(w2) + D(15.0) * fabs(w3) + fabs(w4));
-            if (!unresolved) {
-                D den = den0 + D(mp.eps_M);
-                D e = eta_num<D>(w1, w2, w3, w4) / den;
-                if (!(mp.eta_max > 0.0 && fabs(e) > D(mp.eta_max)))
-                    eta = R(e);
-                else
-                    fl |= FL_ZERO_BOUND;
-            } else {
-                fl |= FL_ZERO_GUARD;
-            }
-        }
-    }
-    int rl = 0, rr = 0;
-    *vm = cell_face_value<R, D>(w, 0, eta, mp, &rl);
-    *vp = cell_face_value<R, D>(w + 1, 1, eta, mp, &rr);
-    fl |= (uint32_t(rl & 3) << 2) | (uint32_t(rr & 3) << 4);
-    if (eta_out) *eta_out = eta;
-    return fl;
+__device__ __forceinline__ uint32_t face_field(const double* w, const MethodParams& mp, double* vm, double* vp, double tl = 0.0,
+                                               double tr = 0.0, double* eta_out = nullptr) {
+    return mp.k == 2 ? face_field_k2_d(w, mp, vm, vp, tl, tr, eta_out) : face_field_d(w, mp, vm, vp, eta_out);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -669,7 +516,7 @@ static __device__ __noinline__ bool face_near_tie_d(double w1, double w2, double
 // passes; the rest takes the FP64 expressions, some 60 FP64-pipe instructions, which bounded
 // npweno_reconstruct before.
 __device__ __forceinline__ bool far_from_ties(float d0, float d1, float d2, float a1, float a2, float unit, float abs_err,
-                                              const MethodParams& mp, float tol) {
+                                              const MethodParams& mp, float tol, bool exact_ab = false) {
     const float t02 = d0 + d2, s = fabsf(d0) + fabsf(d2);
     const float A = fmaf(-2.f, d1, t02), B = d2 - d0, C = fmaf(14.f, d1, -t02);
     const float aA = fabsf(A), aB = fabsf(B), aC = fabsf(C);
@@ -680,8 +527,9 @@ __device__ __forceinline__ bool far_from_ties(float d0, float d1, float d2, floa
     if (mp.monotone_switch) {
         const float lim = 100.f * tol * mag, E = fmaf(24.f, A, C), aE = fabsf(E), eE = fmaf(64.f, e, lim), b12 = 12.f * aB;
         far_ = fabsf(b12 - aE) > eE + 0x1p-20f * (b12 + aE);  // both ends
-        const float a4 = 4.f * aA;
-        const bool inside = aB < a4 * (1.f - 0x1p-10f) - 8.f * e, outside = aB > fmaf(a4, 1.f + 0x1p-10f, 8.f * e);
+        const float a4 = 4.f * aA, e8 = exact_ab ? 0.0f : 8.f * e;
+        const bool inside = aB < a4 * (1.f - 0x1p-10f) - e8,
+                   outside = aB > fmaf(a4, 1.f + 0x1p-10f, e8) || (exact_ab && aA == 0.0f);
         const float G = fmaf(2.f * A, C, -3.f * B * B);
         far_ = far_ & (outside | (inside & (fabsf(G) > fmaf(40.f * e, aA + aB + aC + e, 2.5f * aA * lim))));
     }
@@ -703,10 +551,19 @@ __device__ __forceinline__ bool face_near_tie(const R* wr, const MethodParams& m
         // a constant stencil: monotone, its denominator and eta exactly 0 against positive thresholds
         if (wr[1] == wr[2] && wr[2] == wr[3] && wr[3] == wr[4]) return false;
         bool ok = true;
-        if constexpr (sizeof(R) == sizeof(float))
-            ok = far_from_ties(wr[2] - wr[1], wr[3] - wr[2], wr[4] - wr[3], fabsf(wr[2]), fabsf(wr[3]), 0x1p-19f, 0.0f, mp,
-                               mp.tie_tol_f);
-        else {
+        if constexpr (sizeof(R) == sizeof(float)) {
+            const float d0 = wr[2] - wr[1], d1 = wr[3] - wr[2], d2 = wr[4] - wr[3];
+            ok = far_from_ties(d0, d1, d2, fabsf(wr[2]), fabsf(wr[3]), 0x1p-19f, 0.0f, mp, mp.tie_tol_f);
+            if (!ok) {
+                // nearly linear data: A and B are a few units of round-off, but then exact.  A difference is
+                // exact where adding it back gives the other cell, either way round.
+                const float t02 = d0 + d2, A = fmaf(-2.f, d1, t02), B = d2 - d0;
+                auto sum_exact = [](float x, float y, float z) { return z - x == y && z - y == x; };
+                if (sum_exact(wr[2], -wr[1], d0) && sum_exact(wr[3], -wr[2], d1) && sum_exact(wr[4], -wr[3], d2) &&
+                    sum_exact(d0, d2, t02) && sum_exact(t02, -2.f * d1, A) && sum_exact(d2, -d0, B))
+                    ok = far_from_ties(d0, d1, d2, fabsf(wr[2]), fabsf(wr[3]), 0x1p-19f, 0.0f, mp, mp.tie_tol_f, true);
+            }
+        } else {
             const float d0 = f64::to_f(wr[2] - wr[1], &ok), d1 = f64::to_f(wr[3] - wr[2], &ok),
                         d2 = f64::to_f(wr[4] - wr[3], &ok), a1 = fabsf(f64::to_f(wr[2], &ok)),
                         a2 = fabsf(f64::to_f(wr[3], &ok));

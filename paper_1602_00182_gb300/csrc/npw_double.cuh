@@ -100,8 +100,8 @@ __device__ __forceinline__ bool switch_v0(double w0, double w1, double w2, doubl
     return switch_fires_d(w0, w1, w2, w3, 0);
 }
 
-// Table k3 shape parameter of the face with eta stencil w0..w3 and its flags, as face_field<double> gives
-// them (the guard is off by default in NPW_FP64)
+// Table k3 shape parameter of the face with eta stencil w0..w3 and its flags, 0 where the switch, the guard
+// or the bound says so (the guard is off by default in NPW_FP64)
 __device__ __forceinline__ double face_eta(double w0, double w1, double w2, double w3, const MethodParams& mp, uint32_t* fl) {
     if (mp.scheme != NPW_RBF_ENO_ && mp.scheme != NPW_RBF_WENO_) return 0.0;
     if (mp.monotone_switch &&
@@ -214,8 +214,11 @@ __device__ __forceinline__ bool k2_switch(double a, double b, double c, double d
     return k2_ratio_fires_d(a, b, c);
 }
 
-// Both shape parameters of one face value of a k = 2 cell (eta_k2_cross): a, b, d the cells beside, at
-// and across from the face, t = -a + 2b - d, trans the transverse difference.  They share the
+// Both shape parameters of one face value of a k = 2 cell, MQ: 2 num / (den + eps_M), Gaussian: half: a,
+// b, d the cells beside, at and across from the face, t = -a + 2b - d.  On the 5-cell cross of Sec. 6 the
+// numerator also carries the transverse second difference trans of the cell, with weight -1/4 for the
+// stencil of the two cells at the face (central) and 1/8 for the extrapolating one: the terms that
+// cancel the transverse curvature of the cell averages at the face midpoint.  Both share the
 // denominator, hence its reciprocal.  need: bit 0 the central, bit 1 the extrapolating one is used;
 // the other is formed only where it might reach the bound (its flag counts).
 __device__ __forceinline__ void eta_k2_pair(double a, double b, double d, double t, double trans, int need,

@@ -1060,7 +1060,7 @@ __device__ __forceinline__ uint32_t face_field_any(const R* w, const MethodParam
     if constexpr (sizeof(R) == sizeof(float)) {
         return fast::face_field(w, mp, vm, vp, tl, tr, eta_out);
     } else {
-        return face_field<R, D>(w, mp, vm, vp, R(tl), R(tr), eta_out);
+        return face_field(w, mp, vm, vp, R(tl), R(tr), eta_out);
     }
 }
 

@@ -430,7 +430,7 @@ __device__ __forceinline__ void stage1d_body(const Stage1DArgs& a, const Tile td
 // the shape parameter, the four candidates of its face (rows 1 and 2 serve both values) and the flux;
 // lanes 1..30 update their cells, upd(j, flux of face j, flux of face j + 1).  X(k, i): the stage input,
 // i in -3..cnt + 2; last: the line's last face is counted here.  The arithmetic and its order are those
-// of face_field<double>, so the results are the same bits.  Bound by the FP64 pipe (see
+// of face_field_d, so the results are the same bits.  Bound by the FP64 pipe (see
 // npw_double.cuh): against the face-by-face body the indicators and weights of a cell are formed once
 // instead of once per face.
 // ---------------------------------------------------------------------------------------
