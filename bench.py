@@ -478,7 +478,7 @@ def block_euler1d(args, characteristic: int):
     stage_s = prof.pr.stage_ms / 1e3
     eta_tot = {k: sum(s["eta"][k] for s in stats) for k in ("switch", "eval", "guard", "bound")}
     kern = ("queue_stage_kernel<float, K=3, characteristic, 1D Euler> (face-based Roe-field body)" if characteristic
-            else "queue_stage_kernel_b5<float, K=3, 1D Euler> (fused RK3 step body)")
+            else "queue_stage_kernel_b4<float, K=3, 1D Euler> (fused RK3 step body)")
     return {
         "metric": "cell-updates/s", "value": cu / (ms / 1e3), "unit": "cell-updates/s", "dtype": "f32",
         "ms_per_solve": ms,
@@ -559,7 +559,7 @@ def block_euler2d(args):
                    "l2": "flushed before every timed solve"},
         "sizes": sizes,
         "roofline": roofline_hbm(BYTES_EULER2D_F32, tot_cu, tot_stage_s,
-                                 "queue_stage_kernel_b5<float, K=3, 2D Euler> (phased 2D body, 32 x 8 tiles)",
+                                 "queue_stage_kernel_b4<float, K=3, 2D Euler> (2D body of warp tasks, 30 x 11 tiles)",
                                  traffic=_ncu_traffic("queue_stage_euler2d_512_dram_bytes_per_launch"),
                                  traffic_unit="bytes per stage launch, 64 squares of 512^2 (2^24 cells, every size's "
                                               "launch)"),
