@@ -548,6 +548,7 @@ int auto_tile(const std::vector<int64_t>& n_of, StageKind kind, int min_warps = 
     return best;
 }
 
+constexpr int FUSED_TILE_MAX = 484;
 // The work queue's tile of these 1D lines.  Fused steps: 484, 228 or 100 cells (whole warp tasks, see
 // step1d_fused_warp_body), the one whose busiest SM of four resident CTAs has the least to do, tile +
 // 28 cells' worth per tile.  Else auto_tile, in tiles of at least 255 cells for the characteristic
@@ -558,7 +559,7 @@ int queue_tile(const std::vector<int64_t>& n_of, bool fused, StageKind kind, boo
     if (!fused) return auto_tile(n_of, kind, characteristic_f32 ? 8 : 2);
     int best = 0;
     int64_t best_cost = 0;
-    for (int t : {100, 228, 484}) {
+    for (int t : {100, 228, FUSED_TILE_MAX}) {
         int64_t tiles = 0;
         for (int64_t n : n_of) tiles += (n + t - 1) / t;
         const int64_t cost = (tiles + 4 * npw::NUM_SMS - 1) / (4 * npw::NUM_SMS) * (t + 28);
@@ -1219,8 +1220,13 @@ npw_status npweno_batch_solve(void* arena, const npw_instance* inst, int32_t cou
         int64_t end = inst[i].offset + inst[i].n * m;
         arena_elems = end > arena_elems ? end : arena_elems;
     }
-    const int automatic = batch_auto_tile(inst, count, m, params);
-    const int64_t nt = batch_table(inst, count, m, params, automatic);
+    int automatic = batch_auto_tile(inst, count, m, params);
+    int64_t nt = batch_table(inst, count, m, params, automatic);
+    if (workspace_bytes < layout_1d(arena_elems, count, nt, elem_size(params)).total) {
+        // a workspace without room for the table of the small tiles: the largest
+        automatic = npw::TILE_1D;
+        nt = batch_table(inst, count, m, params, automatic);
+    }
     if (nt > (int64_t)1 << 30) return fail(NPW_EINVAL, "too many tiles");
     Run1D r{};
     r.arena = arena;
@@ -1624,9 +1630,12 @@ void plan_2d(npw::Inst2D& d, bool warp_tiles) {
 }
 
 bool is_2d_kind(const npw_queue_instance& q) { return q.ny != 0; }
-int64_t items_of(const npw_queue_instance& q, int tile) {
-    if (is_2d_kind(q)) return ((q.nx + npw::TX_2D - 1) / npw::TX_2D) * ((q.ny + npw::TY_2D - 1) / npw::TY_2D);
-    return (q.nx + tile - 1) / tile;
+// work items of an instance: 1D tiles of the given size, or the tiles of plan_2d
+int64_t items_of(const npw_queue_instance& q, int tile, const npw_params* p) {
+    if (!is_2d_kind(q)) return (q.nx + tile - 1) / tile;
+    const bool warp = npw::warp_tiles_2d(p->precision == NPW_FP32_MIXED, p->k);
+    const int tx = warp ? npw::TX_WARP : npw::TX_2D, ty = warp ? npw::TY_WARP : npw::TY_2D;
+    return ((q.nx + tx - 1) / tx) * ((q.ny + ty - 1) / ty);
 }
 int64_t cells_of(const npw_queue_instance& q) { return q.nx * (q.ny ? q.ny : 1) * flux_m(q.flux_kind); }
 
@@ -1656,7 +1665,7 @@ npw_status check_queue(const npw_queue_instance* inst, int count, const npw_para
         if (q.offset < 0) return fail(NPW_EINVAL, "instance %d: negative offset", i);
         const int64_t end = q.offset + cells_of(q);
         arena = end > arena ? end : arena;
-        items += items_of(q, npw::TILE_QUEUE_MIN);
+        items += items_of(q, npw::TILE_QUEUE_MIN, p);
     }
     if (items > ((int64_t)1 << 30)) return fail(NPW_EINVAL, "too many work items");
     *arena_elems = arena;
@@ -1842,6 +1851,13 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
     r.s = reinterpret_cast<cudaStream_t>(stream);
     r.ws = static_cast<unsigned char*>(workspace);
     r.L = queue_layout(arena_elems, count, items_bound, elem_size(params), r.comp);
+    const bool tight = workspace_bytes < r.L.total;  // no room for the table of the small tiles: the largest
+    if (tight) {
+        int64_t items = 0;
+        for (int i = 0; i < count; ++i) items += items_of(inst[i], npw::TILE_1D_MIN, params);
+        items_bound = items;
+        r.L = queue_layout(arena_elems, count, items, elem_size(params), r.comp);
+    }
     if (workspace_bytes < r.L.total)
         return fail(NPW_EINVAL, "workspace too small: %zu < %zu bytes", workspace_bytes, r.L.total);
     // 1D tile: the autotuned (or given) tile of the 1D kind with the most cells
@@ -1859,7 +1875,8 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
     }
     r.fused = r.comp && !any2d;
     // (npw_autotune_1d times the per-stage kernels: its choice is not for fused steps)
-    const int automatic = queue_tile(lines, r.fused, stage_kind(params), r.fp32 && r.characteristic);
+    const int automatic = tight ? (r.fused ? FUSED_TILE_MAX : npw::TILE_1D)
+                                : queue_tile(lines, r.fused, stage_kind(params), r.fp32 && r.characteristic);
     const int tile = r.fused ? (params->tile_1d > 0 ? params->tile_1d : automatic)
                              : resolve_tile(params, main_kind, flux_m(main_kind), automatic);
     // descriptors; mixed-precision 1D instances that fit in shared memory run resident
@@ -1912,6 +1929,7 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
     for (int i = 0; i < count; ++i)
         if (h2d[i])
             for (int32_t t = 0; t < h2[i].tiles_x * h2[i].tiles_y; ++t) items.push_back(npw::Tile{i, t});
+    if ((int64_t)items.size() > items_bound) return fail(NPW_EINVAL, "more work items than the workspace holds");
     // one shape for every instance with queue items: the kernel specialised for it
     r.shape = -1;
     for (int i = 0; i < count && r.shape != npw::QS_ANY; ++i) {
@@ -2003,7 +2021,7 @@ constexpr int kGroups = 7;                // instance shapes (npw::QueueShape): 
 constexpr double kStepSliceS = 0.005;     // longest wait of npw_server_step for a round to end
 
 struct LaneLayout {
-    size_t inst1, inst2, kind, is2d, ctl, items, newitems, list, head, poll, heap_u, heap_u1, heap_u2, heap_s, heap_c;
+    size_t inst1, inst2, kind, is2d, ctl, items, list, head, poll, heap_u, heap_u1, heap_u2, heap_s, heap_c;
     size_t begin, end;
     int64_t max_items;
 };
@@ -2011,9 +2029,9 @@ struct LaneLayout {
 // one lane's part of the arena, starting at byte `begin`
 LaneLayout lane_layout(size_t begin, int64_t heap_cells, int max_slots, size_t esz, bool comp) {
     LaneLayout L{};
-    // a 2D request of at least 6 x 6 cells has at most cells / 42 + 1 tiles of 30 x 11, a 1D one cells /
-    // 63 + 1 tiles of 63 cells
-    L.max_items = heap_cells / 32 + 2 * (int64_t)max_slots;
+    // one list, twice the 256-cell tiles of the heap and four a slot; 1D tiles grow where it would not do
+    const int64_t half = heap_cells / (npw::TX_2D * npw::TY_2D) + 2 * (int64_t)max_slots;
+    L.max_items = 2 * half;
     size_t o = align256(begin);
     L.begin = o;
     L.inst1 = o;
@@ -2027,9 +2045,7 @@ LaneLayout lane_layout(size_t begin, int64_t heap_cells, int max_slots, size_t e
     L.ctl = o;
     o = align256(o + sizeof(npw::Ctl) * (size_t)max_slots);
     L.items = o;
-    o = align256(o + sizeof(npw::Tile) * (size_t)L.max_items);
-    L.newitems = o;
-    o = align256(o + sizeof(npw::Tile) * (size_t)L.max_items);
+    o = align256(align256(o + sizeof(npw::Tile) * (size_t)half) + sizeof(npw::Tile) * (size_t)half);
     L.list = o;
     o = align256(o + sizeof(int32_t) * (size_t)max_slots);
     L.head = o;  // a queue counter pair per launch group
@@ -2196,13 +2212,13 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
         std::vector<int> members;
         bool is2d = false, fused = false;
         int m = 1, tile = npw::TILE_1D;
-        int64_t ib = 0, ie = 0, nb = 0, ne = 0;  // [ib, ie) in items, [nb, ne) in newitems
+        int64_t ib = 0, ie = 0, ne = 0;  // its work items are [ib, ie), those of the admitted requests [ib, ne)
     } grp[kGroups];
     std::vector<npw::InstDev> h1(S);
     std::vector<npw::Inst2D> h2(S);
     std::vector<int32_t> hk(S, 0);
     std::vector<uint8_t> h2d(S, 0);
-    std::vector<npw::Tile> items, newitems;
+    std::vector<npw::Tile> items;
     std::vector<int32_t> fresh;
     for (int k = 0; k < S; ++k) {
         npw_server::Slot& sl = sv->slots[k];
@@ -2231,34 +2247,42 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
         }
         if (sl.fresh) fresh.push_back(k);
     }
+    int64_t total = 0;
+    auto tile_lines = [&](Group& g, int tile) {
+        g.tile = tile;
+        for (int k : g.members) {
+            h1[k].ntiles = (int32_t)tiles_of(h1[k].n, g.tile);
+            total += h1[k].ntiles;
+        }
+    };
+    int64_t total2d = 0;
     for (Group& g : grp) {
-        if (g.is2d || g.members.empty()) continue;
+        if (g.members.empty()) continue;
+        if (g.is2d) {
+            for (int k : g.members) total2d += (int64_t)h2[k].tiles_x * h2[k].tiles_y;
+            continue;
+        }
         std::vector<int64_t> lines;
         for (int k : g.members) lines.push_back(h1[k].n);
-        g.tile = queue_tile(lines, g.fused, lane.mp.k == 3 ? STAGE_DOUBLE : STAGE_FACES, false);
-        for (int k : g.members) h1[k].ntiles = (int32_t)tiles_of(h1[k].n, g.tile);
+        tile_lines(g, queue_tile(lines, g.fused, lane.mp.k == 3 ? STAGE_DOUBLE : STAGE_FACES, false));
     }
-    // work items, contiguous per group; the admitted requests' items likewise
+    // more than the list holds (a few long lines in a heap of their size take small tiles): the largest tiles
+    if (total + total2d > lane.L.max_items)
+        for (Group& g : grp)
+            if (!g.is2d) tile_lines(g, g.fused ? FUSED_TILE_MAX : npw::TILE_1D);
+    // work items, contiguous per group, the admitted requests' first
     for (int gi = 0; gi < kGroups; ++gi) {
         Group& g = grp[gi];
-        g.ib = (int64_t)items.size();
-        g.nb = (int64_t)newitems.size();
-        for (int k : g.members) {
-            const bool fr = sv->slots[k].fresh;
-            if (!g.is2d) {
-                for (int32_t t = 0; t < h1[k].ntiles; ++t) {
-                    items.push_back(npw::Tile{k, t * g.tile});
-                    if (fr) newitems.push_back(npw::Tile{k, t * g.tile});
-                }
-            } else {
-                for (int32_t t = 0; t < h2[k].tiles_x * h2[k].tiles_y; ++t) {
-                    items.push_back(npw::Tile{k, t});
-                    if (fr) newitems.push_back(npw::Tile{k, t});
-                }
+        g.ib = g.ne = (int64_t)items.size();
+        for (const bool fr : {true, false}) {
+            for (int k : g.members) {
+                if (sv->slots[k].fresh != fr) continue;
+                const int32_t nt = g.is2d ? h2[k].tiles_x * h2[k].tiles_y : h1[k].ntiles;
+                for (int32_t t = 0; t < nt; ++t) items.push_back(npw::Tile{k, g.is2d ? t : t * g.tile});
             }
+            if (fr) g.ne = (int64_t)items.size();
         }
         g.ie = (int64_t)items.size();
-        g.ne = (int64_t)newitems.size();
     }
     if (items.empty()) return NPW_OK;
     if ((int64_t)items.size() > lane.L.max_items) return fail(NPW_EINVAL, "server: too many work items");
@@ -2272,21 +2296,18 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
                              ls));
     const npw::QueueArgs q0 = lane_queue(sv, ln);
     const npw::Tile* ditems = q0.items;
-    const npw::Tile* dnew = reinterpret_cast<const npw::Tile*>(a + L.newitems);
     if (!fresh.empty()) {
         // start the admitted requests: reset, alpha^0 over their items, first dt and step limit
         int32_t* dlist = reinterpret_cast<int32_t*>(a + L.list);
         NPW_CUDA(cudaMemcpyAsync(dlist, fresh.data(), sizeof(int32_t) * fresh.size(), cudaMemcpyHostToDevice, ls));
-        NPW_CUDA(cudaMemcpyAsync(a + L.newitems, newitems.data(), sizeof(npw::Tile) * newitems.size(),
-                                 cudaMemcpyHostToDevice, ls));
         NPW_CUDA(npw::launch_queue_ctl(q0.ctl, q0.inst1, q0.inst2, q0.is2d, dlist, (int)fresh.size(), 0, 0, ls));
         count_launch();
         for (int gi = 0; gi < kGroups; ++gi) {
             const Group& g = grp[gi];
-            if (g.ne <= g.nb) continue;
+            if (g.ne <= g.ib) continue;
             npw::QueueArgs qn = q0;
-            qn.items = dnew + g.nb;
-            qn.nitems = (int32_t)(g.ne - g.nb);
+            qn.items = ditems + g.ib;
+            qn.nitems = (int32_t)(g.ne - g.ib);
             qn.tile = g.tile;
             const cudaError_t e = lane.fp32 ? npw::launch_queue_alpha<float>(qn, ls) : npw::launch_queue_alpha<double>(qn, ls);
             if (e != cudaSuccess) return cuda_fail(e, "server alpha launch");
@@ -2298,9 +2319,9 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
         if (lane.fp32) {  // compensated float 1D items: s = u, c = 0
             for (int gi = 0; gi < kGroups; ++gi) {
                 const Group& g = grp[gi];
-                if (g.is2d || g.ne <= g.nb) continue;
-                NPW_CUDA(npw::launch_comp_begin(reinterpret_cast<const float*>(q0.u), q0.s, q0.c, q0.inst1, dnew + g.nb,
-                                                (int)(g.ne - g.nb), g.tile, g.m, ls));
+                if (g.is2d || g.ne <= g.ib) continue;
+                NPW_CUDA(npw::launch_comp_begin(reinterpret_cast<const float*>(q0.u), q0.s, q0.c, q0.inst1, ditems + g.ib,
+                                                (int)(g.ne - g.ib), g.tile, g.m, ls));
                 count_launch();
             }
         }
