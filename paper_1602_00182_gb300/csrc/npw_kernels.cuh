@@ -441,7 +441,9 @@ __device__ __forceinline__ void warp_chunk_d(int first, int cnt, bool last, int 
     const bool weno = mp.scheme == NPW_WENO_JS_ || mp.scheme == NPW_RBF_WENO_;
     const int q = first + lane;     // face on the right of cell q - 1
     const int e = min(q - 1, cnt);  // (past the line: its last neighbour)
-    const bool own = (lane < CHUNK_D || q == cnt) && face_owned(q, cnt, last);
+    // a chunk counts its first 30 faces, and the last face of the line at lane 30, where no chunk follows (lane
+    // 31 is lane 1 of the next)
+    const bool own = (lane < CHUNK_D || (lane == CHUNK_D && q == cnt)) && face_owned(q, cnt, last);
     double vm[M], vp[M], h[M], hl[M];
 #pragma unroll
     for (int k = 0; k < M; ++k) {

@@ -54,3 +54,18 @@ def test_float_lines_count_each_face_once(npw, path, n, m):
     assert s["steps"] >= 2 and _total(s) == 3 * (n + 1) * m * s["steps"]
     p.batch_mode = 1  # the per-stage kernels, whose phases count by another rule
     assert _run(npw, "batch", _line(n, m), kind, bc, 1.9 / n, p)["eta"] == s["eta"]
+
+
+# double: the work queue (tiles of 60 cells and more), the cluster (last slices of 30, 31, 32, 61 and 91
+# cells) and the per-stage kernels (a last tile of 31 and 61 cells of 1024 + .., whole lines)
+@pytest.mark.parametrize("m", [1, 3])
+@pytest.mark.parametrize("path,n,tile", [("queue", n, t) for n in (30, 31, 32, 61, 91, 121) for t in (0, 256)] +
+                         [("solve", n, 0) for n in (31, 495, 496, 497, 511, 526, 976, 1456)] +
+                         [("batch", n, t) for n in (31, 91, 1024 + 30, 1024 + 31, 1024 + 61) for t in (0, 1024)])
+def test_double_counts_are_the_oracles(npw, path, n, tile, m):
+    kind, bc = (npw.NPW_FLUX_EULER1D, 1) if m == 3 else (npw.NPW_FLUX_BURGERS, 0)
+    u0 = _line(n, m)
+    s = _run(npw, path, u0, kind, bc, 1.9 / n, npw.Params(eta_max=0.05, eta_guard=1e-3, tile_1d=tile))
+    _, ref = O.solve(u0, 1.0 / n, 1.9 / n, 0.4, kind, bc, O.Params(eta_max=0.05, eta_guard=1e-3))
+    assert s["steps"] == ref["steps"] >= 2 and _total(s) == 3 * (n + 1) * m * s["steps"]
+    assert s["eta"] == ref["eta"]
