@@ -1102,13 +1102,18 @@ __device__ __forceinline__ uint32_t face_field_any(const R* w, const MethodParam
 // characteristic variant the fields are projected by L, reconstructed, and mapped back by R.
 // T (optional, component-wise): transverse second differences [2][M] of the face's left and
 // right cells, for the k = 2 shape parameter on the 5-cell cross (Sec. 6).  eta (optional):
-// the M shape parameters of the face (characteristic: of the characteristic fields).
+// the M shape parameters of the face (characteristic: of the characteristic fields).  False where
+// the Roe state of the face is not valid: no values, flags 0.
 template <typename R, typename D, int KIND, int M, bool CHAR>
 __device__ __forceinline__ bool face_all(const R* S, const MethodParams& mp, R* vm, R* vp, uint32_t* flags,
                                          const D* T = nullptr, R* eta = nullptr) {
     if (CHAR) {
         R Rm[3][3], Lm[3][3];
-        if (!euler_eig<R>(S + 2 * M, S + 3 * M, mp_val<R>(mp.gamma, mp.gamma_f), Rm, Lm)) return false;
+        if (!euler_eig<R>(S + 2 * M, S + 3 * M, mp_val<R>(mp.gamma, mp.gamma_f), Rm, Lm)) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) flags[a] = 0u;
+            return false;
+        }
         R wm[3], wp[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {

@@ -230,7 +230,7 @@ __global__ void reconstruct_kernel(const R* __restrict__ u, int64_t n, int bc, c
     R a[M], b[M], e[M];
     uint32_t fl[M];
     bool ok = face_all<R, D, NPW_FLUX_EULER1D_, M, CHAR>(S, mp, a, b, fl, (const D*)nullptr, e);
-    if (flags) {
+    if (flags && ok) {  // (no decision was taken at a face without a valid Roe state)
         R line[M][6];
         if constexpr (CHAR) {
             R Rm[3][3], Lm[3][3];
