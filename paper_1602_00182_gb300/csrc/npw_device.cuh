@@ -255,7 +255,7 @@ __device__ __forceinline__ double cell_value_k2_d(const double* c, int side, dou
         const double p0 = row == 0 ? 0.5 : (row < 0 ? 1.5 : -0.5), p1 = row == 0 ? 0.5 : (row < 0 ? -0.5 : 1.5);
         const double far_ = ga ? -2.0 : -1.5, near_ = ga ? 0.0 : 0.5, mid = ga ? 0.5 : 0.25;
         const double q0 = row == 0 ? mid : (row < 0 ? far_ : near_), q1 = row == 0 ? mid : (row < 0 ? near_ : far_);
-        return (p0 + q0 * eta) * c[1 - q] + (p1 + q1 * eta) * c[2 - q];
+        return fma(p0 + q0 * eta, c[1 - q], 0.0) + (p1 + q1 * eta) * c[2 - q];  // (as f64::dot)
     };
     if (mp.scheme == NPW_ENO_ || mp.scheme == NPW_RBF_ENO_) return r == 0 ? cand(0) : cand(1);
     const double g0 = c[2] - c[1], g1 = c[1] - c[0];
@@ -264,7 +264,7 @@ __device__ __forceinline__ double cell_value_k2_d(const double* c, int side, dou
     x1 = x1 * x1;
     const double a0 = f64::div(side == 0 ? 2.0 / 3.0 : 1.0 / 3.0, x0), a1 = f64::div(side == 0 ? 1.0 / 3.0 : 2.0 / 3.0, x1);
     const double sum = a0 + a1;
-    return f64::div(a0, sum) * cand(0) + f64::div(a1, sum) * cand(1);
+    return fma(f64::div(a0, sum), cand(0), 0.0) + f64::div(a1, sum) * cand(1);
 }
 
 // One field at one face, k = 2.  w[0..5] = cells i-2..i+3 around face i+1/2; v^- from cell i
@@ -418,8 +418,8 @@ __device__ __forceinline__ uint32_t face_field_d(const double* w, const MethodPa
     double a[3], b[3], unused[3];
     f64::cell_weights(w, mp.eps_weno, a, unused);
     f64::cell_weights(w + 1, mp.eps_weno, unused, b);
-    *vm = (a[0] * m0 + a[1] * m1) + a[2] * m2;
-    *vp = (b[0] * p0 + b[1] * p1) + b[2] * p2;
+    *vm = f64::dot(a[0], m0, a[1], m1, a[2], m2);
+    *vp = f64::dot(b[0], p0, b[1], p1, b[2], p2);
     return fl;
 }
 

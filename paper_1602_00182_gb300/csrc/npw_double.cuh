@@ -34,10 +34,16 @@ __device__ __forceinline__ bool recip(double x, double* y) {
     *y = fma(y0, e, y0);
     return ok;
 }
-// n / x correctly rounded, y of recip(x), n 0 or in [2^-872, 2^877)
+// n / x, y of recip(x), n in [2^-872, 2^877)
 __device__ __forceinline__ double quot(double n, double x, double y) {
     const double q = n * y;
     return fma(fma(-x, q, n), y, q);
+}
+// the same with n = 0 allowed: the correction makes +0 of a -0, so the sign is taken from n y (one integer
+// instruction)
+__device__ __forceinline__ double quot0(double n, double x, double y) {
+    const double q = n * y, r = fma(fma(-x, q, n), y, q);
+    return __hiloint2double((__double2hiint(r) & 0x7FFFFFFF) | (__double2hiint(q) & (int)0x80000000), __double2loint(r));
 }
 __device__ __forceinline__ bool num_ok(double n) {
     const uint32_t h = (uint32_t)__double2hiint(n) & 0x7FFFFFFFu;
@@ -47,7 +53,7 @@ static __device__ __noinline__ double div_any(double n, double x) { return n / x
 __device__ __forceinline__ double div(double n, double x) {
     double y;
     const bool ok = recip(x, &y) & num_ok(n);
-    return ok ? quot(n, x, y) : div_any(n, x);
+    return ok ? quot0(n, x, y) : div_any(n, x);
 }
 
 // a truncated to float (0 where it is 0); *ok false outside [2^-99, 2^99)
@@ -134,8 +140,10 @@ __device__ __forceinline__ void face_coefs(double eta, int rbf, double* k) {
     k[4] = -7.0 / 6.0 + (ga ? 3.0 : 6.0) * eta;
     k[5] = 11.0 / 6.0 + (ga ? -3.0 : -4.5) * eta;
 }
+// 0 + k0 x0 + k1 x1 + k2 x2 from the left (fma(k0, x0, 0) costs what the product does; the 0 counts where every
+// product is -0)
 __device__ __forceinline__ double dot(double k0, double x0, double k1, double x1, double k2, double x2) {
-    return (k0 * x0 + k1 * x1) + k2 * x2;
+    return (fma(k0, x0, 0.0) + k1 * x1) + k2 * x2;
 }
 
 // WENO weights where a denominator leaves the range of recip, by the operator /
@@ -247,7 +255,7 @@ __device__ __forceinline__ void eta_k2_pair(double a, double b, double d, double
             const float n = to_f(num, &ok), m = to_f(den, &ok);
             if (ok && fabsf(n) * (ga ? 1.0f : 2.0f) < mp.eta_max_f * fabsf(m) * (1.0f - 0x1p-18f)) continue;
         }
-        const double q = (den_ok & num_ok(num)) ? quot(num, den, y) : div_any(num, den);
+        const double q = (den_ok & num_ok(num)) ? quot0(num, den, y) : div_any(num, den);
         double e = ga ? q : q + q;
         if (mp.has_bound && abs_above(e, mp.eta_max)) {
             *fl |= FL_ZERO_BOUND;

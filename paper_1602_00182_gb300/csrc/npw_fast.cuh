@@ -762,7 +762,7 @@ __device__ __forceinline__ void face_coefs(V eta, const FParams& fp, V* k) {
 }
 template <typename V>
 __device__ __forceinline__ V dot3(V k0, V x0, V k1, V x1, V k2, V x2) {
-    return vfma(k2, x2, vfma(k1, x1, vmul(k0, x0)));
+    return vfma(k2, x2, vfma(k1, x1, vfma(k0, x0, vset<V>(0.0f))));  // (0 + ..: three products of -0 give +0)
 }
 
 // Jiang-Shu indicators in single precision, shared by both faces of the cell, formed four times

@@ -321,7 +321,7 @@ struct DivDx {
     __device__ __forceinline__ explicit DivDx(double d) : dx(d) { ok = f64::recip(d, &y); }
     __device__ __forceinline__ double operator()(double hl, double hr) const {
         const double dh = hr - hl;
-        return -(ok & f64::num_ok(dh) ? f64::quot(dh, dx, y) : f64::div_any(dh, dx));
+        return -(ok & f64::num_ok(dh) ? f64::quot0(dh, dx, y) : f64::div_any(dh, dx));
     }
 };
 
@@ -462,8 +462,8 @@ __device__ __forceinline__ void warp_chunk_d(int first, int cnt, bool last, int 
             f64::cell_weights(c, mp.eps_weno, wm, wp);
 #pragma unroll
             for (int r = 0; r < 3; ++r) wp[r] = __shfl_down_sync(0xffffffffu, wp[r], 1);
-            vm[k] = (wm[0] * r1 + wm[1] * r2) + wm[2] * r3;
-            vp[k] = (wp[0] * r0 + wp[1] * r1) + wp[2] * r2;
+            vm[k] = f64::dot(wm[0], r1, wm[1], r2, wm[2], r3);
+            vp[k] = f64::dot(wp[0], r0, wp[1], r1, wp[2], r2);
         } else {
             const int rl = eno_choice<double>(c[0], c[1], c[2], c[3], c[4]);
             const int rr = __shfl_down_sync(0xffffffffu, rl, 1);
