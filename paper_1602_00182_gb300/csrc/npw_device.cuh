@@ -548,8 +548,11 @@ __device__ __forceinline__ bool far_from_ties(float d0, float d1, float d2, floa
 template <typename R>
 __device__ __forceinline__ bool face_near_tie(const R* wr, const MethodParams& mp, double tol) {
     if (mp.k == 3 && (mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_) && mp.guard_switch && mp.tie_tol_f <= 0x1p-14f) {
-        // a constant stencil: monotone, its denominator and eta exactly 0 against positive thresholds
-        if (wr[1] == wr[2] && wr[2] == wr[3] && wr[3] == wr[4]) return false;
+        // a constant stencil: monotone; its denominator and numerator against positive thresholds are exactly 0 in
+        // float (15 w is exact in double) and where w = 0, but round-off of 15 w and 3 w in double
+        if (wr[1] == wr[2] && wr[2] == wr[3] && wr[3] == wr[4] &&
+            (sizeof(R) == sizeof(float) || wr[1] == R(0.0) || (!mp.has_guard && !mp.has_bound)))
+            return false;
         bool ok = true;
         if constexpr (sizeof(R) == sizeof(float)) {
             const float d0 = wr[2] - wr[1], d1 = wr[3] - wr[2], d2 = wr[4] - wr[3];
