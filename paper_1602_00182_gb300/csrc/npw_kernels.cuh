@@ -621,6 +621,9 @@ __device__ __forceinline__ void warp_block_pass(int b0, int n, bool last, int la
         return r;
     };
     const int ix = min(b0 - 1 + lane, n), iy = min(b0 + 31 + lane, n);
+    // face b0 + p is counted by this block for p < 62 and p < n - b0; face n, if `last`, also at p = 62, where no
+    // block follows (at p = 63 the next block holds cell n - 1 and counts it)
+    const int own_x = n - b0 - (last ? 0 : 1), rest = own_x - 32, own_y = rest > (last ? 30 : 29) ? 29 : rest;
     float ax[M], ay[M], bx[M], by[M], hx[M], hy[M];
 #pragma unroll
     for (int k = 0; k < M; ++k) {
@@ -630,11 +633,8 @@ __device__ __forceinline__ void warp_block_pass(int b0, int n, bool last, int la
         for (int q = 0; q < 5; ++q) c[q] = F2{make_float2(X(k, ix - 2 + q), X(k, iy - 2 + q))};
         const F2 w[1][4] = {{c[1], c[2], c[3], c[4]}};
         fast::face_eta_n<F2, 1>(w, fp, eta, fl);
-        // face b0 + p, counted by this block for p < 62; face n, if `last`, also at p = 62, where no block
-        // follows (at p = 63 the next block holds cell n - 1 and counts it)
-        if (face_owned(b0 + lane, n, last)) ec.face_k3(fl[0][0]);
-        const int f = b0 + 32 + lane;
-        if ((lane < 30 || (lane == 30 && f == n)) && face_owned(f, n, last)) ec.face_k3(fl[0][1]);
+        if (lane <= own_x) ec.face_k3(fl[0][0]);
+        if (lane <= own_y) ec.face_k3(fl[0][1]);
         fast::cell_recon<F2>(c, eta[0], before(eta[0]), fp, &vm, &vp);
         const F2 vl = before(vm);
         ax[k] = vl.v.x;
