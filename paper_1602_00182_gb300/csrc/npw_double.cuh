@@ -4,11 +4,11 @@
 // The FP64 pipe of GB300 takes a warp instruction every 16 cycles per SM: one costs as much issue time
 // as 64 float or integer ones, and comparisons count like adds.  So:
 //   * A quotient n / x is the Markstein iteration (P. Markstein, IBM J. Res. Dev. 34(1), 1990): y
-//     from the float reciprocal of x (2^-22) by one cubic step, within about one ulp of 1 / x; q0 =
-//     n y; q = q0 + (n - x q0) y with both operations fused, which is the correctly rounded quotient.
-//     x y and n - x q0 are exact to the last bit that matters because x lies in [2^-99, 2^99) and n is 0
-//     or in [2^-872, 2^877); elsewhere the operator / is called, out of line.  Quotients with one
-//     denominator share y: 3 FP64 instructions each after 3 for y, against about 9 for the operator.
+//     from the float reciprocal of x (2^-22) by one cubic step, nearly always 1 / x correctly rounded;
+//     q0 = n y; q = q0 + (n - x q0) y with both operations fused, which is the correctly rounded quotient
+//     but for divisors just below a power of two (see recip).  n - x q0 is exact because x lies in [2^-99,
+//     2^99) and n is 0 or in [2^-872, 2^877).  Elsewhere the operator / is called, out of line.  Quotients
+//     with one denominator share y: 3 FP64 instructions each after 3 for y, against about 9 for the operator.
 //   * 2 c and 4 c and x / 4 are exact, so their products join the following sum in one fused
 //     instruction that rounds as the sum alone.
 //   * The monotone switch is decided in float from the exact-to-53-bits differences, with bounds that
@@ -24,8 +24,8 @@
 namespace npw {
 namespace f64 {
 
-// y ~ 1 / x within about one ulp; false where x is outside [2^-99, 2^99) in magnitude
-__device__ __forceinline__ bool recip(double x, double* y) {
+// y ~ 1 / x for the quotients below; false where x is outside [2^-99, 2^99) in magnitude
+__device__ __forceinline__ bool recip_near(double x, double* y) {
     float xf;
     const bool ok = fast::seed_f(x, &xf);
     const double y0 = fast::widen_nz(fast::rcp_fast(xf));
@@ -34,6 +34,21 @@ __device__ __forceinline__ bool recip(double x, double* y) {
     *y = fma(y0, e, y0);
     return ok;
 }
+// x whose mantissa begins with 13 ones, where the quotient with that y may be rounded wrongly.  With X, N the 53-bit
+// integer mantissas, n / x lies c / (2 X) ulp from a rounding boundary, c a nonzero integer, and the quotient
+// before its last rounding within |d eta| X 2^-105 ulp of n / x, d the error of n y rounded and eta that of y,
+// both in ulps.  With d = 1/2 (at a boundary) a wrong rounding takes eta >= (2^53 / X)^2 / 2, and d = 3/2 takes
+// eta N > 2^52 with N < X.  A correctly rounded y gives neither (Markstein's theorem); the cubic step leaves
+// eta < 1/2 + 2^-15 for x near 2 (|1 - x y0| < 1.5 2^-23 there, cubed, and the last rounding), hence no wrong
+// quotient below X = 2^53 (1 - 2^-14).
+__device__ __forceinline__ bool hard(double x) { return (~(uint32_t)__double2hiint(x) & 0x000FFF80u) == 0u; }
+// one Newton step: y correctly rounded, but where the mantissa of x is all ones (false)
+__device__ __forceinline__ bool refine(double x, double* y) {
+    *y = fma(fma(-x, *y, 1.0), *y, *y);
+    return ((~(uint32_t)__double2hiint(x) & 0x000FFFFFu) | ~(uint32_t)__double2loint(x)) != 0u;
+}
+// 1 / x for quot: false outside the range and for hard x
+__device__ __forceinline__ bool recip(double x, double* y) { return recip_near(x, y) & !hard(x); }
 // n / x, y of recip(x), n in [2^-872, 2^877)
 __device__ __forceinline__ double quot(double n, double x, double y) {
     const double q = n * y;
@@ -146,8 +161,33 @@ __device__ __forceinline__ double dot(double k0, double x0, double k1, double x1
     return (fma(k0, x0, 0.0) + k1 * x1) + k2 * x2;
 }
 
-// WENO weights where a denominator leaves the range of recip, by the operator /
+// WENO weights alpha_r / sum alpha of both sides from the squared denominators; false where a quotient
+// may be wrong: outside the range of recip, or (REFINED: the mantissa all ones) for a hard sum.  The first
+// quotients take any x: their dividends are the constants 0.1 and 0.3 (0.6), and a wrong one takes c = +-1, an X
+// in the hard range that divides 2^53 N -+ 1 or 2^54 N -+ 1; none of these eight integers has a divisor there.
+template <bool REFINED>
+__device__ __forceinline__ bool weights_from(double x0, double x1, double x2, double wm[3], double wp[3]) {
+    auto inv = [](double x, double* y) { return recip_near(x, y) & (REFINED ? refine(x, y) : !hard(x)); };
+    double y0, y1, y2, ym, yp;
+    bool ok = recip_near(x0, &y0);
+    ok = recip_near(x1, &y1) & ok;
+    ok = recip_near(x2, &y2) & ok;
+    const double am0 = quot(0.3, x0, y0), ap0 = quot(0.1, x0, y0), a6 = quot(0.6, x1, y1), am2 = quot(0.1, x2, y2),
+                 ap2 = quot(0.3, x2, y2);
+    const double sm = (am0 + a6) + am2, sp = (ap0 + a6) + ap2;
+    ok = inv(sm, &ym) & ok;
+    ok = inv(sp, &yp) & ok;
+    wm[0] = quot(am0, sm, ym);
+    wm[1] = quot(a6, sm, ym);
+    wm[2] = quot(am2, sm, ym);
+    wp[0] = quot(ap0, sp, yp);
+    wp[1] = quot(a6, sp, yp);
+    wp[2] = quot(ap2, sp, yp);
+    return ok;
+}
+// the rest, out of line: refined reciprocals (one cell in 4000 has a hard sum), else the operator /
 static __device__ __noinline__ void weights_any(double x0, double x1, double x2, double wm[3], double wp[3]) {
+    if (weights_from<true>(x0, x1, x2, wm, wp)) return;
     const double am[3] = {0.3 / x0, 0.6 / x1, 0.1 / x2}, ap[3] = {0.1 / x0, 0.6 / x1, 0.3 / x2};
     const double sm = (am[0] + am[1]) + am[2], sp = (ap[0] + ap[1]) + ap[2];
     for (int r = 0; r < 3; ++r) {
@@ -169,23 +209,7 @@ __device__ __forceinline__ void cell_weights(const double* c, double eps_weno, d
     x0 = x0 * x0;
     x1 = x1 * x1;
     x2 = x2 * x2;
-    double y0, y1, y2;
-    bool ok = recip(x0, &y0);
-    ok = recip(x1, &y1) & ok;
-    ok = recip(x2, &y2) & ok;
-    const double am0 = quot(0.3, x0, y0), ap0 = quot(0.1, x0, y0), a6 = quot(0.6, x1, y1), am2 = quot(0.1, x2, y2),
-                 ap2 = quot(0.3, x2, y2);
-    const double sm = (am0 + a6) + am2, sp = (ap0 + a6) + ap2;
-    double ym, yp;
-    ok = recip(sm, &ym) & ok;
-    ok = recip(sp, &yp) & ok;
-    wm[0] = quot(am0, sm, ym);
-    wm[1] = quot(a6, sm, ym);
-    wm[2] = quot(am2, sm, ym);
-    wp[0] = quot(ap0, sp, yp);
-    wp[1] = quot(a6, sp, yp);
-    wp[2] = quot(ap2, sp, yp);
-    if (__builtin_expect(!ok, 0)) {
+    if (__builtin_expect(!weights_from<false>(x0, x1, x2, wm, wp), 0)) {
         double m[3], p[3];
         weights_any(x0, x1, x2, m, p);
         for (int r = 0; r < 3; ++r) {
