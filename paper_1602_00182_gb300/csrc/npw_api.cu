@@ -725,12 +725,17 @@ void fill_stats(const npw::Ctl& c, npw_solve_stats* o) {
     o->eta_bound = (int64_t)c.n_bound;
 }
 
-npw_status collect_stats(const Run1D& r, npw_solve_stats* out) {
-    std::vector<npw::Ctl> hc(r.count);
+// the control words after everything launched so far (a bounded wait)
+npw_status read_ctl(const Run1D& r, std::vector<npw::Ctl>& hc) {
+    hc.resize(r.count);
     npw_status st = bounded_sync(r.s);  // before the (blocking) copy into pageable memory
     if (st) return st;
     NPW_CUDA(cudaMemcpyAsync(hc.data(), r.ws + r.L.ctl, sizeof(npw::Ctl) * r.count, cudaMemcpyDeviceToHost, r.s));
     profile_collect();
+    return NPW_OK;
+}
+
+npw_status stats_of(const Run1D& r, const std::vector<npw::Ctl>& hc, npw_solve_stats* out) {
     npw_status first = NPW_OK;
     for (int i = 0; i < r.count; ++i) {
         if (out) fill_stats(hc[i], &out[i]);
@@ -739,6 +744,12 @@ npw_status collect_stats(const Run1D& r, npw_solve_stats* out) {
     if (first == NPW_ENONFINITE) return fail(first, "an instance became non-finite");
     if (first != NPW_OK) return fail(first, "an instance reached its step limit or stopped advancing");
     return NPW_OK;
+}
+
+npw_status collect_stats(const Run1D& r, npw_solve_stats* out) {
+    std::vector<npw::Ctl> hc;
+    npw_status st = read_ctl(r, hc);
+    return st ? st : stats_of(r, hc, out);
 }
 
 // Library-owned side streams (created once per device) for the resident launches.
@@ -927,13 +938,17 @@ npw_status replay_steps(const Run1D& r, const StepGraph& g, long long graphs) {
     return NPW_OK;
 }
 
+// most steps launched before the host waits for them: the wait limit covers these, not the whole solve, and no
+// more than these are still queued when it runs out
+constexpr int POLL_STEPS = 256;
+
 npw_status run_to_end(Run1D& r, npw_solve_stats* out) {
     long long act = 0, rem = 0;
     npw_status st = poll(r, &act, &rem);
     StepGraph graph;
     bool direct_done = false;
     while (st == NPW_OK && act > 0) {
-        long long chunk = rem < 1 ? 1 : (rem > 256 ? 256 : rem);
+        long long chunk = rem < 1 ? 1 : (rem > POLL_STEPS ? POLL_STEPS : rem);
         // long chunks replay the captured graph (after one direct step has set up the kernels'
         // attributes); the remainder, and short runs, launch directly
         if (chunk > GRAPH_STEPS && direct_done) {
@@ -1107,8 +1122,10 @@ static npw_status single_run(void* u, int64_t n, int32_t m, double dx, double t_
 }  // extern "C"
 namespace {
 int cluster_ctas(const npw_params* p, int64_t n, int m);
-// the run of r by one cluster of ctas CTAs: a solve of `in`, or (single_step) one step of dt
-npw_status cluster_run(const Run1D& r, const npw_instance& in, int ctas, int single_step, double dt, bool* fits) {
+// one launch of a cluster of ctas CTAs: one step of dt (single_step), or the first or the next (resume) POLL_STEPS
+// steps of a solve of `in`
+npw_status cluster_run(const Run1D& r, const npw_instance& in, int ctas, int single_step, double dt, bool resume,
+                       bool* fits) {
     npw::ResidentArgs a{};
     a.arena = r.arena;
     a.carry = reinterpret_cast<float*>(r.ws + r.L.cbuf);
@@ -1118,6 +1135,8 @@ npw_status cluster_run(const Run1D& r, const npw_instance& in, int ctas, int sin
     a.one = npw::InstDev{0, in.n, in.dx, in.t_end, in.cfl, in.bc, 0};
     a.dt_fixed = dt;
     a.single_step = single_step;
+    a.resume = resume;
+    a.launch_steps = POLL_STEPS;
     auto ev = stage_begin(r.s);
     const cudaError_t e = r.fp32 ? npw::launch_cluster<float>(a, r.kind, in.n, ctas, r.s, fits)
                                  : npw::launch_cluster<double>(a, r.kind, in.n, ctas, r.s, fits);
@@ -1138,7 +1157,7 @@ npw_status npweno_rk3_step(void* u, int64_t n, int32_t m, double dx, double dt, 
     if (!(dt >= 0.0)) return fail(NPW_EINVAL, "dt must be >= 0");
     bool whole = false;
     if (const int ctas = cluster_ctas(params, n, m)) {
-        if ((st = cluster_run(r, in, ctas, 1, dt, &whole))) return st;
+        if ((st = cluster_run(r, in, ctas, 1, dt, false, &whole))) return st;
     }
     if (!whole) {
         if ((st = setup_1d(r, &in, 1, dt, 2))) return st;
@@ -1186,8 +1205,13 @@ npw_status npweno_solve(void* u, int64_t n, int32_t m, double dx, double t_end, 
     if (!(cfl > 0.0)) return fail(NPW_EINVAL, "cfl must be > 0");
     if (const int ctas = cluster_ctas(params, n, m)) {
         bool fits = false;
-        if ((st = cluster_run(r, in, ctas, 0, 0.0, &fits))) return st;
-        if (fits) return collect_stats(r, out);
+        std::vector<npw::Ctl> hc;
+        if ((st = cluster_run(r, in, ctas, 0, 0.0, false, &fits))) return st;
+        while (fits) {
+            if ((st = read_ctl(r, hc))) return st;
+            if (hc[0].done) return stats_of(r, hc, out);
+            if ((st = cluster_run(r, in, ctas, 0, 0.0, true, &fits))) return st;
+        }
     }
     if ((st = setup_1d(r, &in, 1, 0.0, 1))) return st;
     return run_to_end(r, out);

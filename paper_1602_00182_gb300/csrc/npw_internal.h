@@ -201,10 +201,12 @@ struct ResidentArgs {
     const int32_t* list;     // instance indices handled by this launch, one per CTA
     int32_t count;
     MethodParams mp;
-    // solve1d_cluster_kernel: its one line, and a single step of dt_fixed instead of a solve
+    // solve1d_cluster_kernel: its one line; a single step of dt_fixed instead of a solve; the most steps of this
+    // launch, and whether it continues the run that the control word holds
     InstDev one;
     double dt_fixed;
-    int32_t single_step;
+    int32_t single_step, resume;
+    int32_t launch_steps;
 };
 
 struct Stage2DArgs {

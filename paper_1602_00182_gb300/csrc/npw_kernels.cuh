@@ -1406,9 +1406,11 @@ __global__ void __launch_bounds__(K == 3 ? 512 : 1024) solve1d_resident_kernel(R
 // cells on each side.  A boundary cell is stored into the neighbour's ghost cells as well, through
 // distributed shared memory, and one cluster barrier ends each stage.  In the last stage every CTA
 // also stores its largest wave speed into a slot of every other, so that each advances t, alpha and dt
-// by itself to the same values.  Float: the increment form of the resident kernel (un, d1 / new state,
-// d2; carry in global memory); double: the Shu-Osher form of the per-stage kernel (un, u1, u2).  The
-// arithmetic per cell is theirs, so the results are the same bits.
+// by itself to the same values.  A launch takes at most launch_steps steps, so that the host's wait for it
+// is bounded; the next one (resume) goes on from the control word, the arena and the carry.  Float: the
+// increment form of the resident kernel (un, d1 / new state, d2; carry in global memory); double: the
+// Shu-Osher form of the per-stage kernel (un, u1, u2).  The arithmetic per cell is theirs, so the results are
+// the same bits.
 // For a single instance this replaces three launches per step, each with too few cells to fill the
 // GPU, by three barriers of a microsecond or less; it uses 16 SMs, so long lines stay with the
 // per-stage kernels (see cluster_ctas).
@@ -1475,7 +1477,7 @@ __global__ void __launch_bounds__(512) solve1d_cluster_kernel(ResidentArgs a) {
 #pragma unroll
         for (int k = 0; k < M; ++k) {
             un[k * NS + RES_GHOST + i] = c < 0 ? inflow[k] : g[(int64_t)k * n + c];
-            if (F32 && i >= 0 && i < cnt) cr[(int64_t)k * n + s0 + i] = 0.0f;
+            if (F32 && !a.resume && i >= 0 && i < cnt) cr[(int64_t)k * n + s0 + i] = 0.0f;
         }
     }
     const fast::FParams fp = fast::fparams(a.mp);
@@ -1531,9 +1533,23 @@ __global__ void __launch_bounds__(512) solve1d_cluster_kernel(ResidentArgs a) {
         s_alpha = alpha;
         s_dt = dt;
     };
-    if (rank == 0 && threadIdx.x == 0) memset(ctl, 0, sizeof(Ctl));
-    cluster.sync();  // every CTA of the cluster has started: its shared memory may be written
-    {
+    if (threadIdx.x == 0 && a.resume) {
+        t = ctl->t;
+        dt = ctl->dt;
+        alpha = ctl->alpha;
+        alpha_max = ctl->alpha_max;
+        steps = ctl->steps;
+        cap = ctl->step_cap;
+        last = ctl->last;
+        s_lam = (float)(dt / in.dx);
+        s_alpha = alpha;
+        s_dt = dt;
+        s_done = 0;
+    } else if (rank == 0 && threadIdx.x == 0) {
+        memset(ctl, 0, sizeof(Ctl));
+    }
+    cluster.sync();  // every CTA of the cluster has started (its shared memory may be written) and read ctl
+    if (!a.resume) {
         const double b = line_max();
         if (threadIdx.x == 0) {
             s_done = 0;
@@ -1557,7 +1573,8 @@ __global__ void __launch_bounds__(512) solve1d_cluster_kernel(ResidentArgs a) {
         __syncthreads();
     }
     const DivDx dxq(F32 ? 1.0 : in.dx);
-    while (!s_done) {
+#pragma unroll 1
+    for (int taken = 0; taken < a.launch_steps && !s_done; ++taken) {
         const float lam = s_lam;
         const R alphaR = R(s_alpha), dtR = R(s_dt);
         vmax = R(0.0);
@@ -1673,7 +1690,9 @@ __global__ void __launch_bounds__(512) solve1d_cluster_kernel(ResidentArgs a) {
         ctl->alpha_max = alpha_max;
         ctl->steps = steps;
         ctl->status = status;
-        ctl->done = 1;
+        ctl->step_cap = cap;
+        ctl->last = last;
+        ctl->done = a.single_step || s_done;
     }
 }
 
