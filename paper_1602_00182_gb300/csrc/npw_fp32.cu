@@ -16,12 +16,8 @@ static cudaError_t launch_res(const ResidentArgs& a, int64_t max_n, int threads,
     constexpr int M = kind_m<KIND>();
     const size_t smem = resident_smem_bytes(max_n, M);
     auto kern = solve1d_resident_kernel<KIND, K>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RESIDENT_SMEM_MAX);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    const cudaError_t e = allow_smem<solve1d_resident_kernel<KIND, K>>(RESIDENT_SMEM_MAX);
+    if (e != cudaSuccess) return e;
     kern<<<a.count, threads, smem, s>>>(a);
     return cudaGetLastError();
 }

@@ -11,12 +11,12 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <mutex>
 #include <type_traits>
 
 #include "npw_device.cuh"
 #include "npw_fast.cuh"
 #include "npw_internal.h"
+#include "npw_per_device.h"
 
 namespace npw {
 
@@ -1696,6 +1696,13 @@ __global__ void __launch_bounds__(512) solve1d_cluster_kernel(ResidentArgs a) {
     }
 }
 
+// dynamic shared memory of up to `bytes` for a kernel, on the current device
+template <auto KERNEL>
+cudaError_t allow_smem(size_t bytes) {
+    static PerDevice<bool> set;
+    return set.once([&] { return cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); });
+}
+
 // bytes of shared memory of a slice of `per` cells
 template <typename R>
 constexpr size_t cluster_smem(int64_t per, int m) {
@@ -1719,17 +1726,15 @@ cudaError_t launch_cluster_k(const ResidentArgs& a, int64_t n, int ctas, cudaStr
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     // the attributes, and whether the largest slice's cluster of this size fits, once per device
-    static std::mutex mu;
-    static signed char known[64][MAX_CLUSTER + 1];  // 0 not asked, 1 fits, -1 does not
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || ctas > MAX_CLUSTER) return cudaErrorInvalidValue;
-    {
-        std::lock_guard<std::mutex> g(mu);
-        signed char& k = known[dev][ctas];
+    if (ctas > MAX_CLUSTER) return cudaErrorInvalidValue;
+    struct Known {
+        signed char of[MAX_CLUSTER + 1] = {};  // 0 not asked, 1 fits, -1 does not
+    };
+    static PerDevice<Known> known;
+    const cudaError_t asked = known.with([&](Known& v) {
+        signed char& k = v.of[ctas];
         if (k == 0) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RESIDENT_SMEM_MAX);
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RESIDENT_SMEM_MAX);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             int clusters = 0;
             cudaLaunchConfig_t most = cfg;
@@ -1740,7 +1745,9 @@ cudaError_t launch_cluster_k(const ResidentArgs& a, int64_t n, int ctas, cudaStr
             k = clusters > 0 ? 1 : -1;
         }
         *fits = k > 0;
-    }
+        return cudaSuccess;
+    });
+    if (asked != cudaSuccess) return asked;
     return *fits ? cudaLaunchKernelEx(&cfg, kern, a) : cudaSuccess;
 }
 template <typename R>
@@ -2860,23 +2867,15 @@ struct Launchers {
         constexpr int M = kind_m<KIND>();
         if constexpr (sizeof(R) == sizeof(double) && !CHAR && K == 3) {
             auto kern = stage1d_double_kernel<KIND>;
-            static bool attr_set = false;
-            if (!attr_set) {
-                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
-                if (e != cudaSuccess) return e;
-                attr_set = true;
-            }
+            const cudaError_t e = allow_smem<stage1d_double_kernel<KIND>>(80 * 1024);
+            if (e != cudaSuccess) return e;
             const int chunks = (a.tile + CHUNK_D - 1) / CHUNK_D;
             kern<<<a.ntiles, cta_threads(chunks * 32), (size_t)(a.tile + 6) * M * sizeof(R), s>>>(a);
         } else if constexpr (sizeof(R) == sizeof(double) || CHAR) {
             const size_t smem = (size_t)((a.tile + 6) + (a.tile + 1)) * M * sizeof(R);
             auto kern = stage1d_kernel<R, D, KIND, CHAR, K>;
-            static bool attr_set = false;
-            if (!attr_set) {
-                cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-                if (e != cudaSuccess) return e;
-                attr_set = true;
-            }
+            const cudaError_t e = allow_smem<stage1d_kernel<R, D, KIND, CHAR, K>>(160 * 1024);
+            if (e != cudaSuccess) return e;
             kern<<<a.ntiles, cta_threads(a.tile + 1), smem, s>>>(a);
         } else {
             return cudaErrorInvalidValue;  // float, component-wise: stage_fast
@@ -2892,12 +2891,8 @@ struct Launchers {
         constexpr int M = kind_m<KIND>();
         const size_t smem = (size_t)(a.tile + 6) * 4 * M * sizeof(float);
         auto kern = stage1d_fast_kernel<KIND, K>;
-        static bool attr_set = false;
-        if (!attr_set) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-            if (e != cudaSuccess) return e;
-            attr_set = true;
-        }
+        const cudaError_t e = allow_smem<stage1d_fast_kernel<KIND, K>>(160 * 1024);
+        if (e != cudaSuccess) return e;
         kern<<<a.ntiles, cta_threads((a.tile + 3) * M), smem, s>>>(a);
         return cudaGetLastError();
     }
@@ -2976,14 +2971,13 @@ struct Launchers {
                     stage2d_warp_kernel<NPW_FLUX_BURGERS_><<<tiles, THREADS_1D, stage2d_warp_smem_floats<1>() * sizeof(float), s>>>(a);
                     break;
                 case NPW_FLUX_EULER2D * 4 + 3: {
-                    static bool carveout = false;  // four CTAs of 45 KB an SM
-                    if (!carveout) {
-                        const cudaError_t e = cudaFuncSetAttribute(stage2d_warp_kernel<NPW_FLUX_EULER2D_>,
-                                                                   cudaFuncAttributePreferredSharedMemoryCarveout,
-                                                                   (int)cudaSharedmemCarveoutMaxShared);
-                        if (e != cudaSuccess) return e;
-                        carveout = true;
-                    }
+                    static PerDevice<bool> carveout;  // four CTAs of 45 KB an SM
+                    const cudaError_t e = carveout.once([] {
+                        return cudaFuncSetAttribute(stage2d_warp_kernel<NPW_FLUX_EULER2D_>,
+                                                    cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                    (int)cudaSharedmemCarveoutMaxShared);
+                    });
+                    if (e != cudaSuccess) return e;
                     stage2d_warp_kernel<NPW_FLUX_EULER2D_><<<tiles, THREADS_1D, stage2d_warp_smem_floats<4>() * sizeof(float), s>>>(a);
                     break;
                 }
