@@ -1810,8 +1810,8 @@ __device__ __forceinline__ float halo_get(const float* u, const Inst2D& in, int 
 // 2D stage kernel of the mixed path, k = 2 (float state, component-wise) in phases, each a balanced
 // loop over independent work items:
 //   C  reconstruction of every (cell, field) of both directions: v^- at its right / upper face
-//      and v^+ at its left / lower face, one set of smoothness indicators for both (k = 2: the
-//      cell's own switch and shape parameters, with the transverse term of the 5-cell cross)
+//      and v^+ at its left / lower face, one set of smoothness indicators for both, with the cell's
+//      own switch and shape parameters (and the transverse term of the 5-cell cross)
 //   F  Lax-Friedrichs flux of every face (all fields)
 //   U  flux difference and Shu-Osher stage combination of every cell
 // Every face value gets the arithmetic of fast::face_field, so the result is the same as the
@@ -1825,7 +1825,7 @@ __host__ __device__ constexpr int stage2d_fast_smem_floats() {
 }
 
 // One tile (index `tile` of the instance's tiles_x x tiles_y tiles) of one stage.
-template <int KIND, int K>
+template <int KIND>
 __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const Inst2D& in, Ctl* ctl, int tile,
                                                   float* smem) {
     constexpr int M = kind_m<KIND>();
@@ -1833,11 +1833,11 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
     constexpr int NFX = (TX_2D + 1) * TY_2D;  // x faces: (qx, qy), qx = 0..TX between cells qx-1, qx
     constexpr int NFY = TX_2D * (TY_2D + 1);  // y faces: (qx, qy), qy = 0..TY
     constexpr int NF = NFX + NFY;
-    // field-major layout: su[k][by][bx], and ef, vmf, vpf [k][face] (x faces, then y faces), so
+    // field-major layout: su[k][by][bx], and hf, vmf, vpf [k][face] (x faces, then y faces), so
     // that consecutive threads (consecutive cells or faces of one field) hit consecutive banks
     float* su = smem;                          // [BY * BX * M]
-    float* ef = su + BY * BX * M;              // [M][NF] eta per (field, face); then the fluxes
-    float* vmf = ef + NF * M;                  // v^- per (field, face)
+    float* hf = su + BY * BX * M;              // [M][NF] flux per (field, face)
+    float* vmf = hf + NF * M;                  // v^- per (field, face)
     float* vpf = vmf + NF * M;                 // v^+ per (field, face)
     __shared__ float red[32];
     __shared__ int redbad[32];
@@ -1851,7 +1851,7 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
     const float* uin = reinterpret_cast<const float*>(a.uin) + in.off;
     const int tid = threadIdx.x, nthr = blockDim.x;
     const fast::FParams fp = fast::fparams(a.mp);
-    const bool cross = K == 2 && a.mp.cross_2d && (a.mp.scheme == NPW_RBF_ENO_ || a.mp.scheme == NPW_RBF_WENO_);
+    const bool cross = a.mp.cross_2d && (a.mp.scheme == NPW_RBF_ENO_ || a.mp.scheme == NPW_RBF_WENO_);
     // the field index is a compile-time constant in each loop (an indexed parameter array would
     // put the stage arguments in local memory)
 #pragma unroll
@@ -1881,47 +1881,20 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
     auto own_x = [=](int qx, int qy) { return qy < rows_in && face_owned(qx, cols_in, last_x); };
     auto own_y = [=](int qx, int qy) { return qx < cols_in && face_owned(qy, rows_in, last_y); };
 #define NPW_SU(bx, by, k) su[((k) * BY + (by)) * BX + (bx)]
-    // E: item = (face, field); x face (qx, qy) has the eta stencil su[qy+3][qx+1 .. qx+4],
-    // y face (qx, qy) su[qy+1 .. qy+4][qx+3]
-    for (int it = tid; K == 3 && it < NF * M; it += nthr) {
-        const int k = it / NF, f = it - k * NF;
-        float w0, w1, w2, w3;
-        bool own;
-        if (f < NFX) {
-            const int qy = f / (TX_2D + 1), qx = f - qy * (TX_2D + 1);
-            w0 = NPW_SU(qx + 1, qy + 3, k);
-            w1 = NPW_SU(qx + 2, qy + 3, k);
-            w2 = NPW_SU(qx + 3, qy + 3, k);
-            w3 = NPW_SU(qx + 4, qy + 3, k);
-            own = own_x(qx, qy);
-        } else {
-            const int g = f - NFX;
-            const int qy = g / TX_2D, qx = g - qy * TX_2D;
-            w0 = NPW_SU(qx + 3, qy + 1, k);
-            w1 = NPW_SU(qx + 3, qy + 2, k);
-            w2 = NPW_SU(qx + 3, qy + 3, k);
-            w3 = NPW_SU(qx + 3, qy + 4, k);
-            own = own_y(qx, qy);
-        }
-        uint32_t fl = 0;
-        ef[k * NF + f] = fast::face_eta(w0, w1, w2, w3, fp, &fl);
-        if (own) ec.face_k3(fl);
-    }
-    __syncthreads();
     // C: item = (cell, field); x: cells cx = -1..TX of each row (TX + 2 per row), y: cells
     // cy = -1..TY of each column.  Cell -1 only gives v^- at face 0, cell TX (TY) only v^+ at the
     // last face.
     constexpr int NCX = (TX_2D + 2) * TY_2D, NCY = TX_2D * (TY_2D + 2);
     for (int it = tid; it < (NCX + NCY) * M; it += nthr) {
         const int k = it / (NCX + NCY), c = it - k * (NCX + NCY);
-        float cc[5];
-        double trans = 0.0;  // k = 2 cross: transverse second difference of the cell
+        float cc[3];
+        double trans = 0.0;  // cross: transverse second difference of the cell
         int fl_idx, fr_idx;  // faces left / right of the cell (-1 when outside the tile)
         bool own_l, own_r;   // those faces are counted by this tile
         if (c < NCX) {
             const int qy = c / (TX_2D + 2), cx = c - qy * (TX_2D + 2) - 1;
 #pragma unroll
-            for (int j = 0; j < 5; ++j) cc[j] = NPW_SU(cx + 1 + j, qy + 3, k);
+            for (int j = 0; j < 3; ++j) cc[j] = NPW_SU(cx + 2 + j, qy + 3, k);
             fl_idx = cx >= 0 ? qy * (TX_2D + 1) + cx : -1;
             fr_idx = cx < TX_2D ? qy * (TX_2D + 1) + cx + 1 : -1;
             own_l = cx >= 0 && own_x(cx, qy);
@@ -1935,7 +1908,7 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
             const int g = c - NCX;
             const int cy = g / TX_2D - 1, qx = g - (cy + 1) * TX_2D;
 #pragma unroll
-            for (int j = 0; j < 5; ++j) cc[j] = NPW_SU(qx + 3, cy + 1 + j, k);
+            for (int j = 0; j < 3; ++j) cc[j] = NPW_SU(qx + 3, cy + 2 + j, k);
             fl_idx = cy >= 0 ? NFX + cy * TX_2D + qx : -1;
             fr_idx = cy < TY_2D ? NFX + (cy + 1) * TX_2D + qx : -1;
             own_l = cy >= 0 && own_y(qx, cy);
@@ -1945,21 +1918,15 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
                         fast::widen(NPW_SU(qx + 4, cy + 3, k));
         }
         float vm, vp;
-        if constexpr (K == 3) {
-            const float er = fr_idx >= 0 ? ef[k * NF + fr_idx] : 0.0f;
-            const float el = fl_idx >= 0 ? ef[k * NF + fl_idx] : 0.0f;
-            fast::cell_recon(cc, er, el, fp, &vm, &vp);
-        } else {
-            const uint32_t d = fast::cell_recon_k2(cc + 1, trans, a.mp, fp, &vm, &vp);
-            if (own_r) fast::count_k2(ec, d, 0);
-            if (own_l) fast::count_k2(ec, d, 1);
-        }
+        const uint32_t d = fast::cell_recon_k2(cc, trans, a.mp, fp, &vm, &vp);
+        if (own_r) fast::count_k2(ec, d, 0);
+        if (own_l) fast::count_k2(ec, d, 1);
         if (fr_idx >= 0) vmf[k * NF + fr_idx] = vm;
         if (fl_idx >= 0) vpf[k * NF + fl_idx] = vp;
     }
     flush_counts(ec, ctl, a.mp);
     __syncthreads();
-    // F: item = face (all fields); the fluxes overwrite the eta array
+    // F: item = face (all fields)
     for (int f = tid; f < NFX + NFY; f += nthr) {
         float vm[M], vp[M], h[M];
 #pragma unroll
@@ -1972,7 +1939,7 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
         else
             lf_flux<float, KIND, M>(vm, vp, ay, a.mp, 1, h);
 #pragma unroll
-        for (int k = 0; k < M; ++k) ef[k * NF + f] = h[k];
+        for (int k = 0; k < M; ++k) hf[k * NF + f] = h[k];
     }
     __syncthreads();
 #undef NPW_SU
@@ -1991,7 +1958,7 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
         float U[M];
 #pragma unroll
         for (int k = 0; k < M; ++k) {
-            const float* hx = ef + k * NF;
+            const float* hx = hf + k * NF;
             const float* hy = hx + NFX;
             float L = -((hx[qy * (TX_2D + 1) + qx + 1] - hx[qy * (TX_2D + 1) + qx]) * idxR);
             L = L - (hy[(qy + 1) * TX_2D + qx] - hy[qy * TX_2D + qx]) * idyR;
@@ -2034,9 +2001,9 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
 }
 
 // ---------------------------------------------------------------------------------------
-// 2D stage of the mixed path, k = 3 (float state, component-wise), in warp tasks.  The phases are
-// those of stage2d_fast_body (eta of every face; reconstruction of every cell, both directions; flux;
-// update), but a task is one row of the tile and one pair of fields, a lane one face, cell or column
+// 2D stage of the mixed path, k = 3 (float state, component-wise), in warp tasks.  Phases: eta of every
+// face; reconstruction of every cell, both directions; flux; update.  A task is one row of the tile and one
+// pair of fields, a lane one face, cell or column
 // of it: TX_WARP + 2 = 32 cells of a row fill the lanes, and with TY_WARP = 11 the 46, 48, 23 and 11
 // tasks of the phases (2D Euler) leave the eight warps nearly even.  A task's addresses are then a
 // lane offset from a row, where the flat loop over (face, field) spent as much on indices as on the
@@ -2555,10 +2522,10 @@ __global__ void __launch_bounds__(THREADS_1D) stage1d_fast_kernel(Stage1DArgs a)
     stage1d_fast_body<KIND, K>(a, td, a.inst[td.inst], a.ctl + td.inst, smem_raw);
 }
 
-template <int KIND, int K>
+template <int KIND>
 __global__ void __launch_bounds__(TX_2D * TY_2D) stage2d_fast_kernel(Stage2DArgs a) {
     extern __shared__ __align__(16) float smem_f[];
-    stage2d_fast_body<KIND, K>(a, *a.inst, a.ctl, blockIdx.x, smem_f);
+    stage2d_fast_body<KIND>(a, *a.inst, a.ctl, blockIdx.x, smem_f);
 }
 
 template <int KIND>
@@ -2604,7 +2571,7 @@ __device__ __forceinline__ void queue_item_2d(const Stage2DArgs& a2, const Inst2
     if constexpr (warp_tiles_2d(sizeof(R) == sizeof(float), K))
         stage2d_warp_body<KIND>(a2, in, ctl, tile, reinterpret_cast<float*>(smem));
     else if constexpr (sizeof(R) == sizeof(float))
-        stage2d_fast_body<KIND, K>(a2, in, ctl, tile, reinterpret_cast<float*>(smem));
+        stage2d_fast_body<KIND>(a2, in, ctl, tile, reinterpret_cast<float*>(smem));
     else
         stage2d_body<R, double, KIND, K>(a2, in, ctl, tile, smem);
 }
@@ -2982,13 +2949,13 @@ struct Launchers {
                     break;
                 }
                 case NPW_FLUX_ADVECTION * 4 + 2:
-                    stage2d_fast_kernel<NPW_FLUX_ADVECTION_, 2><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<1>() * sizeof(float), s>>>(a);
+                    stage2d_fast_kernel<NPW_FLUX_ADVECTION_><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<1>() * sizeof(float), s>>>(a);
                     break;
                 case NPW_FLUX_BURGERS * 4 + 2:
-                    stage2d_fast_kernel<NPW_FLUX_BURGERS_, 2><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<1>() * sizeof(float), s>>>(a);
+                    stage2d_fast_kernel<NPW_FLUX_BURGERS_><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<1>() * sizeof(float), s>>>(a);
                     break;
                 case NPW_FLUX_EULER2D * 4 + 2:
-                    stage2d_fast_kernel<NPW_FLUX_EULER2D_, 2><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<4>() * sizeof(float), s>>>(a);
+                    stage2d_fast_kernel<NPW_FLUX_EULER2D_><<<tiles, TX_2D * TY_2D, stage2d_fast_smem_floats<4>() * sizeof(float), s>>>(a);
                     break;
                 default:
                     return cudaErrorInvalidValue;
