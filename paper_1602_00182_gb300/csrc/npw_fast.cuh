@@ -926,7 +926,8 @@ __device__ __forceinline__ void eta_k2_quot(float af, float bf, float df, double
     const double base = fma(2.0, b, -(a + d));
     const double den = fma(5.0, b, fma(2.0, d, -a)) + fp.eps_M;
     const float bound = fp.eta_max;
-    if (trans == 0.0) need = 1;
+    // (integer test: a comparison in double takes an FP64-pipe slot)
+    const bool line = (((uint32_t)__double2hiint(trans) << 1) | (uint32_t)__double2loint(trans)) == 0u;
     float denf, vc = 0.0f, vx = 0.0f;
     if (seed_f(den, &denf)) {
         const float rf = __fdividef(1.0f, denf);
@@ -936,23 +937,23 @@ __device__ __forceinline__ void eta_k2_quot(float af, float bf, float df, double
             const double q = num * r0;
             return narrow(fma(q, e, q));
         };
-        if (need & 1) vc = value(trans == 0.0 ? base : fma(-0.25, trans, base));
-        if (need & 2) vx = value(fma(0.125, trans, base));
-        if (bound > 0.0f && need != 3 && trans != 0.0) {
+        if (line) {
+            vc = vx = value(base);
+        } else if (need == 3) {
+            vc = value(fma(-0.25, trans, base));
+            vx = value(fma(0.125, trans, base));
+        } else {
+            const float v = value(fma((need & 1) ? -0.25 : 0.125, trans, base));
+            ((need & 1) ? vc : vx) = v;
             const float span = 0.376f * fabsf(narrow(trans) * rf) * (fp.rbf == NPW_RBF_GA_ ? 1.0f : 2.0f);
-            const float have = fabsf((need & 1) ? vc : vx) * (fp.rbf == NPW_RBF_GA_ ? 1.0f : 2.0f);
-            if (!((have + span) * (1.0f + 0x1p-10f) < bound)) {
-                if (need & 1)
-                    vx = value(fma(0.125, trans, base));
-                else
-                    vc = value(fma(-0.25, trans, base));
-            }
+            const float have = fabsf(v) * (fp.rbf == NPW_RBF_GA_ ? 1.0f : 2.0f);
+            if (bound > 0.0f && !((have + span) * (1.0f + 0x1p-10f) < bound))
+                ((need & 1) ? vx : vc) = value(fma((need & 1) ? 0.125 : -0.25, trans, base));
         }
     } else {
         vc = div_rn_f(fma(-0.25, trans, base), den);
-        vx = trans == 0.0 ? vc : div_rn_f(fma(0.125, trans, base), den);
+        vx = line ? vc : div_rn_f(fma(0.125, trans, base), den);
     }
-    if (trans == 0.0) vx = vc;
     if (fp.rbf != NPW_RBF_GA_) {
         vc *= 2.0f;
         vx *= 2.0f;
