@@ -963,14 +963,18 @@ __device__ __forceinline__ void eta_k2_quot(float af, float bf, float df, double
     *ex = zx ? 0.0f : vx;
     if (zc | zx) *fl |= FL_ZERO_BOUND;
 }
-// (out of line: by value what it reads)
-static __device__ __noinline__ void eta_k2_quot_any(float af, float bf, float df, double trans, double eps_M, float eta_max,
-                                                    int rbf, float* ec, float* ex, uint32_t* fl) {
+// (out of line: by value what it reads and what it returns -- (central, extrapolating, flags) -- so that the
+// caller's values stay in registers)
+static __device__ __noinline__ float4 eta_k2_quot_any(float af, float bf, float df, double trans, double eps_M, float eta_max,
+                                                      int rbf) {
     FParams fp;
     fp.eps_M = eps_M;
     fp.eta_max = eta_max;
     fp.rbf = rbf;
-    eta_k2_quot<false>(af, bf, df, trans, 3, fp, ec, ex, fl);
+    float ec, ex;
+    uint32_t fl = 0;
+    eta_k2_quot<false>(af, bf, df, trans, 3, fp, &ec, &ex, &fl);
+    return make_float4(ec, ex, __uint_as_float(fl), 0.0f);
 }
 // fl: FL_ZERO_GUARD / FL_ZERO_BOUND where the guard / the bound set a shape parameter to 0
 __device__ __forceinline__ void eta_k2_pair(const float* cf, int side, double trans, int need, const MethodParams& mp,
@@ -993,10 +997,14 @@ __device__ __forceinline__ void eta_k2_pair(const float* cf, int side, double tr
             }
         }
     }
-    if (zero_or_normal(af) & zero_or_normal(bf) & zero_or_normal(df))
+    if (zero_or_normal(af) & zero_or_normal(bf) & zero_or_normal(df)) {
         eta_k2_quot<true>(af, bf, df, trans, need, fp, ec, ex, fl);
-    else
-        eta_k2_quot_any(af, bf, df, trans, fp.eps_M, fp.eta_max, fp.rbf, ec, ex, fl);
+    } else {
+        const float4 v = eta_k2_quot_any(af, bf, df, trans, fp.eps_M, fp.eta_max, fp.rbf);
+        *ec = v.x;
+        *ex = v.y;
+        *fl |= __float_as_uint(v.z);
+    }
 }
 // the shape parameters of a k = 2 face value that are used (bit 0 central, bit 1 extrapolating): an ENO
 // value with stencil r takes row r on the right face, r - 1 on the left one
