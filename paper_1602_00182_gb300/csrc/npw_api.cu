@@ -521,25 +521,49 @@ bool compensated(const npw_params* p) {
 }
 
 // Automatic tile of the 1D per-stage kernels for the given lines: w warps' worth of cells (32 w less the
-// faces beyond the cells, or w chunks of the double body), with w the power of two that leaves the
-// busiest SM the fewest warps of work, ceil(tiles / SMs) x w; the larger tile where several tie
-// (its halo is a smaller share).  Against a fixed 1024-cell tile, which puts a 200-cell line on one
-// SM and a 20011-cell line on 20: FP64 advection N = 200, one step 90 -> 63 us, 100 steps 8.2 ->
-// 5.4 ms; FP64 1D Euler N = 20011, one step 1071 -> 194 us; mixed Burgers N = 5613, 150 steps
-// 3.75 -> 2.50 ms.
-enum StageKind { STAGE_FACES, STAGE_COMP, STAGE_DOUBLE };
+// faces beyond the cells, or w chunks of the double body), w the power of two of least cost; the larger tile
+// where several tie (its halo is a smaller share).  `beside`: CTAs of other work of the same run.
+//   FP64 bodies (bound by the FP64 pipe): the busiest SM's warps of work, ceil(tiles / SMs) w.  Against a
+// fixed 1024-cell tile, which puts a 20011-cell line on 20 SMs: 1D Euler N = 20011, one step 1071 -> 194 us.
+//   Float bodies: a tile also costs its halo and its start (4 warps' worth; 12 for the face-based one), a
+// round of eight warps its latency (10), and a line all its tiles' atomic counts (0.02 a warp).  Without
+// these terms a batch of 400 lines of 64 to 8000 cells took tiles of 125 cells, slower than fixed ones of
+// 1024: mixed Euler per stage (batch_mode 1), 1024 cells / 125 / this rule: WENO-JS5 3.17 / 3.80 / 2.74 ms,
+// RBF-WENO5 4.04 / 4.35 / 3.28 ms; one step of 300000 Euler cells 105 / 113 / 91 us; 60 lines of 300 to
+// 3000 cells 126 / 115 / 102 us a step.
+//   The mixed characteristic k = 2 body of the RBF schemes (91 registers, FP64-pipe bound): tiles of up to four
+// warps, which share an SM best: one step of 300000 cells 275 us (1024 cells), 294 (1023) and 223 (127).
+//   Lines beside resident instances or 2D tiles on every SM need no spreading: the largest tile (Euler batch of
+// 400, k = 2, resident instances beside 100 lines: 8.4 ms with 1024 cells, 8.9 with 125, 7.8 with this).
+enum StageKind { STAGE_FP64, STAGE_DOUBLE, STAGE_COMP, STAGE_FACES_F32, STAGE_FACES_MIXED };
 StageKind stage_kind(const npw_params* p) {
     if (compensated(p)) return STAGE_COMP;
-    return p->precision == NPW_FP64 && p->k == 3 && !p->characteristic ? STAGE_DOUBLE : STAGE_FACES;
+    if (p->precision == NPW_FP32_MIXED)
+        return p->k == 2 && (p->scheme == NPW_RBF_ENO || p->scheme == NPW_RBF_WENO) ? STAGE_FACES_MIXED : STAGE_FACES_F32;
+    return p->k == 3 && !p->characteristic ? STAGE_DOUBLE : STAGE_FP64;
 }
-int auto_tile(const std::vector<int64_t>& n_of, StageKind kind, int min_warps = 1) {
+int auto_tile(const std::vector<int64_t>& n_of, StageKind kind, int64_t beside = 0, int min_warps = 1) {
+    const bool f32 = kind == STAGE_COMP || kind == STAGE_FACES_F32;
+    int max_warps = npw::TILE_1D / 32;
+    if (kind == STAGE_FACES_MIXED) max_warps = 4;
+    if (f32 && beside >= npw::NUM_SMS) min_warps = max_warps;
     int best = 0;
-    int64_t best_cost = 0;
-    for (int w = min_warps; w <= npw::TILE_1D / 32; w *= 2) {
+    double best_cost = 0.0;
+    for (int w = min_warps; w <= max_warps; w *= 2) {
         const int t = kind == STAGE_DOUBLE ? npw::CHUNK_D * w : 32 * w - (kind == STAGE_COMP ? 3 : 1);
-        int64_t tiles = 0;
-        for (int64_t n : n_of) tiles += (n + t - 1) / t;
-        const int64_t cost = (tiles + npw::NUM_SMS - 1) / npw::NUM_SMS * w;
+        int64_t tiles = 0, longest = 0;
+        for (int64_t n : n_of) {
+            const int64_t k = (n + t - 1) / t;
+            tiles += k;
+            longest = k > longest ? k : longest;
+        }
+        const int64_t per_sm = (tiles + npw::NUM_SMS - 1) / npw::NUM_SMS;
+        double cost = (double)(per_sm * w);
+        if (f32) {
+            const double work = (double)(per_sm * (w + (kind == STAGE_COMP ? 4 : 12)) + 10 * ((w + 7) / 8));
+            const double counts = 0.02 * (double)(longest * (w < 8 ? w : 8));
+            cost = work > counts ? work : counts;
+        }
         if (best == 0 || cost <= best_cost) {
             best = t;
             best_cost = cost;
@@ -549,14 +573,18 @@ int auto_tile(const std::vector<int64_t>& n_of, StageKind kind, int min_warps = 
 }
 
 constexpr int FUSED_TILE_MAX = 484;
-// The work queue's tile of these 1D lines.  Fused steps: 484, 228 or 100 cells (whole warp tasks, see
-// step1d_fused_warp_body), the one whose busiest SM of four resident CTAs has the least to do, tile +
-// 28 cells' worth per tile.  Else auto_tile, in tiles of at least 255 cells for the characteristic
-// float body, whose CTAs hold few warps per SM.  Against fixed 1024-cell (fused: 512-cell) tiles: 64
-// characteristic Euler lines of 256 to 16384 cells, 60 steps, 6.9 -> 4.9 ms; the FP64 lane of a server
-// with 24 requests up to 4096 cells went from 24 to 7 ms.
-int queue_tile(const std::vector<int64_t>& n_of, bool fused, StageKind kind, bool characteristic_f32) {
-    if (!fused) return auto_tile(n_of, kind, characteristic_f32 ? 8 : 2);
+// The work queue's tile of these 1D lines, beside `beside` 2D tiles.  Fused steps: 484, 228 or 100 cells (whole
+// warp tasks, see step1d_fused_warp_body), the one whose busiest SM of four resident CTAs has the least to
+// do, tile + 28 cells' worth per tile.  Else auto_tile; the float bodies in tiles of at least 253 cells (the
+// queue's CTAs have eight warps), the characteristic ones by the FP64 bodies' cost (three CTAs an SM take
+// items as they come).  Against fixed 1024-cell (fused: 512-cell) tiles: 64 characteristic Euler lines of
+// 256 to 16384 cells, 60 steps, 6.9 -> 4.9 ms; the FP64 lane of a server with 24 requests up to 4096 cells
+// went from 24 to 7 ms.
+int queue_tile(const std::vector<int64_t>& n_of, bool fused, StageKind kind, int64_t beside) {
+    if (!fused) {
+        const bool faces = kind == STAGE_FACES_F32 || kind == STAGE_FACES_MIXED;
+        return auto_tile(n_of, faces ? STAGE_FP64 : kind, beside, faces || kind == STAGE_COMP ? 8 : 2);
+    }
     int best = 0;
     int64_t best_cost = 0;
     for (int t : {100, 228, FUSED_TILE_MAX}) {
@@ -588,7 +616,7 @@ int batch_auto_tile(const npw_instance* inst, int count, int m, const npw_params
     std::vector<int64_t> n_of;
     for (int i = 0; i < count; ++i)
         if (!resident_ok(p, m, inst[i].n)) n_of.push_back(inst[i].n);
-    return auto_tile(n_of, stage_kind(p));
+    return auto_tile(n_of, stage_kind(p), count - (int64_t)n_of.size());
 }
 // entries of a batch's tile table: every instance in the smallest tile a run may choose, or the
 // per-stage ones in the automatic tile
@@ -1892,15 +1920,17 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
     for (int k = 1; k < 3; ++k) main_kind = kind_cells[k] > kind_cells[main_kind] ? k : main_kind;
     // a batch of compensated float 1D items alone takes one launch per RK3 step
     bool any2d = false;
+    int64_t tiles2d = 0;
     std::vector<int64_t> lines;
     for (int i = 0; i < count; ++i) {
         any2d |= inst[i].ny != 0;
+        if (inst[i].ny != 0) tiles2d += items_of(inst[i], 1, params);
         if (inst[i].ny == 0 && !resident_ok(params, flux_m(inst[i].flux_kind), inst[i].nx)) lines.push_back(inst[i].nx);
     }
     r.fused = r.comp && !any2d;
     // (npw_autotune_1d times the per-stage kernels: its choice is not for fused steps)
     const int automatic = tight ? (r.fused ? FUSED_TILE_MAX : npw::TILE_1D)
-                                : queue_tile(lines, r.fused, stage_kind(params), r.fp32 && r.characteristic);
+                                : queue_tile(lines, r.fused, stage_kind(params), tiles2d);
     const int tile = r.fused ? (params->tile_1d > 0 ? params->tile_1d : automatic)
                              : resolve_tile(params, main_kind, flux_m(main_kind), automatic);
     // descriptors; mixed-precision 1D instances that fit in shared memory run resident
@@ -2288,7 +2318,7 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
         }
         std::vector<int64_t> lines;
         for (int k : g.members) lines.push_back(h1[k].n);
-        tile_lines(g, queue_tile(lines, g.fused, lane.mp.k == 3 ? STAGE_DOUBLE : STAGE_FACES, false));
+        tile_lines(g, queue_tile(lines, g.fused, lane.mp.k == 3 ? STAGE_DOUBLE : STAGE_FP64, 0));
     }
     // more than the list holds (a few long lines in a heap of their size take small tiles): the largest tiles
     if (total + total2d > lane.L.max_items)
