@@ -573,23 +573,35 @@ int auto_tile(const std::vector<int64_t>& n_of, StageKind kind, int64_t beside =
 }
 
 constexpr int FUSED_TILE_MAX = 484;
-// The work queue's tile of these 1D lines, beside `beside` 2D tiles.  Fused steps: 484, 228 or 100 cells (whole
-// warp tasks, see step1d_fused_warp_body), the one whose busiest SM of four resident CTAs has the least to
-// do, tile + 28 cells' worth per tile.  Else auto_tile; the float bodies in tiles of at least 253 cells (the
+// The work queue's tile of these 1D lines of up to m fields, beside `beside` 2D tiles.  Fused steps, k = 3: 484,
+// 228 or 100 cells (whole warp tasks, see step1d_fused_warp_body), the one whose busiest SM of four resident
+// CTAs has the least to do, tile + 28 cells' worth per tile.  Fused, k = 2 (the flat body): the largest of 1024
+// .. 128 cells whose arrays take 44 KB at most (four CTAs an SM) and which gives every SM a tile; 96 Euler
+// lines of 4000 to 20000 cells, WENO-JS3: 256 cells 1.49 ms, 512 1.30 ms.  Else auto_tile; the float bodies in tiles of at least 253 cells (the
 // queue's CTAs have eight warps), the characteristic ones by the FP64 bodies' cost (three CTAs an SM take
 // items as they come).  Against fixed 1024-cell (fused: 512-cell) tiles: 64 characteristic Euler lines of
 // 256 to 16384 cells, 60 steps, 6.9 -> 4.9 ms; the FP64 lane of a server with 24 requests up to 4096 cells
 // went from 24 to 7 ms.
-int queue_tile(const std::vector<int64_t>& n_of, bool fused, StageKind kind, int64_t beside) {
+int queue_tile(const std::vector<int64_t>& n_of, bool fused, StageKind kind, int64_t beside, int k, int m) {
     if (!fused) {
         const bool faces = kind == STAGE_FACES_F32 || kind == STAGE_FACES_MIXED;
         return auto_tile(n_of, faces ? STAGE_FP64 : kind, beside, faces || kind == STAGE_COMP ? 8 : 2);
     }
+    auto tiles_in = [&](int t) {
+        int64_t tiles = 0;
+        for (int64_t n : n_of) tiles += (n + t - 1) / t;
+        return tiles;
+    };
+    if (k == 2) {
+        int t = 1024;
+        while (t > 128 && (npw::fused1d_smem_floats(t, m) * sizeof(float) > (size_t)44 * 1024 || tiles_in(t) < npw::NUM_SMS))
+            t /= 2;
+        return t;
+    }
     int best = 0;
     int64_t best_cost = 0;
     for (int t : {100, 228, FUSED_TILE_MAX}) {
-        int64_t tiles = 0;
-        for (int64_t n : n_of) tiles += (n + t - 1) / t;
+        const int64_t tiles = tiles_in(t);
         const int64_t cost = (tiles + 4 * npw::NUM_SMS - 1) / (4 * npw::NUM_SMS) * (t + 28);
         if (best == 0 || cost <= best_cost) {
             best = t;
@@ -1921,16 +1933,21 @@ npw_status npweno_queue_solve(void* arena, const npw_queue_instance* inst, int32
     // a batch of compensated float 1D items alone takes one launch per RK3 step
     bool any2d = false;
     int64_t tiles2d = 0;
+    int line_m = 1;  // most fields of a line in the queue
     std::vector<int64_t> lines;
     for (int i = 0; i < count; ++i) {
         any2d |= inst[i].ny != 0;
         if (inst[i].ny != 0) tiles2d += items_of(inst[i], 1, params);
-        if (inst[i].ny == 0 && !resident_ok(params, flux_m(inst[i].flux_kind), inst[i].nx)) lines.push_back(inst[i].nx);
+        const int m = flux_m(inst[i].flux_kind);
+        if (inst[i].ny == 0 && !resident_ok(params, m, inst[i].nx)) {
+            lines.push_back(inst[i].nx);
+            line_m = m > line_m ? m : line_m;
+        }
     }
     r.fused = r.comp && !any2d;
     // (npw_autotune_1d times the per-stage kernels: its choice is not for fused steps)
     const int automatic = tight ? (r.fused ? FUSED_TILE_MAX : npw::TILE_1D)
-                                : queue_tile(lines, r.fused, stage_kind(params), tiles2d);
+                                : queue_tile(lines, r.fused, stage_kind(params), tiles2d, params->k, line_m);
     const int tile = r.fused ? (params->tile_1d > 0 ? params->tile_1d : automatic)
                              : resolve_tile(params, main_kind, flux_m(main_kind), automatic);
     // descriptors; mixed-precision 1D instances that fit in shared memory run resident
@@ -2318,7 +2335,7 @@ npw_status lane_round(npw_server* sv, int ln, int steps) {
         }
         std::vector<int64_t> lines;
         for (int k : g.members) lines.push_back(h1[k].n);
-        tile_lines(g, queue_tile(lines, g.fused, lane.mp.k == 3 ? STAGE_DOUBLE : STAGE_FP64, 0));
+        tile_lines(g, queue_tile(lines, g.fused, lane.mp.k == 3 ? STAGE_DOUBLE : STAGE_FP64, 0, lane.mp.k, g.m));
     }
     // more than the list holds (a few long lines in a heap of their size take small tiles): the largest tiles
     if (total + total2d > lane.L.max_items)

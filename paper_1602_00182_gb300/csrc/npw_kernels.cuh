@@ -2579,10 +2579,13 @@ __device__ __forceinline__ void queue_item_2d(const Stage2DArgs& a2, const Inst2
 // CTAs per SM the register allocation aims for: 4 for the specialised mixed-precision k = 3 kernels
 // (64 registers a thread for the f32x2 pairs; their shared memory allows as many), 3 for the
 // characteristic one (it takes 116 registers when left alone, and two CTAs are too few warps to hide its
-// long chains), else no bound
+// long chains), 4 for k = 2 on 1D Euler (74 registers when left alone, three CTAs: 96 lines, WENO-JS3, 512-cell
+// tiles 1.40 ms, with four 1.30 ms), else no bound
 template <typename R, int K, bool CHAR, int SHAPE>
 constexpr int queue_min_blocks() {
-    return sizeof(R) == sizeof(float) && K == 3 && SHAPE != QS_ANY ? (CHAR ? 3 : 4) : 1;
+    if (sizeof(R) != sizeof(float) || SHAPE == QS_ANY) return 1;
+    if (K == 2) return SHAPE == QS_1D_EULER && !CHAR ? 4 : 1;
+    return CHAR ? 3 : 4;
 }
 
 template <typename R, int K, bool CHAR, int SHAPE>

@@ -56,3 +56,20 @@ def test_lines_together(npw, k, precision, m, char, mode):
                                          eta_max=1.0)) for tile in (0, 256, 1024)]
     for u, stats in out[1:]:
         assert torch.equal(u, out[0][0]) and stats == out[0][1]
+
+
+@pytest.mark.parametrize("m", [1, 3])
+@pytest.mark.parametrize("ns", [[40], [129], [3000, 500], [20000, 9000, 257], [152 * 512 + 1], [152 * 1024]])
+def test_fused_steps_of_k2(npw, ns, m):
+    """The automatic tile of the queue's fused k = 2 steps (128 to 1024 cells) against 256 cells."""
+    kind, bc = (npw.NPW_FLUX_EULER1D, 1) if m == 3 else (npw.NPW_FLUX_BURGERS, 0)
+    specs = [dict(kind=kind, nx=n, dx=1.0 / n, t_end=0.9 / n, cfl=0.3, bc=bc) for n in ns]
+    table, _, _ = npw.make_queue_instances(specs)
+    u0 = torch.tensor(np.concatenate([_line(n, m, n).ravel() for n in ns]), dtype=torch.float32, device="cuda")
+    out = []
+    for tile in (0, 256):
+        u = u0.clone()
+        st, stats = npw.npweno_queue_solve(u, table, npw.Params(k=2, precision=1, batch_mode=1, tile_1d=tile, eta_max=1.0))
+        assert st == 0
+        out.append((u, stats))
+    assert torch.equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
