@@ -475,25 +475,29 @@ __device__ __forceinline__ bool switch_v0_near(const double* w, double tol) {
     }
     return near;
 }
+// near tie of a k = 2 face of the RBF schemes, in double; w[1..4] = cells i-1..i+2
+__device__ __forceinline__ bool face_near_tie_k2(const double* w, const MethodParams& mp, double tol) {
+    bool near = false;
+    if (mp.monotone_switch) near = k2_ratio_near(w[1], w[2], w[3], tol) || k2_ratio_near(w[2], w[3], w[4], tol);
+    for (int side = 0; side < 2; ++side) {
+        const double* c = w + 1 + side;  // cell i (side 0, v^-) or i + 1 (side 1, v^+)
+        const double a = side == 0 ? c[0] : c[2], b = c[1], d = side == 0 ? c[2] : c[0];
+        const double den0 = -a + 5.0 * b + 2.0 * d, mag = fabs(a) + 5.0 * fabs(b) + 2.0 * fabs(d);
+        if (mp.eta_guard > 0.0) near = near || tie_rel(fabs(den0), mp.eta_guard * mag, tol);
+        if (mp.eta_max > 0.0) {
+            const double e = (mp.rbf == NPW_RBF_GA_ ? 1.0 : 2.0) * (-a + 2.0 * b - d) / (den0 + mp.eps_M);
+            near = near || tie_rel(fabs(e), mp.eta_max, tol);
+        }
+    }
+    return near;
+}
 static __device__ __noinline__ bool face_near_tie_d(double w1, double w2, double w3, double w4, const MethodParams& mp,
                                                     double tol) {
     const double w[6] = {0.0, w1, w2, w3, w4, 0.0};  // (both orders use cells i-1..i+2)
     const bool rbf = mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_;
     bool near = false;
     if (mp.k == 2) {
-        if (rbf && mp.monotone_switch) near = k2_ratio_near(w[1], w[2], w[3], tol) || k2_ratio_near(w[2], w[3], w[4], tol);
-        if (rbf) {
-            for (int side = 0; side < 2; ++side) {
-                const double* c = w + 1 + side;  // cell i (side 0, v^-) or i + 1 (side 1, v^+)
-                const double a = side == 0 ? c[0] : c[2], b = c[1], d = side == 0 ? c[2] : c[0];
-                const double den0 = -a + 5.0 * b + 2.0 * d, mag = fabs(a) + 5.0 * fabs(b) + 2.0 * fabs(d);
-                if (mp.eta_guard > 0.0) near = near || tie_rel(fabs(den0), mp.eta_guard * mag, tol);
-                if (mp.eta_max > 0.0) {
-                    const double e = (mp.rbf == NPW_RBF_GA_ ? 1.0 : 2.0) * (-a + 2.0 * b - d) / (den0 + mp.eps_M);
-                    near = near || tie_rel(fabs(e), mp.eta_max, tol);
-                }
-            }
-        }
+        if (rbf) near = face_near_tie_k2(w, mp, tol);
         return near;
     }
     if (rbf && mp.monotone_switch)
@@ -545,9 +549,10 @@ __device__ __forceinline__ bool far_from_ties(float d0, float d1, float d2, floa
     return far_;
 }
 
-template <typename R>
+// K2: float data of order k = 2, known at compile time
+template <typename R, bool K2>
 __device__ __forceinline__ bool face_near_tie(const R* wr, const MethodParams& mp, double tol) {
-    if (mp.k == 3 && (mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_) && mp.guard_switch && mp.tie_tol_f <= 0x1p-14f) {
+    if (!K2 && mp.k == 3 && (mp.scheme == NPW_RBF_ENO_ || mp.scheme == NPW_RBF_WENO_) && mp.guard_switch && mp.tie_tol_f <= 0x1p-14f) {
         // a constant stencil: monotone; its denominator and numerator against positive thresholds are exactly 0 in
         // float (15 w is exact in double) and where w = 0, but round-off of 15 w and 3 w in double
         if (wr[1] == wr[2] && wr[2] == wr[3] && wr[3] == wr[4] &&
@@ -575,6 +580,10 @@ __device__ __forceinline__ bool face_near_tie(const R* wr, const MethodParams& m
         if (ok) return false;
     }
     if (mp.scheme != NPW_RBF_ENO_ && mp.scheme != NPW_RBF_WENO_) return false;
+    if constexpr (K2) {
+        const double w[6] = {0.0, (double)wr[1], (double)wr[2], (double)wr[3], (double)wr[4], 0.0};
+        return face_near_tie_k2(w, mp, tol);
+    }
     return face_near_tie_d((double)wr[1], (double)wr[2], (double)wr[3], (double)wr[4], mp, tol);
 }
 
