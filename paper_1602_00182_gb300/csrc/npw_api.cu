@@ -113,7 +113,6 @@ npw::MethodParams method(const npw_params* p) {
     mp.max_steps = p->max_steps > 0 ? p->max_steps : 0;
     mp.eps_weno_f = (float)mp.eps_weno;
     mp.eps_M_f = (float)mp.eps_M;
-    mp.eps_M_lo_f = (float)(mp.eps_M - (double)mp.eps_M_f);
     mp.eta_guard_f = (float)mp.eta_guard;
     mp.eta_max_f = (float)mp.eta_max;
     mp.gamma_f = (float)mp.gamma;

@@ -86,7 +86,7 @@ struct MethodParams {
     int64_t max_steps; // step limit of a solve (0 = automatic, see step_cap)
     // the same values rounded once to float on the host, for the float state (a conversion
     // in the kernels would take FP64-pipe slots)
-    float eps_weno_f, eps_M_f, eps_M_lo_f, eta_guard_f, eta_max_f;  // eps_M ~ eps_M_f + eps_M_lo_f
+    float eps_weno_f, eps_M_f, eta_guard_f, eta_max_f;
     float gamma_f, adv_speed_f, adv_speed_y_f;
     float inflow_f[4];
     // mixed precision, k = 3: constants of the common path of the shape parameter and of the
