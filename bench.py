@@ -268,7 +268,8 @@ def headline_burgers(args, rank, world, local_rank):
     else:
         secondary["fp64_pipe"] = "no FP64 instruction on the common path (eta from float pairs)"
     roof = roofline_hbm(BYTES_SCALAR_F32, cu_a, res_s,
-                        "solve1d_resident_kernel<BURGERS, 3>, size class n > 4096 (512 threads, 2 CTAs/SM)",
+                        "solve1d_resident_kernel<BURGERS, 3>, size class n > 4096 "
+                        + ("(512 threads, 1 CTA/SM)" if len(big) <= 152 else "(256 threads, 2 CTAs/SM)"),
                         traffic=_ncu_traffic("solve1d_resident_burgers_classA_dram_bytes_per_launch"),
                         secondary=secondary,
                         resident_launches=[int(x) for x in pr.resident_launches],
@@ -477,7 +478,7 @@ def block_euler1d(args, characteristic: int):
     cu_queue = sum(n * s["steps"] for n, s in zip(ns, stats) if characteristic or n > res_limit)
     stage_s = prof.pr.stage_ms / 1e3
     eta_tot = {k: sum(s["eta"][k] for s in stats) for k in ("switch", "eval", "guard", "bound")}
-    kern = ("queue_stage_kernel<float, K=3, characteristic, 1D Euler> (face-based Roe-field body)" if characteristic
+    kern = ("queue_stage_kernel_b3<float, K=3, characteristic, 1D Euler> (face-based Roe-field body)" if characteristic
             else "queue_stage_kernel_b4<float, K=3, 1D Euler> (fused RK3 step body)")
     return {
         "metric": "cell-updates/s", "value": cu / (ms / 1e3), "unit": "cell-updates/s", "dtype": "f32",

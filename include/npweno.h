@@ -94,9 +94,11 @@ typedef struct {
                                 per-stage kernels; 1 = every instance through the per-stage kernels */
     int32_t tile_1d;         /* cells per CTA of the 1D per-stage kernels: 256, 512, 1024 or 2048; 0 = the
                                 value npw_autotune_1d chose for this flux kind, m, k, precision and
-                                characteristic flag on this device, else a size up to 1024 that spreads
-                                the lines over the SMs.  Results do not depend on it (each face gets the
-                                same arithmetic in any tiling) */
+                                characteristic flag on this device, else a size up to 1024 that suits the
+                                lines.  Not used where a line is solved whole: by a thread-block cluster
+                                (npweno_rk3_step and npweno_solve on short lines) or by one CTA (resident
+                                instances).  Results do not depend on it (each face gets the same
+                                arithmetic in any tiling) */
     double eta_max;          /* optional bound, not in the paper: eta = 0 where |eta| > eta_max.  The printed eta
                                 (Table k3, Table k2) is singular where its denominator crosses zero (a monotone
                                 stencil with zero slope at the face for k = 3, v ~ 0 at the face for k = 2), and
@@ -204,7 +206,9 @@ size_t npw_workspace_size(int64_t n, int32_t m, const npw_params* params);
  * One TVD-RK3 step (Sec. 5.1, Shu-Osher form) of u [m][n] (device, in/out) with the given
  * dt.  alpha of the Lax-Friedrichs flux is max_i |f'(u_i^n)| over the field, frozen over the
  * three stages.  Each stage is one fused kernel: halo load, shape parameter, switch,
- * candidates, weights, flux, flux difference (eq. PDE1) and the stage combination.
+ * candidates, weights, flux, flux difference (eq. PDE1) and the stage combination.  A short line
+ * (k = 3, component-wise, n m up to 40000 in NPW_FP32_MIXED, 1500 in NPW_FP64) takes the whole step
+ * in one launch of a thread-block cluster, with the same bits.
  * If alpha_out is not NULL the alpha used is written there (host double; the call then
  * synchronises the stream).
  */
@@ -216,8 +220,11 @@ npw_status npweno_rk3_step(void* u, int64_t n, int32_t m, double dx, double dt, 
  * Advance u [m][n] (device, in/out) from t = 0 to t_end with dt = cfl * dx / alpha^n, alpha^n
  * = max_i |f'(u_i^n)| (Sec. 5.1 with the CFL rule of Sec. 5.2); the step that reaches t_end to
  * within 1e-10 of a step is shortened to end exactly at t_end.  Time control runs on the
- * device; the host polls a completion word between launches.  out (host) may be NULL.
- * Returns NPW_ENONFINITE if the state stops being finite.
+ * device; the host polls between launches of up to 256 steps (short lines, as above: one launch of a
+ * cluster, else per-stage kernels).  Each of these waits is limited (NPW_WAIT_TIMEOUT_S in the
+ * environment, seconds, default 1800): when one runs out the call returns NPW_ETIMEOUT with up to 256
+ * steps still queued, and u and workspace must stay allocated until the stream has drained.  out
+ * (host) may be NULL.  Returns NPW_ENONFINITE if the state stops being finite.
  */
 npw_status npweno_solve(void* u, int64_t n, int32_t m, double dx, double t_end, double cfl, int32_t flux_kind,
                         int32_t bc, const npw_params* params, void* workspace, size_t workspace_bytes,
@@ -261,14 +268,16 @@ npw_status npweno_solve_2d(void* u, int64_t nx, int64_t ny, int32_t m, double dx
  * the method; the paper has no counterpart) advanced together, each with its own dt, alpha,
  * t_end and step count.  Every RK3 stage is one launch of a persistent kernel whose CTAs take
  * (instance, tile) work items from a device counter until none is left -- 1D tiles of
- * params->tile_1d cells (0: the autotuned or default size), 2D tiles of 32 x 8 cells -- and run
+ * params->tile_1d cells (0: the autotuned or automatic size), 2D tiles of 30 x 11 cells (NPW_FP32_MIXED,
+ * k = 3) or 32 x 8 -- and run
  * the per-stage body of that instance's kind (the same arithmetic as npweno_batch_solve and
  * npweno_solve_2d, so the same bits); steps are replayed as CUDA graphs between bounded polls.
  * NPW_FP32_MIXED component-wise runs solve 1D instances that fit in shared memory whole in one
  * CTA (the resident kernel, batch_mode 0) beside the queue; when the queued instances are all
  * 1D, each RK3 step is a single launch (u^n loaded once per tile with a 9-cell halo, the three
  * stages in shared memory, the same bits as the per-stage launches; tile_1d 0 then takes 484, 228 or
- * 100 cells, whichever spreads the lines best).  A batch whose instances share one
+ * 100 cells (k = 2: 1024 to 128), whichever spreads the lines best, and npw_autotune_1d, which times the
+ * per-stage kernels, has no part in it).  A batch whose instances share one
  * dimension and flux kind runs a kernel compiled for that shape.  Characteristic runs take 1D
  * Euler instances only.
  *   arena: device, the instances' fields ([m][n] or [m][ny][nx] at `offset`, element type of
@@ -373,7 +382,9 @@ void npw_server_destroy(npw_server* s);
  * Times TVD-RK3 steps of a 2^21-cell periodic instance of smooth synthetic data (a quiet
  * Euler state for m = 3) with each tile size 256, 512, 1024, 2048 cells per CTA, keeps the
  * fastest in a process-wide table keyed by device, flux kind, m, k, precision and
- * characteristic flag, and returns it.  Later runs with params->tile_1d = 0 use it.
+ * characteristic flag, and returns it.  Later runs with params->tile_1d = 0 use it in the per-stage 1D
+ * kernels: npweno_rk3_step, npweno_solve and npweno_batch_solve where they run those, and the work
+ * queue's per-stage items.  The queue's fused steps and the request server choose their own tiles.
  *   scratch: caller-owned device memory of at least npw_autotune_scratch_bytes(m, params)
  *            bytes (its contents are overwritten).
  *   stream:  cudaStream_t (void*); the call synchronises with it (bounded wait).

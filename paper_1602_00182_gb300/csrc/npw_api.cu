@@ -1216,10 +1216,16 @@ npw_status npweno_rk3_step(void* u, int64_t n, int32_t m, double dx, double dt, 
 // CTAs of the cluster that solves one line whole (solve1d_cluster_kernel), 0: the per-stage kernels.  One
 // slice per CTA of at least 8 cells; 16 CTAs leave 9/10 of the SMs idle, so the line may not be longer
 // than what they work off in the time that the launches of a stage take: float CLUSTER_F32 cells and
-// fields together, double CLUSTER_F64 (an FP64 stage costs tens of float ones).  Against the per-stage
-// launches: FP64 advection N = 200, 100 steps 3.8 -> 2.5 ms and one step 51 -> 35 us (two launches for
-// eight), mixed Burgers N = 5613, 150 steps 2.5 -> 1.26 ms.  A stage of 200 FP64 cells is 8 us of
-// dependent FP64 instructions (about 90 cycles each), whatever the number of SMs.
+// fields together, double CLUSTER_F64 (an FP64 stage costs tens of float ones).  A stage of 200 FP64 cells is
+// 8 us of dependent FP64 instructions (about 90 cycles each), whatever the number of SMs.  One step of a solve,
+// cluster / per-stage launches, us, by n m:
+//   float, WENO-JS5       Burgers  20000 12/22   40000 16/22   50000 19/23   70000 23/23   100000 30/23
+//                         Euler    20000 15/25   40000 17/25   50000 24/26   70000 25/29   100000 33/29
+//   float, RBF-WENO5      Burgers  20000 16/24   40000 23/27   50000 25/26   70000 30/29   100000 40/30
+//                         Euler    20000 20/27   40000 24/30   50000 32/31   70000 35/34   100000 47/35
+//   double, RBF-WENO5     Burgers  200 27/41     1500 34/45    2000 40/47    3000 46/46    5000 65/44
+//                         Euler    200 61/77     1500 66/80    2000 68/83    3000 74/88    5000 85/94
+// One call of npweno_rk3_step gains more (one launch for eight operations): N = 200 FP64 46 -> 29 us.
 }  // extern "C"
 namespace {
 constexpr int64_t CLUSTER_F32 = 40000, CLUSTER_F64 = 1500;

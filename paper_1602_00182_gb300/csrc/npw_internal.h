@@ -222,7 +222,8 @@ struct Stage2DArgs {
 
 // Persistent work-queue stage kernel: the CTAs of one launch pull work items (instance, tile)
 // from a device counter until the list is exhausted; 1D items are tiles of `tile` cells (start
-// cell in Tile.start), 2D items tiles of TX_2D x TY_2D cells (tile index in Tile.start).  Every
+// cell in Tile.start), 2D items tiles of TX_2D x TY_2D cells, or TX_WARP x TY_WARP (warp_tiles_2d), with the
+// tile index in Tile.start.  Every
 // instance has its own descriptor, control word and step; items of finished instances return
 // at once.  The last CTA to leave resets the counter for the next launch.
 struct QueueArgs {

@@ -2026,7 +2026,7 @@ __device__ __forceinline__ void stage2d_fast_body(const Stage2DArgs& a, const In
 // method, and the two fields of a pair share every f32x2 instruction.  Each face value has the
 // arithmetic of the flat body, so the results are the same bits.  Bound by instruction issue (64% of
 // the slots) and the barriers between the phases; FMA pipe 44%.  One stage of 2048^2 2D Euler cells: 645
-// -> 320 M warp instructions, 643 -> 407 us.  (A form that kept a row window in registers and marched
+// -> 312 M warp instructions, 643 -> 401 us.  (A form that kept a row window in registers and marched
 // without shared memory issued 256 M, but its 17 KB loop body missed the instruction cache: 657 us.)
 // Shared memory (V: a pair of fields, or the one field): the (TX_WARP + 6) x (TY_WARP + 6) block and
 // three face arrays of 32 lanes x (TY_WARP x-face rows, TY_WARP + 1 y-face rows).
@@ -2559,9 +2559,9 @@ __global__ void __launch_bounds__(TX_2D * TY_2D) stage2d_kernel(Stage2DArgs a) {
 // ---------------------------------------------------------------------------------------
 // Persistent work-queue kernel (QueueArgs): one launch per stage for every instance of a batch,
 // 1D and 2D together.  Each CTA takes the next item from q.head[0] until the list is exhausted
-// and runs the per-item body of the instance's kind: for the float state the compensated 1D
-// body (or the face-based characteristic body) and the phased 2D body, for the double state the
-// face-based bodies.  The bodies are those of the one-CTA-per-item kernels, so the results are
+// and runs the per-item body of the instance's kind: for the float state the compensated 1D body (or the
+// fused step, or the face-based characteristic body) and the 2D body of warp tasks (k = 2: the flat one); for the
+// double state the chunk body in 1D (k = 3, component-wise) and the face-based bodies.  The bodies are those of the one-CTA-per-item kernels, so the results are
 // the same bits.  The last CTA to finish resets the counters for the next launch (the next
 // launch is ordered after this one on the stream).
 // ---------------------------------------------------------------------------------------
