@@ -839,7 +839,7 @@ npw_status launch_resident_set(const ResidentLaunch& rl, const std::vector<int32
         const int64_t n = n_of[i];
         cls[n > 4096 ? 0 : (n > 2048 ? 1 : (n > 1024 ? 2 : 3))].push_back(i);
     }
-    // Threads of a CTA.  k = 3 (116 registers a thread, 512 threads an SM): a class with a CTA for no
+    // Threads of a CTA.  k = 3 (120 registers a thread, 512 threads an SM): a class with a CTA for no
     // more than every SM takes the larger CTA, since its longest instance is then the critical path; a
     // larger class takes two or more CTAs per SM, one computing while another waits at its barrier.
     // Burgers, N in [64, 8192], 300 steps: 1024 instances (146 in the largest class) 9.1 ms with 512
