@@ -276,7 +276,7 @@ npw_status npweno_solve_2d(void* u, int64_t nx, int64_t ny, int32_t m, double dx
  * CTA (the resident kernel, batch_mode 0) beside the queue; when the queued instances are all
  * 1D, each RK3 step is a single launch (u^n loaded once per tile with a 9-cell halo, the three
  * stages in shared memory, the same bits as the per-stage launches; tile_1d 0 then takes 484, 228 or
- * 100 cells (k = 2: 1024 to 128), whichever spreads the lines best, and npw_autotune_1d, which times the
+ * 100 cells (k = 2: 1024 to 64), whichever spreads the lines best, and npw_autotune_1d, which times the
  * per-stage kernels, has no part in it).  A batch whose instances share one
  * dimension and flux kind runs a kernel compiled for that shape.  Characteristic runs take 1D
  * Euler instances only.

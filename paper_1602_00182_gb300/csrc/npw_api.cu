@@ -525,7 +525,8 @@ bool compensated(const npw_params* p) {
 //   FP64 bodies (bound by the FP64 pipe): the busiest SM's warps of work, ceil(tiles / SMs) w.  Against a
 // fixed 1024-cell tile, which puts a 20011-cell line on 20 SMs: 1D Euler N = 20011, one step 1071 -> 194 us.
 //   Float bodies: a tile also costs its halo and its start (4 warps' worth; 12 for the face-based one), a
-// round of eight warps its latency (10), and a line all its tiles' atomic counts (0.02 a warp).  Without
+// round of eight warps its latency (10), and a line all its tiles' atomic counts (0.02 a warp); more than a
+// round a tile only where every SM has one (characteristic, 60000 cells: 509-cell tiles 15% slower).  Without
 // these terms a batch of 400 lines of 64 to 8000 cells took tiles of 125 cells, slower than fixed ones of
 // 1024: mixed Euler per stage (batch_mode 1), 1024 cells / 125 / this rule: WENO-JS5 3.17 / 3.80 / 2.74 ms,
 // RBF-WENO5 4.04 / 4.35 / 3.28 ms; one step of 300000 Euler cells 105 / 113 / 91 us; 60 lines of 300 to
@@ -556,6 +557,7 @@ int auto_tile(const std::vector<int64_t>& n_of, StageKind kind, int64_t beside =
             tiles += k;
             longest = k > longest ? k : longest;
         }
+        if (f32 && w > 8 && w > min_warps && tiles < npw::NUM_SMS) break;  // (leaves SMs idle)
         const int64_t per_sm = (tiles + npw::NUM_SMS - 1) / npw::NUM_SMS;
         double cost = (double)(per_sm * w);
         if (f32) {
@@ -575,7 +577,7 @@ constexpr int FUSED_TILE_MAX = 484;
 // The work queue's tile of these 1D lines of up to m fields, beside `beside` 2D tiles.  Fused steps, k = 3: 484,
 // 228 or 100 cells (whole warp tasks, see step1d_fused_warp_body), the one whose busiest SM of four resident
 // CTAs has the least to do, tile + 28 cells' worth per tile.  Fused, k = 2 (the flat body): the largest of 1024
-// .. 128 cells whose arrays take 44 KB at most (four CTAs an SM) and which gives every SM a tile; 96 Euler
+// .. 64 cells whose arrays take 44 KB at most (four CTAs an SM) and which gives every SM a tile; 96 Euler
 // lines of 4000 to 20000 cells, WENO-JS3: 256 cells 1.49 ms, 512 1.30 ms.  Else auto_tile; the float bodies in tiles of at least 253 cells (the
 // queue's CTAs have eight warps), the characteristic ones by the FP64 bodies' cost (three CTAs an SM take
 // items as they come).  Against fixed 1024-cell (fused: 512-cell) tiles: 64 characteristic Euler lines of
@@ -593,7 +595,7 @@ int queue_tile(const std::vector<int64_t>& n_of, bool fused, StageKind kind, int
     };
     if (k == 2) {
         int t = 1024;
-        while (t > 128 && (npw::fused1d_smem_floats(t, m) * sizeof(float) > (size_t)44 * 1024 || tiles_in(t) < npw::NUM_SMS))
+        while (t > 64 && (npw::fused1d_smem_floats(t, m) * sizeof(float) > (size_t)44 * 1024 || tiles_in(t) < npw::NUM_SMS))
             t /= 2;
         return t;
     }

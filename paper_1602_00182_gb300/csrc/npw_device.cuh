@@ -262,7 +262,7 @@ __device__ __forceinline__ double cell_value_k2_d(const double* c, int side, dou
     double x0 = mp.eps_weno + g0 * g0, x1 = mp.eps_weno + g1 * g1;
     x0 = x0 * x0;
     x1 = x1 * x1;
-    const double a0 = f64::div(side == 0 ? 2.0 / 3.0 : 1.0 / 3.0, x0), a1 = f64::div(side == 0 ? 1.0 / 3.0 : 2.0 / 3.0, x1);
+    const double a0 = f64::div_third(side == 0 ? 2.0 / 3.0 : 1.0 / 3.0, x0), a1 = f64::div_third(side == 0 ? 1.0 / 3.0 : 2.0 / 3.0, x1);
     const double sum = a0 + a1;
     return fma(f64::div(a0, sum), cand(0), 0.0) + f64::div(a1, sum) * cand(1);
 }

@@ -71,6 +71,12 @@ __device__ __forceinline__ double div(double n, double x) {
     return ok ? quot0(n, x, y) : div_any(n, x);
 }
 
+// n / x for n = 1/3 or 2/3: any x, hard ones too (the argument at weights_from, for the mantissa of 1/3)
+__device__ __forceinline__ double div_third(double n, double x) {
+    double y;
+    return recip_near(x, &y) ? quot(n, x, y) : div_any(n, x);
+}
+
 // a truncated to float (0 where it is 0); *ok false outside [2^-99, 2^99)
 __device__ __forceinline__ float to_f(double a, bool* ok) {
     float f;

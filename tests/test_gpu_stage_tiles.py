@@ -61,7 +61,7 @@ def test_lines_together(npw, k, precision, m, char, mode):
 @pytest.mark.parametrize("m", [1, 3])
 @pytest.mark.parametrize("ns", [[40], [129], [3000, 500], [20000, 9000, 257], [152 * 512 + 1], [152 * 1024]])
 def test_fused_steps_of_k2(npw, ns, m):
-    """The automatic tile of the queue's fused k = 2 steps (128 to 1024 cells) against 256 cells."""
+    """The automatic tile of the queue's fused k = 2 steps (64 to 1024 cells) against 256 cells."""
     kind, bc = (npw.NPW_FLUX_EULER1D, 1) if m == 3 else (npw.NPW_FLUX_BURGERS, 0)
     specs = [dict(kind=kind, nx=n, dx=1.0 / n, t_end=0.9 / n, cfl=0.3, bc=bc) for n in ns]
     table, _, _ = npw.make_queue_instances(specs)
